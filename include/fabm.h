@@ -158,7 +158,12 @@ enum {
     FABM_HIST_AUTO = 0,    /* FP64 precision: FABM_HIST_FP64; split precision: tensor
                               cores for batches of at least 64 columns, else FP32C;
                               FP64X2 precision: FABM_HIST_X2                         */
-    FABM_HIST_FP64 = 1,    /* double on CUDA cores (FP64 precision only)             */
+    FABM_HIST_FP64 = 1,    /* double on CUDA cores (FP64 precision only): the points of
+                              the last two superblocks of 128 to 1024 steps summed
+                              directly, older ones by transforms of a superblock's
+                              points (32 bytes of device memory per step and column
+                              beyond two superblocks; without that room, every point
+                              is summed directly)                                    */
     FABM_HIST_TENSOR = 2,  /* three-term bf16 split on tcgen05 tensor cores, exact
                               per 64-point segment, far history of each 64-step block
                               with 64 targets per MMA (split precision)              */
@@ -225,9 +230,10 @@ int fabm_get_recurrence_warps(const fabm_solver *s);
  * prediction for all N steps is smallest (a probe that reaches N is timed
  * as it is).
  * Longer probes predict better where the history only dominates late in a
- * long solve.  Candidates: for FABM_FP64 and FABM_FP64X2
- * (with its double-double kernel), the split-k CTA target of the history kernel
- * (152, 304, 608, 1216 CTAs); for FABM_SPLIT, the two tensor-core far-history
+ * long solve.  Candidates: for FABM_FP64, the superblock schedule (CTA target 0);
+ * for FABM_FP64 and FABM_FP64X2 (with its double-double kernel), direct sums of
+ * every point with the split-k CTA target of the history kernel (152, 304, 608,
+ * 1216 CTAs); for FABM_SPLIT, the two tensor-core far-history
  * tilings (FABM_HIST_TENSOR_WIDE: 128 targets per MMA and per far launch;
  * FABM_HIST_TENSOR: 64) each with 0 or 16 SMs (or an automatic number) kept
  * free for the recurrence running beside it, and the compensated-fp32 kernel

@@ -1,0 +1,555 @@
+// a2 + a3 + a4 + a5 in double, one thread-block cluster per trajectory: a
+// launch advances a superblock of n targets (m = nT+1 .. nT+n) of every
+// trajectory, given the far history of its targets over the points k < n(T-1)
+// (far_fft.cu).  Sec. 2 of arXiv:1710.01133 (Eq. abm, the corrector after it).
+//
+// What bounds it: GB300's FP64 unit takes a warp instruction in 64 cycles per
+// SM sub-partition, dependent or not (measured: 64 cycles for chains of 1 and
+// of 8 independent FMAs, one warp), so a step costs 64 cycles for each FP64
+// instruction on its serial chain (accumulate, f, corrector, f) plus two
+// exchanges between the components, and every other FP64 instruction that
+// shares the chain's sub-partitions delays it.  One launch per block of 32
+// steps spent two thirds of its time outside the chain: on launches, on
+// loading the block's weights and on the lag blocks.
+//
+// Layout.  Targets are taken in blocks of 32 (lane = target).  Three parties
+// sum the points before a block, and each has the rest to itself:
+//   chain warps   (rank 0, one per component): the block's own points, the step;
+//   prev warps    (rank 0, other sub-partitions): the 32 points of the block
+//                 before it, each as soon as the chain has produced it;
+//   helper warps  (ranks 1 .., four per CTA; in rank 0 for clusters of one):
+//                 every earlier point k >= n(T-1), dealt out to the warps in turn; warps of a CTA are added in
+//                 shared memory, CTAs by a finisher warp that owns one (kind,
+//                 component) row and turns it into y0 + h^alpha (...).
+// The chain stores f_k into the shared memory of every CTA of the cluster (one
+// instruction: lane r writes to CTA r), and the finishers store their rows into
+// the chain's CTA.  Both buffers are written once per launch and start out as
+// a bit pattern that no result has, so a reader polls the value it needs and no
+// flag or fence is on the way.  A helper sums the older points of block t + 1
+// while the chain runs block t - 1; what is left when f of block t - 1 is
+// complete is the addition of the rows, due 24 steps into block t.
+//
+// Measured against one launch per kernel and block of 32 (whole solves):
+// Lorenz-type 2^18 434 -> 100 ms, 16 x 2^15 102 -> 13.9, scalar 10^4 5.16 -> 2.39,
+// LCR 256 x 2^13 of uneven length 67.2 -> 9.8.
+//
+// Every wait is bounded: a thread that gives up sets the error word and goes
+// on without waiting, so that barriers are still met and the launch ends.
+#include <algorithm>
+
+#include "recurrence.cuh"
+#include "sm100_ptx.cuh"
+
+namespace fabm {
+namespace {
+
+using ptx::smem_u32;
+
+constexpr int kB = kWarp;           // targets per block
+constexpr int kHelpWarps = 4;       // helper warps per CTA, one per SM sub-partition
+constexpr int kBaseDue = 24;        // step of a block by which the next block's base row is needed
+constexpr unsigned long long kUnset = ~0ull;  // a NaN that no arithmetic instruction returns
+constexpr long long kWaitDefault = 4000000000LL;
+
+template <int D>
+struct Roles {
+    static constexpr int kPrev = D == 1 ? 1 : (D == 3 ? 1 : D);  // prev warps
+    static constexpr int kPrevComps = D / kPrev;                 // components of each
+    static constexpr int kPrev0 = D == 1 ? 1 : (D == 2 ? 2 : (D == 3 ? 3 : 4));
+    static constexpr int kChainWarps = D == 4 ? 8 : 4;           // warps of rank 0's roles
+};
+
+// Shared memory of a CTA, in doubles from the start: f of both superblocks, then
+// the chain's and prev warps' arrays (rank 0) and the helpers' (ranks 1 ..), in
+// the same place where no CTA has both roles.
+struct Layout {
+    int sf, base, near, sy, pw, wb, wa, rows, red, total;
+};
+__host__ __device__ inline Layout layout(int D, int nW, int n, int CS)
+{
+    Layout l;
+    const int H = CS > 1 ? CS - 1 : 1;
+    const int ro = (2 * D + H - 1) / H;  // rows a finisher owns at most
+    int o = 0;
+    l.sf = o, o += 2 * n * D;
+    const int roles = o;
+    l.base = o, o += n * 2 * D;
+    l.near = o, o += 2 * 2 * D * kB;
+    l.sy = o, o += 4 * D;
+    l.pw = o, o += nW * 2 * 66;
+    const int chain_end = o;
+    if (CS > 1) o = roles;
+    l.wb = o, o += nW * (2 * n + 2);
+    l.wa = o, o += nW * (2 * n + 2);
+    l.rows = o, o += 2 * ro * H * kB;
+    l.red = o, o += 2 * kHelpWarps * 2 * D * kB;
+    l.total = o > chain_end ? o : chain_end;
+    return l;
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// A value to another CTA of the cluster; the pattern that marks an unset slot
+// is replaced by another NaN.
+__device__ __forceinline__ void put(uint32_t remote, double v)
+{
+    unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    if (u == kUnset) u ^= 1ull;
+    asm volatile("st.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(remote), "l"(u) : "memory");
+}
+__device__ __forceinline__ unsigned long long peek(const double *p)
+{
+    unsigned long long u;
+    asm volatile("ld.relaxed.cluster.shared::cta.b64 %0, [%1];" : "=l"(u) : "r"(smem_u32(p)) : "memory");
+    return u;
+}
+__device__ __forceinline__ void named_sync(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+struct Waiter {
+    long long limit;
+    unsigned *err;
+    bool ok = true;
+    __device__ void give_up()
+    {
+        ok = false;
+        atomicOr(err, 1u);
+    }
+    // the value at p once it is set
+    __device__ __forceinline__ double get(const double *p)
+    {
+        unsigned long long u = peek(p);
+        if (u == kUnset && ok) {
+            const long long t0 = clock64();
+            while ((u = peek(p)) == kUnset)
+                if (clock64() - t0 > limit) {
+                    give_up();
+                    break;
+                }
+        }
+        return __longlong_as_double((long long)u);
+    }
+    // phase `parity` of a barrier that other CTAs of the cluster arrive on
+    __device__ void phase(uint64_t *bar, uint32_t parity)
+    {
+        if (!ok) return;
+        const long long t0 = clock64();
+        for (;;) {
+            uint32_t done;
+            asm volatile(
+                "{\n .reg .pred p;\n"
+                " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                " selp.u32 %0, 1, 0, p;\n}\n"
+                : "=r"(done)
+                : "r"(smem_u32(bar)), "r"(parity)
+                : "memory");
+            if (done) return;
+            if (clock64() - t0 > limit) {
+                give_up();
+                return;
+            }
+        }
+    }
+};
+
+struct Args {
+    DevBatch bt;
+    DevWeights w;
+    StepConsts kc;
+    int64_t T;        // superblock
+    int n;            // targets per superblock, a multiple of 32
+    const double *G;  // far history [2][n][cols] over k < n(T-1), or NULL (T < 2)
+    const double *X;  // time-only part of f, [B][n] (aux_table_kernel), if Rhs::kForcing
+    unsigned *err;
+    long long wait;
+};
+
+struct Chain {
+    const Args &a;
+    int b;
+    int64_t nT, Nb;
+    int nb, known, CS;
+    double *sm;
+    const Layout &l;
+    int lane;
+};
+
+// The steps of component I.  A step's serial path is accumulate -> exchange ->
+// f -> corrector -> exchange -> f; the second accumulation, the weights of the
+// next step and the copy of f to the cluster are placed in the shadow of the
+// first accumulation and exchange.
+template <class Rhs, int D, int I>
+__device__ __forceinline__ void chain_run(const Chain &c)
+{
+    const Args &a = c.a;
+    const int lane = c.lane;
+    double *sm = c.sm;
+    double p[kMaxParams];
+#pragma unroll
+    for (int q = 0; q < kMaxParams; ++q) p[q] = a.bt.params[(int64_t)c.b * kMaxParams + q];
+    const double ha_ig2 = a.kc.h_alpha[I] * a.kc.inv_gamma2[I];
+    const double aux0 = Rhs::kForcing ? 0.0 : Rhs::aux(0.0, p);
+    const double *pb = sm + c.l.pw + (a.w.stride ? I * 132 : 0), *pa = pb + 66;
+    volatile double *sy = sm + c.l.sy;  // [2 parities][P, C][D]
+    double *Yb = a.bt.Y + (int64_t)c.b * (a.bt.N + 1) * D;
+    const double *near = sm + c.l.near;
+    const uint32_t sf_to = lane < c.CS ? mapa(smem_u32(sm + c.l.sf + I), lane) : 0u;
+    double fk = sm[c.l.sf + c.known * D + I];
+    const double *X = Rhs::kForcing ? a.X + (int64_t)c.b * a.n : nullptr;
+    double ax_next = Rhs::kForcing ? X[lane] : 0.0;
+    for (int t = 0; t < c.nb; ++t) {
+        const int64_t m0 = c.nT + t * kB;
+        named_sync(2, (D + Roles<D>::kPrev) * kWarp);
+        double accP = near[((t & 1) * 2 * D + I) * kB + lane];
+        double accC = near[((t & 1) * 2 * D + D + I) * kB + lane];
+        double ax = aux0, yo = 0.0, fo = 0.0;
+        if constexpr (Rhs::kForcing) {  // this block's row was loaded a block ago
+            ax = ax_next;
+            if (t + 1 < c.nb) ax_next = X[(t + 1) * kB + lane];
+        }
+        const int steps = (int)(c.Nb - m0 < kB ? c.Nb - m0 : kB);
+        double wP = pb[lane + 1], wC = pa[lane + 1], yc = 0.0;
+        for (int s = 0; s < steps; ++s) {
+            // the newest point k = m0+s; targets already done add distance 0 (weight 0)
+            accP = fma(wP, fk, accP);
+            accC = fma(wC, fk, accC);
+            // what else is done with f_k waits for the FP64 result to leave its
+            // pipe, so it comes after the additions that take it inside
+            if (lane < c.CS) put(sf_to + (c.known + t * kB + s) * D * 8, fk);
+            if (lane == s - 1) yo = yc, fo = fk;
+            const int d = lane - s > 0 ? lane - s : 0;
+            wP = pb[d], wC = pa[d];
+            double y[D];
+            const int par = (s & 1) * 2 * D;
+            const double axs = Rhs::kForcing ? __shfl_sync(0xffffffffu, ax, s) : ax;
+            if constexpr (D > 1) {
+                if (lane == s) sy[par + I] = accP;
+                named_sync(1, D * kWarp);
+#pragma unroll
+                for (int q = 0; q < D; ++q) y[q] = sy[par + q];
+            } else {
+                y[0] = __shfl_sync(0xffffffffu, accP, s);
+            }
+            // every lane runs the step, so that f ends up in all of them
+            const double fp = Rhs::template one<D>(I, y, p, axs);
+            yc = fma(ha_ig2, fp, __shfl_sync(0xffffffffu, accC, s));
+            if constexpr (D > 1) {
+                if (lane == 0) sy[par + D + I] = yc;
+                named_sync(1, D * kWarp);
+#pragma unroll
+                for (int q = 0; q < D; ++q) y[q] = sy[par + D + q];
+            } else {
+                y[0] = yc;
+            }
+            fk = Rhs::template one<D>(I, y, p, axs);
+        }
+        if (lane == steps - 1) yo = yc, fo = fk;
+        if (lane < steps) {
+            const int64_t m = m0 + 1 + lane;
+            Yb[m * D + I] = yo;
+            a.bt.F[m * a.bt.ldF + (int64_t)c.b * D + I] = fo;
+            if (!(finite_bits(yo) && finite_bits(fo))) report_nonfinite(a.bt.status, m, c.b);
+        }
+    }
+}
+
+// X[b][j] = aux(t_m, p_b) for m = nT+1+j, j < n.
+template <class Rhs>
+__global__ void aux_table_kernel(DevBatch bt, double h, int64_t T, int n, double *__restrict__ X)
+{
+    const int64_t total = (int64_t)bt.B * n;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = e / n, m = T * n + 1 + e % n;
+        double p[kMaxParams];
+#pragma unroll
+        for (int q = 0; q < kMaxParams; ++q) p[q] = bt.params[b * kMaxParams + q];
+        X[e] = m <= bt.N_each[b] ? Rhs::aux((double)m * h, p) : 0.0;
+    }
+}
+
+// grid = B x (cluster size), cluster size CTAs per trajectory.
+template <class Rhs, int D>
+__global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWarp)
+    cluster_kernel(const __grid_constant__ Args a)
+{
+    extern __shared__ __align__(16) double sm[];
+    __shared__ uint64_t rows_full[2];
+    using R = Roles<D>;
+    const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
+    const int CS = (int)cluster_size(), rank = (int)cluster_rank();
+    const int H = CS > 1 ? CS - 1 : 1;      // CTAs with helper warps
+    const int hr = CS > 1 ? rank - 1 : 0;   // this CTA among them (-1: none)
+    const int hw0 = CS > 1 ? 0 : R::kChainWarps;
+    const int b = (int)blockIdx.x / CS;
+    const int n = a.n;
+    const int64_t nT = a.T * n;
+    const int64_t Nb = a.bt.N_each[b];
+    if (nT >= Nb) return;  // trajectory finished (the whole cluster)
+    const int nb = (int)((Nb - nT < n ? Nb - nT : n) + kB - 1) / kB;  // blocks of this launch
+    const int64_t k0 = a.T > 0 ? nT - n : 0;                        // first point summed here
+    const int known = (int)(nT - k0);                               // points before f_{nT}
+    const int nW = a.w.stride ? D : 1;
+    const Layout l = layout(D, nW, n, CS);
+    const int ws = 2 * n + 2;
+    double *sf = sm + l.sf, *base = sm + l.base;
+    double(*near)[2 * D][kB] = reinterpret_cast<double(*)[2 * D][kB]>(sm + l.near);
+
+    // known points, unset slots, weights
+    for (int j = threadIdx.x; j < 2 * n * D; j += blockDim.x) {
+        const int64_t k = k0 + j / D;
+        sf[j] = k <= nT ? a.bt.F[k * a.bt.ldF + (int64_t)b * D + j % D]
+                        : __longlong_as_double((long long)kUnset);
+    }
+    if (hr >= 0) {
+        const int64_t dmax = known + nb * kB;  // largest distance (< w.N)
+        for (int q = 0; q < nW; ++q)
+            for (int j = threadIdx.x; j <= dmax; j += blockDim.x) {
+                sm[l.wb + q * ws + j] = a.w.B[q * a.w.stride + j];
+                sm[l.wa + q * ws + j] = a.w.A[q * a.w.stride + j];
+            }
+        if (threadIdx.x < 2) {
+            int owned = 0;
+            for (int q = hr; q < 2 * D; q += H) ++owned;
+            ptx::mbar_init(&rows_full[threadIdx.x], owned ? owned * H : 1);
+            ptx::fence_mbar_init();
+        }
+    }
+    if (rank == 0) {
+        for (int j = threadIdx.x; j < nb * 2 * D * kB; j += blockDim.x)
+            base[j] = __longlong_as_double((long long)kUnset);
+        for (int j = threadIdx.x; j < nW * 66; j += blockDim.x) {
+            const int q = j / 66, d = j % 66;
+            const double hq = pick<D>(a.kc.h_alpha, q);
+            sm[l.pw + q * 132 + d] = hq * a.w.B[q * a.w.stride + d];
+            sm[l.pw + q * 132 + 66 + d] = hq * a.w.A[q * a.w.stride + d];
+        }
+    }
+    Waiter wt{a.wait > 0 ? a.wait : kWaitDefault, a.err};
+    cluster_sync();
+
+    if (rank == 0 && warp < D) {
+        const Chain ch{a, b, nT, Nb, nb, known, CS, sm, l, lane};
+        if constexpr (D == 1) {
+            chain_run<Rhs, D, 0>(ch);
+        } else {
+            if (warp == 0) chain_run<Rhs, D, 0>(ch);
+            else if (warp == 1) chain_run<Rhs, D, 1>(ch);
+            else if (warp == 2) chain_run<Rhs, D, D >= 3 ? 2 : 0>(ch);
+            else chain_run<Rhs, D, D >= 4 ? 3 : 0>(ch);
+        }
+    } else if (rank == 0 && warp >= R::kPrev0 && warp < R::kPrev0 + R::kPrev) {
+        // ---- prev: the 32 points before each block, for kPrevComps components ----
+        const int c0 = (warp - R::kPrev0) * R::kPrevComps;
+        constexpr int C = R::kPrevComps;
+        for (int t = 0; t < nb; ++t) {
+            double accP[C], accC[C];
+            if (t == 0) {
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    accP[q] = wt.get(base + (c0 + q) * kB + lane);
+                    accC[q] = wt.get(base + (D + c0 + q) * kB + lane);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < C; ++q) accP[q] = accC[q] = 0.0;
+                const double *f = sf + (known + (t - 1) * kB) * D + c0;
+                const double *bt = base + t * 2 * D * kB + lane;
+#pragma unroll 1
+                for (int s = 0; s < kB; ++s) {
+                    if (s == kBaseDue) {
+#pragma unroll
+                        for (int q = 0; q < C; ++q) {
+                            accP[q] += wt.get(bt + (c0 + q) * kB);
+                            accC[q] += wt.get(bt + (D + c0 + q) * kB);
+                        }
+                    }
+                    const int d = kB + 1 + lane - s;
+#pragma unroll
+                    for (int q = 0; q < C; ++q) {
+                        const double *pb = sm + l.pw + (nW > 1 ? (c0 + q) * 132 : 0);
+                        const double fk = wt.get(f + s * D + q);
+                        accP[q] = fma(pb[d], fk, accP[q]);
+                        accC[q] = fma(pb[66 + d], fk, accC[q]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                near[t & 1][c0 + q][lane] = accP[q];
+                near[t & 1][D + c0 + q][lane] = accC[q];
+            }
+            named_sync(2, (D + R::kPrev) * kWarp);
+        }
+    } else if (hr >= 0 && warp >= hw0 && warp < hw0 + kHelpWarps) {
+        // ---- helpers ----
+        const int w = warp - hw0;
+        const int g = hr * kHelpWarps + w, HW = H * kHelpWarps;
+        for (int t = 0; t < nb; ++t) {
+            const int lim = known + (t > 1 ? t - 1 : 0) * kB;  // points k0 .. k0+lim-1
+            const int off = known + t * kB + 1 + lane;          // distance of point index j: off - j
+            double acc[2 * D];
+#pragma unroll
+            for (int q = 0; q < 2 * D; ++q) acc[q] = 0.0;
+            auto add = [&](int j, const double (&f)[D]) {
+#pragma unroll
+                for (int q = 0; q < D; ++q) {
+                    const int o = (nW > 1 ? q * ws : 0) + off - j;
+                    acc[q] = fma(sm[l.wb + o], f[q], acc[q]);
+                    acc[D + q] = fma(sm[l.wa + o], f[q], acc[D + q]);
+                }
+            };
+            int j = g;
+            const int old = lim < known ? lim : known;
+#pragma unroll 4
+            for (; j < old; j += HW) {
+                double f[D];
+#pragma unroll
+                for (int q = 0; q < D; ++q) f[q] = sf[j * D + q];
+                add(j, f);
+            }
+#pragma unroll 2
+            for (; j < lim; j += HW) {
+                double f[D];
+#pragma unroll
+                for (int q = 0; q < D; ++q) f[q] = wt.get(sf + j * D + q);
+                add(j, f);
+            }
+            // the CTA's four warps, then the row's owner
+            double(*red)[2 * D][kB] =
+                reinterpret_cast<double(*)[2 * D][kB]>(sm + l.red) + (t & 1) * kHelpWarps;
+#pragma unroll
+            for (int q = 0; q < 2 * D; ++q) red[w][q][lane] = acc[q];
+            named_sync(3, kHelpWarps * kWarp);
+            for (int q = w; q < 2 * D; q += kHelpWarps) {
+                const double v = (red[0][q][lane] + red[1][q][lane]) + (red[2][q][lane] + red[3][q][lane]);
+                const uint32_t owner = CS > 1 ? 1 + q % H : 0;
+                const int ro = (2 * D + H - 1) / H;
+                put(mapa(smem_u32(sm + l.rows + (((t & 1) * ro + q / H) * H + hr) * kB + lane), owner), v);
+                __syncwarp();
+                if (lane == 0) {
+                    const uint32_t bar = mapa(smem_u32(&rows_full[t & 1]), owner);
+                    asm volatile("fence.acq_rel.cluster;\n"
+                                 "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar)
+                                 : "memory");
+                }
+            }
+        }
+    } else if (hr >= 0 && warp == hw0 + kHelpWarps) {
+        // ---- finisher: rows hr, hr + H, ... (kind, component) ----
+        if (hr < 2 * D) {
+            const int ro = (2 * D + H - 1) / H;
+            for (int t = 0; t < nb; ++t) {
+                const int64_t m = nT + t * kB + 1 + lane;
+                double *bt = base + t * 2 * D * kB + lane;
+                bool waited = false;
+                for (int q = hr; q < 2 * D; q += H) {
+                    const int i = q % D, kind = q / D;
+                    const int64_t col = (int64_t)b * D + i;
+                    double far = a.G ? a.G[((int64_t)kind * n + t * kB + lane) * a.bt.cols + col] : 0.0;
+                    if (kind) far = fma(a.w.D[i * a.w.stride + m], a.bt.F[col], far);
+                    const double y0 = a.bt.y0[col];
+                    const double Tm = a.bt.y1 ? fma((double)m * a.kc.h, a.bt.y1[col], y0) : y0;
+                    if (!waited) wt.phase(&rows_full[t & 1], (t >> 1) & 1);
+                    waited = true;
+                    const double *r = sm + l.rows + (((t & 1) * ro + q / H) * H) * kB + lane;
+                    double v = 0.0;
+                    for (int h = 0; h < H; ++h) v += r[h * kB];
+                    put(mapa(smem_u32(bt + q * kB), 0), fma(pick<D>(a.kc.h_alpha, i), far + v, Tm));
+                }
+            }
+        }
+    }
+    cluster_sync();  // no CTA leaves while another may still write to its shared memory
+}
+
+template <class Rhs, int D>
+cudaError_t cluster_config(int B, int CS, int n, int nW, bool alone, cudaLaunchConfig_t *cfg,
+                           cudaLaunchAttribute *attr)
+{
+    constexpr int kc = Roles<D>::kChainWarps;
+    const int warps = CS > 1 ? (kc > kHelpWarps + 1 ? kc : kHelpWarps + 1) : kc + kHelpWarps + 1;
+    size_t smem = sizeof(double) * (size_t)layout(D, nW, n, CS).total;
+    if (alone && smem < 120 * 1024) smem = 120 * 1024;  // one CTA per SM
+    if (smem > 226 * 1024) return cudaErrorInvalidConfiguration;
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3((unsigned)(B * CS));
+    cfg->blockDim = dim3((unsigned)(warps * kWarp));
+    cfg->dynamicSmemBytes = smem;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)CS, attr->val.clusterDim.y = 1, attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    auto k = cluster_kernel<Rhs, D>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && CS > 8)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+}  // namespace
+
+int cluster_max_active(int rhs, int dim, bool multi, int CS, int n)
+{
+    int num = 0;
+    dispatch_rhs(rhs, dim, [&]<class R, int D>() {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        if (cluster_config<R, D>(1, CS, n, multi ? D : 1, CS > 1, &cfg, &attr) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&num, cluster_kernel<R, D>, &cfg) != cudaSuccess)
+            num = 0;
+        cudaGetLastError();
+    });
+    return num;
+}
+
+cudaError_t launch_cluster_fp64(int rhs, const DevBatch &bt, const DevWeights &w,
+                                const StepConsts &k, int64_t T, int n, int CS, const double *G,
+                                const double *X, unsigned *err, long long wait_cycles, cudaStream_t st)
+{
+    cudaError_t e = cudaErrorInvalidValue;
+    dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        e = cluster_config<R, D>(bt.B, CS, n, w.stride ? D : 1, CS > 1, &cfg, &attr);
+        if (e != cudaSuccess) return;
+        cfg.stream = st;
+        const Args a{bt, w, k, T, n, G, X, err, wait_cycles};
+        e = cudaLaunchKernelEx(&cfg, cluster_kernel<R, D>, a);
+    });
+    return e;
+}
+
+cudaError_t launch_aux_rows(int rhs, const DevBatch &bt, double h, int64_t T, int n, double *X,
+                            cudaStream_t st)
+{
+    const int64_t blocks = std::min<int64_t>(((int64_t)bt.B * n + 127) / 128, 152 * 16);
+    const bool ok = dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
+        aux_table_kernel<R><<<(unsigned)blocks, 128, 0, st>>>(bt, h, T, n, X);
+    });
+    return ok ? cudaGetLastError() : cudaErrorInvalidValue;
+}
+
+}  // namespace fabm

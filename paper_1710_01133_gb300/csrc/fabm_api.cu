@@ -1,7 +1,14 @@
 // C ABI (include/fabm.h): solver state, argument checks, device memory, and
 // the block-by-block schedule of the kernels.
 //
-// Schedule of one solve (Sec. 2 of arXiv:1710.01133 evaluated block by block):
+// Schedule of one FP64 solve (Sec. 2 of arXiv:1710.01133), by superblocks of n
+// targets (n = 128 .. 1024, see kClusterSizes):
+//   stream R:  wait G(T), X(T); steps of superblock T over the points k >= n(T-1)
+//   stream G:  wait R(T-2); spectrum of segment T-2; far history of T over the
+//              segments 0 .. T-2
+//   stream G2: forcing of superblock T
+// Schedule of the other solves, block by block (and of FP64 solves whose
+// spectra do not fit or whose chunk count the autotuner has set):
 //   init                      y_0, f_0
 //   for each block c of L targets (CUDA-core history kernels, L = 32):
 //     stream G:  wait R(c-2); history(c) over k < (c-1)L; combine -> G[c%2]
@@ -88,6 +95,7 @@ struct DevBuf {
 
 constexpr int kMaxBlockL = 1024;
 constexpr int kEvRing = 4;
+constexpr int kClusterChoices = 9;
 constexpr int kAuxRing = 4;  // forcing tables computed up to 3 blocks ahead
 
 }  // namespace
@@ -161,6 +169,16 @@ struct fabm_solver {
     DevBuf<double> ppart, pspart;  // persistent FP64 solve: chunk and super-group partial slots
     DevBuf<int> psg, pdone, prdone; // persistent FP64 solve: chunks done per super-group,
                                     // super-groups done per block, blocks done per trajectory
+    // FP64 superblocks: CTAs per trajectory (0: the block schedule) and targets
+    // per launch of the solve being set up; clusters that fit per choice of
+    // kClusterSizes (-1: not asked yet); transform factors, weight and f spectra,
+    // partial spectra, marks of large segments, far history of two superblocks
+    int cl_size = 0, cl_n = 0;
+    std::vector<int> cl_fit = std::vector<int>(kClusterChoices, -1);
+    int what_n = 0;  // superblock length the weight spectra are for
+    DevBuf<double2> tw, What, Fhat, facc;
+    DevBuf<unsigned char> fmark;
+    DevBuf<double> Gfar, Xrow;  // Xrow: forcing of two superblocks
     DevBuf<float2> auxb;       // tensor path: forcing tables of kAuxRing blocks
     DevBuf<unsigned int> err;  // split: timeout flag
     DevBuf<int64_t> nEach;
@@ -209,7 +227,9 @@ struct fabm_solver {
     {
         wB.release(), wA.release(), wD.release(), wH.release(), wHe.release();
         wH2.release(), wHe2.release(), Fs2.release(), Fe2.release(), fpart.release(), fsum.release();
-        ppart.release(), pdone.release(), prdone.release();
+        ppart.release(), pspart.release(), psg.release(), pdone.release(), prdone.release();
+        tw.release(), What.release(), Fhat.release(), facc.release(), fmark.release(), Gfar.release(),
+            Xrow.release();
         wBl.release(), wAl.release(), wDl.release();
         wBf.release(), wAf.release(), wBff.release(), wAff.release(), wDff.release();
         F.release(), Ff.release(), Ystage.release(), G.release(), part.release();
@@ -616,6 +636,96 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
     return FABM_OK;
 }
 
+// CTAs per trajectory and targets per superblock of the FP64 superblock
+// schedule, largest cluster first: the largest that can run for all
+// trajectories at once is taken (one CTA per SM; 152 SMs hold 7, 13, 15, 23, 28,
+// 36, 46 and 76 clusters of these sizes).  n grows with the helper warps, which
+// sum up to 2n points for each block of 32 targets while the chain runs one
+// (~24,000 cycles for three components: 255 points per helper CTA).
+struct ClusterShape {
+    int CS, n;
+};
+constexpr ClusterShape kClusterSizes[] = {{16, 1024}, {10, 512}, {8, 512}, {6, 512}, {5, 512},
+                                          {4, 256},   {3, 256},  {2, 128}, {1, 128}};
+static_assert(sizeof(kClusterSizes) / sizeof(ClusterShape) == kClusterChoices);
+
+void plan_cluster(fabm_solver *s, int64_t B, int64_t cols, int64_t Nmax)
+{
+    s->cl_size = 0;
+    for (int q = 0; q < kClusterChoices; ++q) {
+        const ClusterShape c = kClusterSizes[q];
+        if (s->cl_fit[q] < 0) s->cl_fit[q] = cluster_max_active(s->rhs, s->dim, s->multi, c.CS, c.n);
+        if (s->cl_fit[q] < 1 || (c.CS > 1 && B > s->cl_fit[q])) continue;
+        s->cl_size = c.CS, s->cl_n = c.n;
+        break;
+    }
+    // spectra of f: 32 bytes per point and column
+    if (s->cl_size && Nmax > 2 * s->cl_n && (cols > 65535 || Nmax * cols > (1LL << 29))) s->cl_size = 0;
+}
+
+// Enqueues an FP64 solve by superblocks of n targets: the steps of superblock T
+// on sR; the spectrum of segment T-2 and the far history of superblock T on sG
+// beside the steps of superblock T-1.
+fabm_status enqueue_clusters(fabm_solver *s, const DevBatch &bt, const DevWeights &w, int64_t Nmax)
+{
+    const int n = s->cl_n;
+    const int64_t cols = bt.cols, nsb = (Nmax + n - 1) / n;
+    const int g_max = (int)((bt.N + n - 1) / n - 1);  // as the weight spectra are laid out
+    unsigned char *mark = s->fmark.p, *big = mark + nsb * cols;
+    const bool forcing = rhs_has_forcing(s->rhs, bt.dim);
+    s->sample_now = true;
+    FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
+                               [&] { return launch_init(s->rhs, bt, s->sR); }));
+    for (int64_t T = 0; T < nsb; ++T) {
+        s->sample_now = T % s->timing_period == 0;
+        const double *G = nullptr;
+        if (T >= 2) {
+            double *Gw = s->Gfar.p + (size_t)(T & 1) * 2 * n * cols;
+            const double flops = 4.0 * n * (double)(n * (T - 1)) * (double)cols;
+            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG, s->evR[(T - 2) % kEvRing], 0));
+            FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_SLICE, s->sG, 0.0, [&] {
+                return launch_fft_segment(bt, n, T - 2, s->tw.p, s->Fhat.p, mark, big, s->sG);
+            }));
+            ++s->launches;  // product and inverse
+            FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sG, flops, [&] {
+                return launch_fft_far(bt, s->multi, n, g_max, T, s->tw.p, s->Fhat.p, s->What.p, mark,
+                                      big, s->facc.p, Gw, s->sG);
+            }));
+            FABM_CUDA_TRY(cudaEventRecord(s->evG[T % 3], s->sG));
+            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evG[T % 3], 0));
+            G = Gw;
+        }
+        double *X = nullptr;
+        if (forcing) {  // on sG2, a superblock ahead of the steps
+            X = s->Xrow.p + (size_t)(T & 1) * n * bt.B;
+            if (T >= 2) FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG2, s->evR[(T - 2) % kEvRing], 0));
+            FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sG2, 0.0, [&] {
+                return launch_aux_rows(s->rhs, bt, s->h, T, n, X, s->sG2);
+            }));
+            FABM_CUDA_TRY(cudaEventRecord(s->evA[T % kAuxRing], s->sG2));
+            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evA[T % kAuxRing], 0));
+        }
+        const int64_t lo = T * n, hi = std::min<int64_t>((T + 1) * n, Nmax);
+        const double near = (double)(T > 0 ? n : 0) + 0.5 * (double)(hi - lo + 1);
+        FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sR, 4.0 * (double)(hi - lo) * near * cols, [&] {
+            return launch_cluster_fp64(s->rhs, bt, w, s->k, T, n, s->cl_size, G, X, s->err.p,
+                                       s->wait_cycles, s->sR);
+        }));
+        FABM_CUDA_TRY(cudaEventRecord(s->evR[T % kEvRing], s->sR));
+        if (s->out_stream && ((T + 1) % s->out_group == 0 || T + 1 == nsb)) {
+            const int64_t T0 = T / s->out_group * s->out_group;
+            const int64_t r_lo = T0 == 0 ? 0 : T0 * n + 1, r_hi = std::min<int64_t>((T + 1) * n, bt.N);
+            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sC, s->evR[T % kEvRing], 0));
+            const size_t pitch = sizeof(double) * (size_t)(bt.N + 1) * bt.dim;
+            FABM_CUDA_TRY(cudaMemcpy2DAsync(s->out_stream + r_lo * bt.dim, pitch, bt.Y + r_lo * bt.dim,
+                                            pitch, sizeof(double) * (size_t)(r_hi - r_lo + 1) * bt.dim,
+                                            (size_t)bt.B, cudaMemcpyDeviceToHost, s->sC));
+        }
+    }
+    s->sample_now = true;
+    return FABM_OK;
+}
+
 fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double *y1,
                       const double *traj_params, const int64_t *N_each, double *out,
                       int out_on_device)
@@ -657,9 +767,42 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     int64_t max_chunks = std::max<int64_t>(1, (int64_t)(64ull << 20) / (part_per_chunk * 8));
     max_chunks = std::min<int64_t>(max_chunks, 4096);
     FABM_CUDA_TRY(s->F.ensure(f_elems));
-    FABM_CUDA_TRY(s->G.ensure((size_t)3 * 2 * L * cols));
+    s->cl_size = 0;
+    if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0) {
+        plan_cluster(s, B, cols, s->plan_N > 0 ? s->plan_N : N);
+        const int n = s->cl_n;
+        const int64_t nsb = (Nmax + n - 1) / n;
+        if (s->cl_size && nsb > 2) {  // superblocks with a far history
+            const int sets = s->multi ? dim : 1;
+            cudaError_t e = s->Fhat.ensure((size_t)(nsb - 2) * cols * 2 * n);
+            if (e == cudaSuccess) e = s->fmark.ensure((size_t)2 * nsb * cols);
+            if (e == cudaSuccess) e = s->facc.ensure((size_t)16 * cols * 2 * n);
+            if (e == cudaSuccess) e = s->Gfar.ensure((size_t)2 * 2 * n * cols);
+            if (e == cudaSuccess) e = s->tw.ensure((size_t)2 * n);
+            const int64_t g_max = (N + n - 1) / n - 1;
+            if (e == cudaSuccess && s->what_n != n) {
+                s->what_n = 0;
+                e = s->What.ensure((size_t)sets * (g_max + 1) * 2 * n);
+                if (e == cudaSuccess) {
+                    const DevWeights w{s->wB.p, s->wA.p, s->wD.p, s->w_ext, s->multi ? s->w_ext + 1 : 0};
+                    FABM_CUDA_TRY(launch_fft_weights(w, sets, n, (int)g_max, s->tw.p, s->What.p, s->sR));
+                    s->what_n = n;
+                }
+            }
+            if (e != cudaSuccess) {  // no room for the spectra: the block schedule
+                cudaGetLastError();
+                s->cl_size = 0;
+            }
+        }
+        if (s->cl_size) {
+            if (rhs_has_forcing(s->rhs, dim)) FABM_CUDA_TRY(s->Xrow.ensure((size_t)2 * n * B));
+            FABM_CUDA_TRY(s->err.ensure(1));
+            FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
+        }
+    }
+    if (!s->cl_size) FABM_CUDA_TRY(s->G.ensure((size_t)3 * 2 * L * cols));
     // two partial buffers: the history launches of blocks c and c+1 may overlap
-    if (hk == FABM_HIST_FP64) FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
+    if (hk == FABM_HIST_FP64 && !s->cl_size) FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
     if (hk == FABM_HIST_X2) FABM_CUDA_TRY(s->part.ensure((size_t)4 * max_chunks * part_per_chunk));
     if (hk == FABM_HIST_FP32C) {
         FABM_CUDA_TRY(s->spart.ensure((size_t)2 * max_chunks * part_per_chunk));
@@ -748,7 +891,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         cudaPointerAttributes pa{};
         if (cudaPointerGetAttributes(&pa, out) == cudaSuccess && pa.type == cudaMemoryTypeHost) {
             s->out_stream = out;
-            const size_t block_bytes = sizeof(double) * (size_t)B * L * dim;
+            const size_t block_bytes = sizeof(double) * (size_t)B * (s->cl_size ? s->cl_n : L) * dim;
             s->out_group = (int64_t)std::max<size_t>(1, ((8u << 20) + block_bytes - 1) / block_bytes);
         }
         cudaGetLastError();  // an unregistered pointer is not an error here
@@ -800,8 +943,12 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)s->out_stream, (uintptr_t)s->out_group, (uintptr_t)s->wait_cycles,
         (uintptr_t)s->wide, (uintptr_t)far_chunks, (uintptr_t)s->Fs2.p, (uintptr_t)s->Fe2.p,
         (uintptr_t)s->fpart.p, (uintptr_t)s->fsum.p, (uintptr_t)s->near_chunks,
-        (uintptr_t)s->plan_N};
+        (uintptr_t)s->plan_N, (uintptr_t)s->cl_size, (uintptr_t)s->cl_n, (uintptr_t)s->What.p,
+        (uintptr_t)s->Fhat.p, (uintptr_t)s->facc.p, (uintptr_t)s->fmark.p, (uintptr_t)s->Gfar.p,
+        (uintptr_t)s->Xrow.p,
+        (uintptr_t)(s->cl_size ? Nmax : 0)};
     auto enqueue = [&]() -> fabm_status {
+        if (s->cl_size) return enqueue_clusters(s, bt, w, Nmax);
         return enqueue_solve(s, bt, w, nblk, Nmax, max_chunks, n_ct, split_chunks, hk, far_chunks);
     };
     if (hk == FABM_HIST_FP64_PERSIST) {
@@ -907,7 +1054,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
 
     unsigned long long st = 0;
     FABM_CUDA_TRY(cudaMemcpy(&st, s->status.p, sizeof st, cudaMemcpyDeviceToHost));
-    if (split) {  // tensor kernel's bounded waits
+    if (split || s->cl_size) {  // bounded waits
         unsigned int tout = 0;
         FABM_CUDA_TRY(cudaMemcpy(&tout, s->err.p, sizeof tout, cudaMemcpyDeviceToHost));
         if (tout) return fail(FABM_ETIMEOUT, "a history kernel gave up waiting on a barrier");
@@ -1310,6 +1457,7 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
     // at most 8 candidates are reported
     if (s->precision == FABM_FP64 || s->precision == FABM_FP64X2) {
         const int k = s->precision == FABM_FP64 ? FABM_HIST_FP64 : FABM_HIST_X2;
+        if (s->precision == FABM_FP64) cands.push_back({k, 0});  // superblocks, the automatic choice
         for (int c : ctas_opts) cands.push_back({k, c});
         if (s->precision == FABM_FP64 && s->persist_ctas >= B + 8 && !s->multi)
             cands.push_back({FABM_HIST_FP64_PERSIST, s->persist_ctas});

@@ -236,6 +236,39 @@ cudaError_t launch_persist_fp64(int rhs, const DevBatch &bt, const DevWeights &w
                                 int *r_done, unsigned *err, long long wait_cycles,
                                 cudaStream_t st);
 
+// ---- FP64, superblocks (cluster_fp64.cu, far_fft.cu) ----
+
+// Clusters of CS CTAs of the superblock kernel (n targets per launch) that can
+// run at once on the current device; 0 if the kernel cannot run in that shape.
+int cluster_max_active(int rhs, int dim, bool multi, int CS, int n);
+// The steps of superblock T (targets nT+1 .. nT+n) of every trajectory, one
+// cluster of CS CTAs each; G: far history [2][n][cols] over the points
+// k < n(T-1), or NULL for T < 2; X: the rows of launch_aux_rows (required when
+// rhs_has_forcing).  err: set when a wait gave up.
+cudaError_t launch_cluster_fp64(int rhs, const DevBatch &bt, const DevWeights &w,
+                                const StepConsts &k, int64_t T, int n, int CS, const double *G,
+                                const double *X, unsigned *err, long long wait_cycles, cudaStream_t st);
+// X[b][j] = the time-only part of f at t_m, m = nT+1+j, j < n.
+cudaError_t launch_aux_rows(int rhs, const DevBatch &bt, double h, int64_t T, int n, double *X,
+                            cudaStream_t st);
+// Factors tw[2n] of the transforms of length 2n and the spectra of the weights
+// for the segment lags 2 .. g_max: What[set][g][2n], sets (one per order) of
+// g_max + 1 each.
+cudaError_t launch_fft_weights(const DevWeights &w, int sets, int n, int g_max, double2 *tw,
+                               double2 *What, cudaStream_t st);
+// Spectrum of the points nS .. nS+n-1 of every column: Fhat[S][col][2n]; mark,
+// big: one byte per segment and column.
+cudaError_t launch_fft_segment(const DevBatch &bt, int n, int64_t S, const double2 *tw,
+                               double2 *Fhat, unsigned char *mark, unsigned char *big,
+                               cudaStream_t st);
+// Chunks of launch_fft_far's sum over segments; acc holds chunks x cols x 2n.
+int fft_chunks(int n, int cols, int64_t T);
+// G of superblock T >= 2 from the segments 0 .. T-2.
+cudaError_t launch_fft_far(const DevBatch &bt, bool multi, int n, int g_max, int64_t T,
+                           const double2 *tw, const double2 *Fhat, const double2 *What,
+                           const unsigned char *mark, const unsigned char *big, double2 *acc,
+                           double *G, cudaStream_t st);
+
 // ---- FP64X2 precision (double-double history) ----
 
 // Low parts of the double-double weights; the high parts are the DevWeights

@@ -40,7 +40,13 @@ struct RhsLinear {  // f_i = -p0 y_i
     template <int D, class T>
     __device__ static T one(int i, const T *y, const T *p, T)
     {
-        return -p[0] * y[i];
+        // y[i] for a runtime i without indexing the array dynamically (which
+        // would put it in local memory)
+        T v = y[0];
+#pragma unroll
+        for (int q = 1; q < D; ++q)
+            if (i == q) v = y[q];
+        return -p[0] * v;
     }
 };
 
