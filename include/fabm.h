@@ -159,7 +159,7 @@ enum {
                               cores for batches of at least 64 columns, else FP32C;
                               FP64X2 precision: FABM_HIST_X2                         */
     FABM_HIST_FP64 = 1,    /* double on CUDA cores (FP64 precision only): the points of
-                              the last two superblocks of 128 to 1024 steps summed
+                              the last two superblocks of 128 to 512 steps summed
                               directly, older ones by transforms of a superblock's
                               points (32 bytes of device memory per step and column
                               beyond two superblocks; without that room, every point

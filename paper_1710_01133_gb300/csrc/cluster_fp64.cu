@@ -12,26 +12,38 @@
 // steps spent two thirds of its time outside the chain: on launches, on
 // loading the block's weights and on the lag blocks.
 //
-// Layout.  Targets are taken in blocks of 32 (lane = target).  Three parties
-// sum the points before a block, and each has the rest to itself:
+// Layout.  Targets are taken in blocks of 16; lane (kind, a) has target a's
+// predictor (kind 0) or corrector (1) sum, so one FMA adds a point to both sums
+// of a block.  Three parties share a block's sums, each with FP64 units to itself:
 //   chain warps   (rank 0, one per component): the block's own points, the step;
-//   prev warps    (rank 0, other sub-partitions): the 32 points of the block
+//   prev warps    (rank 0, other sub-partitions): the 16 points of the block
 //                 before it, each as soon as the chain has produced it;
-//   helper warps  (ranks 1 .., four per CTA; in rank 0 for clusters of one):
-//                 every earlier point k >= n(T-1), dealt out to the warps in turn; warps of a CTA are added in
-//                 shared memory, CTAs by a finisher warp that owns one (kind,
-//                 component) row and turns it into y0 + h^alpha (...).
+//   helper warps  (ranks 1 .., four per CTA; in rank 0 for clusters of one): every
+//                 earlier point k >= n(T-1), dealt out to the warps in turn; the
+//                 warps of a CTA are added in shared memory, the CTAs by a
+//                 finisher warp that owns a component's row and turns it into
+//                 y0 + h^alpha (...).
 // The chain stores f_k into the shared memory of every CTA of the cluster (one
 // instruction: lane r writes to CTA r), and the finishers store their rows into
 // the chain's CTA.  Both buffers are written once per launch and start out as
 // a bit pattern that no result has, so a reader polls the value it needs and no
 // flag or fence is on the way.  A helper sums the older points of block t + 1
 // while the chain runs block t - 1; what is left when f of block t - 1 is
-// complete is the addition of the rows, due 24 steps into block t.
+// complete is the addition of the rows, due 11 steps into block t.
+//
+// An FP64 result reaches the other units (shared memory, shuffles, integer
+// code) about 50 cycles later than the FP64 unit itself, and a store to 16 CTAs
+// holds up the stores behind it, so only the exchange stands between the
+// instructions of a step, and the copies of f follow it.  Cycles per step: 355
+// for the scalar system (five FP64 instructions), 720 for the Lorenz type (six
+// and two exchanges).  Blocks of 32 with a warp instruction per kind took 457
+// and 765; a chain of newest points only, the rest of the block summed by
+// another warp a target ahead, 560 and 920 (the way there and back is longer
+// than a step).
 //
 // Measured against one launch per kernel and block of 32 (whole solves):
-// Lorenz-type 2^18 434 -> 100 ms, 16 x 2^15 102 -> 13.9, scalar 10^4 5.16 -> 2.39,
-// LCR 256 x 2^13 of uneven length 67.2 -> 9.8.
+// Lorenz-type 2^18 434 -> 91 ms, 16 x 2^15 102 -> 12.7, scalar 10^4 5.16 -> 1.79,
+// LCR 256 x 2^13 of uneven length 67.2 -> 7.8.
 //
 // Every wait is bounded: a thread that gives up sets the error word and goes
 // on without waiting, so that barriers are still met and the launch ends.
@@ -45,16 +57,17 @@ namespace {
 
 using ptx::smem_u32;
 
-constexpr int kB = kWarp;           // targets per block
+constexpr int kB = 16;              // targets per block: a half-warp per kind
 constexpr int kHelpWarps = 4;       // helper warps per CTA, one per SM sub-partition
-constexpr int kBaseDue = 24;        // step of a block by which the next block's base row is needed
+constexpr int kBaseDue = 11;        // step of a block by which the next block's base row is needed
+constexpr int kPw = 2 * (2 * kB + 2);  // h^a B(d), h^a A(d), d <= 2 kB + 1
 constexpr unsigned long long kUnset = ~0ull;  // a NaN that no arithmetic instruction returns
 constexpr long long kWaitDefault = 4000000000LL;
 
 template <int D>
 struct Roles {
     static constexpr int kPrev = D == 1 ? 1 : (D == 3 ? 1 : D);  // prev warps
-    static constexpr int kPrevComps = D / kPrev;                 // components of each
+    static constexpr int kPrevComps = D / kPrev;                  // components of each
     static constexpr int kPrev0 = D == 1 ? 1 : (D == 2 ? 2 : (D == 3 ? 3 : 4));
     static constexpr int kChainWarps = D == 4 ? 8 : 4;           // warps of rank 0's roles
 };
@@ -69,20 +82,20 @@ __host__ __device__ inline Layout layout(int D, int nW, int n, int CS)
 {
     Layout l;
     const int H = CS > 1 ? CS - 1 : 1;
-    const int ro = (2 * D + H - 1) / H;  // rows a finisher owns at most
+    const int ro = (D + H - 1) / H;  // rows a finisher owns at most
     int o = 0;
     l.sf = o, o += 2 * n * D;
     const int roles = o;
     l.base = o, o += n * 2 * D;
-    l.near = o, o += 2 * 2 * D * kB;
+    l.near = o, o += 2 * D * kWarp;
     l.sy = o, o += 4 * D;
-    l.pw = o, o += nW * 2 * 66;
+    l.pw = o, o += nW * kPw;
     const int chain_end = o;
     if (CS > 1) o = roles;
     l.wb = o, o += nW * (2 * n + 2);
     l.wa = o, o += nW * (2 * n + 2);
-    l.rows = o, o += 2 * ro * H * kB;
-    l.red = o, o += 2 * kHelpWarps * 2 * D * kB;
+    l.rows = o, o += 2 * ro * H * kWarp;
+    l.red = o, o += 2 * kHelpWarps * D * kWarp;
     l.total = o > chain_end ? o : chain_end;
     return l;
 }
@@ -190,73 +203,84 @@ struct Chain {
     const Args &a;
     int b;
     int64_t nT, Nb;
-    int nb, known, CS;
+    int known, CS;
     double *sm;
     const Layout &l;
     int lane;
 };
 
-// The steps of component I.  A step's serial path is accumulate -> exchange ->
-// f -> corrector -> exchange -> f; the second accumulation, the weights of the
-// next step and the copy of f to the cluster are placed in the shadow of the
-// first accumulation and exchange.
+// The steps of component I; lane (kind, ta) has the sum of target ta of the
+// block.  A step's serial path is newest point -> exchange -> f -> corrector ->
+// exchange -> f; what else uses f_k is placed behind the addition that takes it
+// inside the FP64 unit.
 template <class Rhs, int D, int I>
 __device__ __forceinline__ void chain_run(const Chain &c)
 {
     const Args &a = c.a;
-    const int lane = c.lane;
+    const int lane = c.lane, ta = lane % kB;
     double *sm = c.sm;
     double p[kMaxParams];
 #pragma unroll
     for (int q = 0; q < kMaxParams; ++q) p[q] = a.bt.params[(int64_t)c.b * kMaxParams + q];
     const double ha_ig2 = a.kc.h_alpha[I] * a.kc.inv_gamma2[I];
     const double aux0 = Rhs::kForcing ? 0.0 : Rhs::aux(0.0, p);
-    const double *pb = sm + c.l.pw + (a.w.stride ? I * 132 : 0), *pa = pb + 66;
+    const double *pw = sm + c.l.pw + (a.w.stride ? I * kPw : 0) + (lane / kB) * (kPw / 2);
     volatile double *sy = sm + c.l.sy;  // [2 parities][P, C][D]
-    double *Yb = a.bt.Y + (int64_t)c.b * (a.bt.N + 1) * D;
-    const double *near = sm + c.l.near;
+    double *Yb = a.bt.Y + ((int64_t)c.b * (a.bt.N + 1) + c.nT + 1) * D + I;
+    double *Fb = a.bt.F + (c.nT + 1) * a.bt.ldF + (int64_t)c.b * D + I;
+    const double *near = sm + c.l.near + I * kWarp + lane;
     const uint32_t sf_to = lane < c.CS ? mapa(smem_u32(sm + c.l.sf + I), lane) : 0u;
-    double fk = sm[c.l.sf + c.known * D + I];
+    double fk = sm[c.l.sf + c.known * D + I], yc = 0.0, yo = 0.0, fo = 0.0;
     const double *X = Rhs::kForcing ? a.X + (int64_t)c.b * a.n : nullptr;
-    double ax_next = Rhs::kForcing ? X[lane] : 0.0;
-    for (int t = 0; t < c.nb; ++t) {
-        const int64_t m0 = c.nT + t * kB;
-        named_sync(2, (D + Roles<D>::kPrev) * kWarp);
-        double accP = near[((t & 1) * 2 * D + I) * kB + lane];
-        double accC = near[((t & 1) * 2 * D + D + I) * kB + lane];
-        double ax = aux0, yo = 0.0, fo = 0.0;
-        if constexpr (Rhs::kForcing) {  // this block's row was loaded a block ago
-            ax = ax_next;
-            if (t + 1 < c.nb) ax_next = X[(t + 1) * kB + lane];
+    double ax = aux0, ax_next = Rhs::kForcing ? X[lane] : 0.0;  // rows of 32 values, one ahead
+    const int steps = (int)(c.Nb - c.nT < a.n ? c.Nb - c.nT : a.n);
+    auto flush = [&](int j0, int cnt) {  // targets j0 .., a lane each
+        if (lane < cnt) {
+            Yb[(int64_t)(j0 + lane) * D] = yo;
+            Fb[(int64_t)(j0 + lane) * a.bt.ldF] = fo;
+            if (!(finite_bits(yo) && finite_bits(fo)))
+                report_nonfinite(a.bt.status, c.nT + 1 + j0 + lane, c.b);
         }
-        const int steps = (int)(c.Nb - m0 < kB ? c.Nb - m0 : kB);
-        double wP = pb[lane + 1], wC = pa[lane + 1], yc = 0.0;
-        for (int s = 0; s < steps; ++s) {
-            // the newest point k = m0+s; targets already done add distance 0 (weight 0)
-            accP = fma(wP, fk, accP);
-            accC = fma(wC, fk, accC);
-            // what else is done with f_k waits for the FP64 result to leave its
-            // pipe, so it comes after the additions that take it inside
-            if (lane < c.CS) put(sf_to + (c.known + t * kB + s) * D * 8, fk);
-            if (lane == s - 1) yo = yc, fo = fk;
-            const int d = lane - s > 0 ? lane - s : 0;
-            wP = pb[d], wC = pa[d];
+    };
+    for (int j0 = 0; j0 < steps; j0 += kB) {
+        if (j0 % kWarp == 0) {
+            if constexpr (Rhs::kForcing) {
+                ax = ax_next;
+                if (j0 + kWarp + lane < a.n) ax_next = X[j0 + kWarp + lane];
+            }
+        }
+        double w = pw[ta + 1];
+        const int cnt = steps - j0 < kB ? steps - j0 : kB;
+        named_sync(2, (D + Roles<D>::kPrev) * kWarp);
+        double acc = near[(j0 / kB & 1) * D * kWarp];
+        for (int s = 0; s < cnt; ++s) {  // target nT+1+j0+s
+            const int j = j0 + s;
+            acc = fma(w, fk, acc);  // targets already done add distance 0 (weight 0)
+            const double f_new = fk;
+            w = pw[ta > s ? ta - s : 0];
+            const double axs = Rhs::kForcing ? __shfl_sync(0xffffffffu, ax, j % kWarp) : ax;
             double y[D];
-            const int par = (s & 1) * 2 * D;
-            const double axs = Rhs::kForcing ? __shfl_sync(0xffffffffu, ax, s) : ax;
+            const int par = (j & 1) * 2 * D;
             if constexpr (D > 1) {
-                if (lane == s) sy[par + I] = accP;
+                if (lane == s) sy[par + I] = acc;
+            } else {
+                y[0] = __shfl_sync(0xffffffffu, acc, s);
+            }
+            const double aC = __shfl_sync(0xffffffffu, acc, kB + s);
+            if constexpr (D > 1) {
                 named_sync(1, D * kWarp);
 #pragma unroll
                 for (int q = 0; q < D; ++q) y[q] = sy[par + q];
-            } else {
-                y[0] = __shfl_sync(0xffffffffu, accP, s);
             }
+            // behind the exchange, so that its store is not queued after these
+            if (lane < c.CS) put(sf_to + (c.known + j) * D * 8, f_new);
+            if (lane == ((j - 1) & (kWarp - 1))) yo = yc, fo = f_new;
+            if (s == 0 && j % kWarp == 0 && j) flush(j - kWarp, kWarp);
             // every lane runs the step, so that f ends up in all of them
             const double fp = Rhs::template one<D>(I, y, p, axs);
-            yc = fma(ha_ig2, fp, __shfl_sync(0xffffffffu, accC, s));
+            yc = fma(ha_ig2, fp, aC);
             if constexpr (D > 1) {
-                if (lane == 0) sy[par + D + I] = yc;
+                sy[par + D + I] = yc;
                 named_sync(1, D * kWarp);
 #pragma unroll
                 for (int q = 0; q < D; ++q) y[q] = sy[par + D + q];
@@ -265,14 +289,10 @@ __device__ __forceinline__ void chain_run(const Chain &c)
             }
             fk = Rhs::template one<D>(I, y, p, axs);
         }
-        if (lane == steps - 1) yo = yc, fo = fk;
-        if (lane < steps) {
-            const int64_t m = m0 + 1 + lane;
-            Yb[m * D + I] = yo;
-            a.bt.F[m * a.bt.ldF + (int64_t)c.b * D + I] = fo;
-            if (!(finite_bits(yo) && finite_bits(fo))) report_nonfinite(a.bt.status, m, c.b);
-        }
     }
+    const int last = (steps - 1) % kWarp;
+    if (lane == last) yo = yc, fo = fk;
+    flush(steps - 1 - last, last + 1);
 }
 
 // X[b][j] = aux(t_m, p_b) for m = nT+1+j, j < n.
@@ -315,7 +335,6 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
     const Layout l = layout(D, nW, n, CS);
     const int ws = 2 * n + 2;
     double *sf = sm + l.sf, *base = sm + l.base;
-    double(*near)[2 * D][kB] = reinterpret_cast<double(*)[2 * D][kB]>(sm + l.near);
 
     // known points, unset slots, weights
     for (int j = threadIdx.x; j < 2 * n * D; j += blockDim.x) {
@@ -332,7 +351,7 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
             }
         if (threadIdx.x < 2) {
             int owned = 0;
-            for (int q = hr; q < 2 * D; q += H) ++owned;
+            for (int q = hr; q < D; q += H) ++owned;
             ptx::mbar_init(&rows_full[threadIdx.x], owned ? owned * H : 1);
             ptx::fence_mbar_init();
         }
@@ -340,18 +359,17 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
     if (rank == 0) {
         for (int j = threadIdx.x; j < nb * 2 * D * kB; j += blockDim.x)
             base[j] = __longlong_as_double((long long)kUnset);
-        for (int j = threadIdx.x; j < nW * 66; j += blockDim.x) {
-            const int q = j / 66, d = j % 66;
-            const double hq = pick<D>(a.kc.h_alpha, q);
-            sm[l.pw + q * 132 + d] = hq * a.w.B[q * a.w.stride + d];
-            sm[l.pw + q * 132 + 66 + d] = hq * a.w.A[q * a.w.stride + d];
+        for (int j = threadIdx.x; j < nW * kPw; j += blockDim.x) {
+            const int q = j / kPw, d = j % (kPw / 2);
+            const double *W = (j % kPw < kPw / 2 ? a.w.B : a.w.A) + q * a.w.stride;
+            sm[l.pw + j] = pick<D>(a.kc.h_alpha, q) * W[d];
         }
     }
     Waiter wt{a.wait > 0 ? a.wait : kWaitDefault, a.err};
     cluster_sync();
 
     if (rank == 0 && warp < D) {
-        const Chain ch{a, b, nT, Nb, nb, known, CS, sm, l, lane};
+        const Chain ch{a, b, nT, Nb, known, CS, sm, l, lane};
         if constexpr (D == 1) {
             chain_run<Rhs, D, 0>(ch);
         } else {
@@ -361,64 +379,56 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
             else chain_run<Rhs, D, D >= 4 ? 3 : 0>(ch);
         }
     } else if (rank == 0 && warp >= R::kPrev0 && warp < R::kPrev0 + R::kPrev) {
-        // ---- prev: the 32 points before each block, for kPrevComps components ----
-        const int c0 = (warp - R::kPrev0) * R::kPrevComps;
+        // ---- prev: the points of the block before each block, kPrevComps components ----
         constexpr int C = R::kPrevComps;
+        const int c0 = (warp - R::kPrev0) * C;
+        const double *pw = sm + l.pw + (lane / kB) * (kPw / 2) + kB + 1 + lane % kB;
         for (int t = 0; t < nb; ++t) {
-            double accP[C], accC[C];
+            double nxt[C];
             if (t == 0) {
 #pragma unroll
-                for (int q = 0; q < C; ++q) {
-                    accP[q] = wt.get(base + (c0 + q) * kB + lane);
-                    accC[q] = wt.get(base + (D + c0 + q) * kB + lane);
-                }
+                for (int q = 0; q < C; ++q) nxt[q] = wt.get(base + (c0 + q) * kWarp + lane);
             } else {
 #pragma unroll
-                for (int q = 0; q < C; ++q) accP[q] = accC[q] = 0.0;
+                for (int q = 0; q < C; ++q) nxt[q] = 0.0;
                 const double *f = sf + (known + (t - 1) * kB) * D + c0;
-                const double *bt = base + t * 2 * D * kB + lane;
 #pragma unroll 1
                 for (int s = 0; s < kB; ++s) {
+                    double w[C];
+#pragma unroll
+                    for (int q = 0; q < C; ++q) w[q] = pw[(nW > 1 ? (c0 + q) * kPw : 0) - s];
                     if (s == kBaseDue) {
 #pragma unroll
-                        for (int q = 0; q < C; ++q) {
-                            accP[q] += wt.get(bt + (c0 + q) * kB);
-                            accC[q] += wt.get(bt + (D + c0 + q) * kB);
-                        }
+                        for (int q = 0; q < C; ++q)
+                            nxt[q] += wt.get(base + (t * D + c0 + q) * kWarp + lane);
                     }
-                    const int d = kB + 1 + lane - s;
 #pragma unroll
-                    for (int q = 0; q < C; ++q) {
-                        const double *pb = sm + l.pw + (nW > 1 ? (c0 + q) * 132 : 0);
-                        const double fk = wt.get(f + s * D + q);
-                        accP[q] = fma(pb[d], fk, accP[q]);
-                        accC[q] = fma(pb[66 + d], fk, accC[q]);
-                    }
+                    for (int q = 0; q < C; ++q) nxt[q] = fma(w[q], wt.get(f + s * D + q), nxt[q]);
                 }
             }
 #pragma unroll
-            for (int q = 0; q < C; ++q) {
-                near[t & 1][c0 + q][lane] = accP[q];
-                near[t & 1][D + c0 + q][lane] = accC[q];
-            }
+            for (int q = 0; q < C; ++q) sm[l.near + ((t & 1) * D + c0 + q) * kWarp + lane] = nxt[q];
             named_sync(2, (D + R::kPrev) * kWarp);
         }
     } else if (hr >= 0 && warp >= hw0 && warp < hw0 + kHelpWarps) {
         // ---- helpers ----
         const int w = warp - hw0;
         const int g = hr * kHelpWarps + w, HW = H * kHelpWarps;
+        const double *wk = sm + (lane < kB ? l.wb : l.wa) + lane % kB + 1;
         for (int t = 0; t < nb; ++t) {
             const int lim = known + (t > 1 ? t - 1 : 0) * kB;  // points k0 .. k0+lim-1
-            const int off = known + t * kB + 1 + lane;          // distance of point index j: off - j
-            double acc[2 * D];
+            const double *wt0 = wk + known + t * kB;           // weight of point index j: wt0[-j]
+            double acc[D];
 #pragma unroll
-            for (int q = 0; q < 2 * D; ++q) acc[q] = 0.0;
+            for (int q = 0; q < D; ++q) acc[q] = 0.0;
             auto add = [&](int j, const double (&f)[D]) {
+                if (nW > 1) {
 #pragma unroll
-                for (int q = 0; q < D; ++q) {
-                    const int o = (nW > 1 ? q * ws : 0) + off - j;
-                    acc[q] = fma(sm[l.wb + o], f[q], acc[q]);
-                    acc[D + q] = fma(sm[l.wa + o], f[q], acc[D + q]);
+                    for (int q = 0; q < D; ++q) acc[q] = fma(wt0[q * ws - j], f[q], acc[q]);
+                } else {
+                    const double v = wt0[-j];
+#pragma unroll
+                    for (int q = 0; q < D; ++q) acc[q] = fma(v, f[q], acc[q]);
                 }
             };
             int j = g;
@@ -438,16 +448,19 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
                 add(j, f);
             }
             // the CTA's four warps, then the row's owner
-            double(*red)[2 * D][kB] =
-                reinterpret_cast<double(*)[2 * D][kB]>(sm + l.red) + (t & 1) * kHelpWarps;
+            double(*red)[D][kWarp] =
+                reinterpret_cast<double(*)[D][kWarp]>(sm + l.red) + (t & 1) * kHelpWarps;
 #pragma unroll
-            for (int q = 0; q < 2 * D; ++q) red[w][q][lane] = acc[q];
+            for (int q = 0; q < D; ++q) red[w][q][lane] = acc[q];
             named_sync(3, kHelpWarps * kWarp);
-            for (int q = w; q < 2 * D; q += kHelpWarps) {
+            if (w < D) {
+                // the slot's last rows, of block t-2, are used up once the chain has
+                // stepped on from that block's first target
+                if (t >= 2) wt.get(sf + (known + (t - 2) * kB + 1) * D);
+                const int q = w, ro = (D + H - 1) / H;
                 const double v = (red[0][q][lane] + red[1][q][lane]) + (red[2][q][lane] + red[3][q][lane]);
                 const uint32_t owner = CS > 1 ? 1 + q % H : 0;
-                const int ro = (2 * D + H - 1) / H;
-                put(mapa(smem_u32(sm + l.rows + (((t & 1) * ro + q / H) * H + hr) * kB + lane), owner), v);
+                put(mapa(smem_u32(sm + l.rows + (((t & 1) * ro + q / H) * H + hr) * kWarp + lane), owner), v);
                 __syncwarp();
                 if (lane == 0) {
                     const uint32_t bar = mapa(smem_u32(&rows_full[t & 1]), owner);
@@ -457,28 +470,23 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
                 }
             }
         }
-    } else if (hr >= 0 && warp == hw0 + kHelpWarps) {
-        // ---- finisher: rows hr, hr + H, ... (kind, component) ----
-        if (hr < 2 * D) {
-            const int ro = (2 * D + H - 1) / H;
-            for (int t = 0; t < nb; ++t) {
-                const int64_t m = nT + t * kB + 1 + lane;
-                double *bt = base + t * 2 * D * kB + lane;
-                bool waited = false;
-                for (int q = hr; q < 2 * D; q += H) {
-                    const int i = q % D, kind = q / D;
-                    const int64_t col = (int64_t)b * D + i;
-                    double far = a.G ? a.G[((int64_t)kind * n + t * kB + lane) * a.bt.cols + col] : 0.0;
-                    if (kind) far = fma(a.w.D[i * a.w.stride + m], a.bt.F[col], far);
-                    const double y0 = a.bt.y0[col];
-                    const double Tm = a.bt.y1 ? fma((double)m * a.kc.h, a.bt.y1[col], y0) : y0;
-                    if (!waited) wt.phase(&rows_full[t & 1], (t >> 1) & 1);
-                    waited = true;
-                    const double *r = sm + l.rows + (((t & 1) * ro + q / H) * H) * kB + lane;
-                    double v = 0.0;
-                    for (int h = 0; h < H; ++h) v += r[h * kB];
-                    put(mapa(smem_u32(bt + q * kB), 0), fma(pick<D>(a.kc.h_alpha, i), far + v, Tm));
-                }
+    } else if (hr >= 0 && hr < D && warp == hw0 + kHelpWarps) {
+        // ---- finisher: the rows of the components hr, hr + H, ... ----
+        const int ro = (D + H - 1) / H, kind = lane / kB, ta = lane % kB;
+        for (int t = 0; t < nb; ++t) {
+            const int64_t m = nT + t * kB + 1 + ta;
+            for (int i = hr; i < D; i += H) {
+                const int64_t col = (int64_t)b * D + i;
+                double far = a.G ? a.G[((int64_t)kind * n + t * kB + ta) * a.bt.cols + col] : 0.0;
+                if (kind) far = fma(a.w.D[i * a.w.stride + m], a.bt.F[col], far);
+                const double y0 = a.bt.y0[col];
+                const double Tm = a.bt.y1 ? fma((double)m * a.kc.h, a.bt.y1[col], y0) : y0;
+                if (i == hr) wt.phase(&rows_full[t & 1], (t >> 1) & 1);
+                const double *r = sm + l.rows + (((t & 1) * ro + i / H) * H) * kWarp + lane;
+                double v = 0.0;
+                for (int h = 0; h < H; ++h) v += r[h * kWarp];
+                put(mapa(smem_u32(base + (t * D + i) * kWarp + lane), 0),
+                    fma(pick<D>(a.kc.h_alpha, i), far + v, Tm));
             }
         }
     }

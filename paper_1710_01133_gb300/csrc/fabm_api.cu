@@ -2,7 +2,7 @@
 // the block-by-block schedule of the kernels.
 //
 // Schedule of one FP64 solve (Sec. 2 of arXiv:1710.01133), by superblocks of n
-// targets (n = 128 .. 1024, see kClusterSizes):
+// targets (n = 128 .. 512, see kClusterSizes):
 //   stream R:  wait G(T), X(T); steps of superblock T over the points k >= n(T-1)
 //   stream G:  wait R(T-2); spectrum of segment T-2; far history of T over the
 //              segments 0 .. T-2
@@ -176,9 +176,9 @@ struct fabm_solver {
     int cl_size = 0, cl_n = 0;
     std::vector<int> cl_fit = std::vector<int>(kClusterChoices, -1);
     int what_n = 0;  // superblock length the weight spectra are for
-    DevBuf<double2> tw, What, Fhat, facc;
+    DevBuf<double2> tw, What, Fhat, facc, fmid;
     DevBuf<unsigned char> fmark;
-    DevBuf<double> Gfar, Xrow;  // Xrow: forcing of two superblocks
+    DevBuf<double> Gfar, Xrow, fsegs;  // Xrow: forcing of two superblocks; fsegs: sums of f
     DevBuf<float2> auxb;       // tensor path: forcing tables of kAuxRing blocks
     DevBuf<unsigned int> err;  // split: timeout flag
     DevBuf<int64_t> nEach;
@@ -228,8 +228,8 @@ struct fabm_solver {
         wB.release(), wA.release(), wD.release(), wH.release(), wHe.release();
         wH2.release(), wHe2.release(), Fs2.release(), Fe2.release(), fpart.release(), fsum.release();
         ppart.release(), pspart.release(), psg.release(), pdone.release(), prdone.release();
-        tw.release(), What.release(), Fhat.release(), facc.release(), fmark.release(), Gfar.release(),
-            Xrow.release();
+        tw.release(), What.release(), Fhat.release(), facc.release(), fmid.release(), fmark.release(), Gfar.release(),
+            Xrow.release(), fsegs.release();
         wBl.release(), wAl.release(), wDl.release();
         wBf.release(), wAf.release(), wBff.release(), wAff.release(), wDff.release();
         F.release(), Ff.release(), Ystage.release(), G.release(), part.release();
@@ -640,13 +640,18 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
 // schedule, largest cluster first: the largest that can run for all
 // trajectories at once is taken (one CTA per SM; 152 SMs hold 7, 13, 15, 23, 28,
 // 36, 46 and 76 clusters of these sizes).  n grows with the helper warps, which
-// sum up to 2n points for each block of 32 targets while the chain runs one
-// (~24,000 cycles for three components: 255 points per helper CTA).
+// sum up to 2n points for each block of 16 targets while the chain runs one (n2:
+// up to two components, n3: more).  Measured, ms for n = 512 / 256 / 128: Lorenz-type
+// 1 x 2^15 11.3 (1024: 11.9), 12 x 2^14 5.9 / 6.1, 16 x 2^14 7.7 / 6.2 / 6.7,
+// 30 x 2^13 - / 3.5 / 3.9, 120 x 2^13 - / 9.4 / 6.5 (64: 7.1); oscillator 16 x 2^14
+// 6.5 / 6.6 / 6.9, 60 x 2^13 - / 5.9 / 3.9 (64: 4.6); LCR 256 x 2^13 - / 10.4 / 7.9
+// (64: 10.6).
 struct ClusterShape {
-    int CS, n;
+    int CS, n2, n3;
 };
-constexpr ClusterShape kClusterSizes[] = {{16, 1024}, {10, 512}, {8, 512}, {6, 512}, {5, 512},
-                                          {4, 256},   {3, 256},  {2, 128}, {1, 128}};
+constexpr ClusterShape kClusterSizes[] = {{16, 512, 512}, {10, 512, 512}, {8, 512, 256},
+                                          {6, 512, 256},  {5, 256, 256},  {4, 256, 256},
+                                          {3, 128, 128},  {2, 128, 128},  {1, 128, 128}};
 static_assert(sizeof(kClusterSizes) / sizeof(ClusterShape) == kClusterChoices);
 
 void plan_cluster(fabm_solver *s, int64_t B, int64_t cols, int64_t Nmax)
@@ -654,9 +659,10 @@ void plan_cluster(fabm_solver *s, int64_t B, int64_t cols, int64_t Nmax)
     s->cl_size = 0;
     for (int q = 0; q < kClusterChoices; ++q) {
         const ClusterShape c = kClusterSizes[q];
-        if (s->cl_fit[q] < 0) s->cl_fit[q] = cluster_max_active(s->rhs, s->dim, s->multi, c.CS, c.n);
+        const int n = s->dim > 2 ? c.n3 : c.n2;
+        if (s->cl_fit[q] < 0) s->cl_fit[q] = cluster_max_active(s->rhs, s->dim, s->multi, c.CS, n);
         if (s->cl_fit[q] < 1 || (c.CS > 1 && B > s->cl_fit[q])) continue;
-        s->cl_size = c.CS, s->cl_n = c.n;
+        s->cl_size = c.CS, s->cl_n = n;
         break;
     }
     // spectra of f: 32 bytes per point and column
@@ -671,7 +677,7 @@ fabm_status enqueue_clusters(fabm_solver *s, const DevBatch &bt, const DevWeight
     const int n = s->cl_n;
     const int64_t cols = bt.cols, nsb = (Nmax + n - 1) / n;
     const int g_max = (int)((bt.N + n - 1) / n - 1);  // as the weight spectra are laid out
-    unsigned char *mark = s->fmark.p, *big = mark + nsb * cols;
+    const FarWork fw{s->Fhat.p, s->facc.p, s->fmid.p, s->fsegs.p, s->fmark.p, s->fmark.p + nsb * cols};
     const bool forcing = rhs_has_forcing(s->rhs, bt.dim);
     s->sample_now = true;
     FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
@@ -684,12 +690,11 @@ fabm_status enqueue_clusters(fabm_solver *s, const DevBatch &bt, const DevWeight
             const double flops = 4.0 * n * (double)(n * (T - 1)) * (double)cols;
             FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG, s->evR[(T - 2) % kEvRing], 0));
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_SLICE, s->sG, 0.0, [&] {
-                return launch_fft_segment(bt, n, T - 2, s->tw.p, s->Fhat.p, mark, big, s->sG);
+                return launch_fft_segment(bt, w, n, T, s->tw.p, fw, s->sG);
             }));
-            ++s->launches;  // product and inverse
+            s->launches += 2;  // two kernels in each of the two calls
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sG, flops, [&] {
-                return launch_fft_far(bt, s->multi, n, g_max, T, s->tw.p, s->Fhat.p, s->What.p, mark,
-                                      big, s->facc.p, Gw, s->sG);
+                return launch_fft_far(bt, s->multi, n, g_max, T, s->tw.p, s->What.p, fw, Gw, s->sG);
             }));
             FABM_CUDA_TRY(cudaEventRecord(s->evG[T % 3], s->sG));
             FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evG[T % 3], 0));
@@ -776,6 +781,8 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
             const int sets = s->multi ? dim : 1;
             cudaError_t e = s->Fhat.ensure((size_t)(nsb - 2) * cols * 2 * n);
             if (e == cudaSuccess) e = s->fmark.ensure((size_t)2 * nsb * cols);
+            if (e == cudaSuccess) e = s->fmid.ensure((size_t)2 * cols);
+            if (e == cudaSuccess) e = s->fsegs.ensure((size_t)nsb * cols);
             if (e == cudaSuccess) e = s->facc.ensure((size_t)16 * cols * 2 * n);
             if (e == cudaSuccess) e = s->Gfar.ensure((size_t)2 * 2 * n * cols);
             if (e == cudaSuccess) e = s->tw.ensure((size_t)2 * n);
@@ -945,7 +952,8 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)s->fpart.p, (uintptr_t)s->fsum.p, (uintptr_t)s->near_chunks,
         (uintptr_t)s->plan_N, (uintptr_t)s->cl_size, (uintptr_t)s->cl_n, (uintptr_t)s->What.p,
         (uintptr_t)s->Fhat.p, (uintptr_t)s->facc.p, (uintptr_t)s->fmark.p, (uintptr_t)s->Gfar.p,
-        (uintptr_t)s->Xrow.p,
+        (uintptr_t)s->Xrow.p, (uintptr_t)s->fsegs.p,
+        (uintptr_t)s->fmid.p,
         (uintptr_t)(s->cl_size ? Nmax : 0)};
     auto enqueue = [&]() -> fabm_status {
         if (s->cl_size) return enqueue_clusters(s, bt, w, Nmax);

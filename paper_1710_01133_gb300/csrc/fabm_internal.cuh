@@ -256,18 +256,24 @@ cudaError_t launch_aux_rows(int rhs, const DevBatch &bt, double h, int64_t T, in
 // g_max + 1 each.
 cudaError_t launch_fft_weights(const DevWeights &w, int sets, int n, int g_max, double2 *tw,
                                double2 *What, cudaStream_t st);
-// Spectrum of the points nS .. nS+n-1 of every column: Fhat[S][col][2n]; mark,
-// big: one byte per segment and column.
-cudaError_t launch_fft_segment(const DevBatch &bt, int n, int64_t S, const double2 *tw,
-                               double2 *Fhat, unsigned char *mark, unsigned char *big,
-                               cudaStream_t st);
-// Chunks of launch_fft_far's sum over segments; acc holds chunks x cols x 2n.
+// Work space of the far history of one solve of nsb superblocks.
+struct FarWork {
+    double2 *Fhat;        // spectra of the segments, [nsb-2][cols][2n]
+    double2 *acc;         // partial spectra, [fft_chunks()][cols][2n]
+    double2 *mid;         // [2][cols]
+    double *fsum;         // sums of the segments, [nsb][cols]
+    unsigned char *mark;  // segments stored scaled down, [nsb][cols], and
+    unsigned char *big;   // whether there is one up to the segment
+};
+// Sums and spectrum of segment T-2 of every column.
+cudaError_t launch_fft_segment(const DevBatch &bt, const DevWeights &w, int n, int64_t T,
+                               const double2 *tw, const FarWork &f, cudaStream_t st);
+// Chunks of launch_fft_far's sum over segments (at most 16).
 int fft_chunks(int n, int cols, int64_t T);
-// G of superblock T >= 2 from the segments 0 .. T-2.
+// G of superblock T >= 2 from the segments 0 .. T-2, after launch_fft_segment(T).
 cudaError_t launch_fft_far(const DevBatch &bt, bool multi, int n, int g_max, int64_t T,
-                           const double2 *tw, const double2 *Fhat, const double2 *What,
-                           const unsigned char *mark, const unsigned char *big, double2 *acc,
-                           double *G, cudaStream_t st);
+                           const double2 *tw, const double2 *What, const FarWork &f, double *G,
+                           cudaStream_t st);
 
 // ---- FP64X2 precision (double-double history) ----
 

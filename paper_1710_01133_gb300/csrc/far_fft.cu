@@ -17,6 +17,17 @@
 // column's sums is relative to its own f, and a column that becomes non-finite
 // leaves the others alone.
 //
+// A transform's rounding error is relative to the largest of its sums, so what
+// is constant goes around it: w(ng+1), the middle weight of a lag's window, is
+// taken off the window's weights, and the inverse kernel adds it times the sum
+// of the segment's f (both with compensated additions).  The weights of a far
+// window differ little (1 - alpha times 2/g relative), so what is left to the
+// transforms, and their error, is a small part of the sums.  Error of whole
+// solves against binary128 (2-norm, direct sums / these): scalar 0.8, 20,000
+// steps 5.8e-16 / 5.3e-16 (8.4e-16 without the middle weights), scalar 1.5
+// 4.8e-16 / 3.4e-16 (1.1e-15), Lorenz type 0.98, 11,000 steps 5.5e-16 / 3.8e-16
+// (9.2e-16), LCR 4.0e-16 / 2.5e-16 (4.4e-16).
+//
 // In-place radix-4 transforms in shared memory, decimation in frequency
 // forward and in time backward, so the spectra stay in digit-reversed order
 // and nothing is reordered.  The weights carry the factor 1/M.
@@ -114,8 +125,9 @@ __global__ void twiddle_kernel(int M, double2 *tw)
     tw[j] = make_double2(c, -s);
 }
 
-// What[set][g] for the lags g = 2 + blockIdx.x: v[u] = w(ng+1+u), u < n, and
-// v[M-u] = w(ng+1-u), 0 < u < n, w = (B + iA) / M.  blockIdx.y: weight set.
+// What[set][g] for the lags g = 2 + blockIdx.x: v[u] = w(ng+1+u) - w(ng+1), u < n,
+// and v[M-u] = w(ng+1-u) - w(ng+1), 0 < u < n, w = (B + iA) / M.  blockIdx.y:
+// weight set.
 __global__ void __launch_bounds__(kThreads)
     weight_spectra_kernel(const double *__restrict__ WB, const double *__restrict__ WA,
                           int64_t wstride, int n, int g_max, const double2 *__restrict__ tw,
@@ -125,10 +137,10 @@ __global__ void __launch_bounds__(kThreads)
     const int M = 2 * n;
     const int64_t g = 2 + blockIdx.x;
     const double *B = WB + blockIdx.y * wstride, *A = WA + blockIdx.y * wstride;
-    const double inv = 1.0 / (double)M;
+    const double inv = 1.0 / (double)M, Bg = B[n * g + 1], Ag = A[n * g + 1];
     for (int u = threadIdx.x; u < M; u += blockDim.x) {
         const int64_t d = n * g + 1 + (u < n ? u : u - M);
-        s[u] = u == n ? make_double2(0.0, 0.0) : make_double2(B[d] * inv, A[d] * inv);
+        s[u] = u == n ? make_double2(0.0, 0.0) : make_double2((B[d] - Bg) * inv, (A[d] - Ag) * inv);
     }
     __syncthreads();
     fft_forward(s, M, tw);
@@ -138,33 +150,107 @@ __global__ void __launch_bounds__(kThreads)
 
 // A value of f above 2^900 would leave the transform no room: such a segment is
 // stored times 2^-200 and marked; big[S][col] = 1 if a segment up to S is marked.
-constexpr double kBig = 0x1p900, kDown = 0x1p-200;
+constexpr double kDown = 0x1p-200;
+constexpr int kBigHi = (1023 + 900) << 20;  // high word of 2^900
+
+// (s, c) += v, the rounding error of the addition kept in c (TwoSum).
+__device__ __forceinline__ void comp_add(double &s, double &c, double v)
+{
+    const double t = s + v, bv = t - s;
+    c += (s - (t - bv)) + (v - bv);
+    s = t;
+}
+// For superblock T, C columns per CTA (a power of two), 256 / C threads each:
+// the sum of segment T-2 of every column (fsum, mark, big), then
+// mid[kind][col] = sum over the segments S <= T-2 of w(n(T-S)+1) fsum[S], sum and
+// error term.  All lanes at work until the trees; with a warp per column inside the transforms'
+// kernels an LCR sweep of 256 x 2^13 took 9.0 instead of 8.5 ms.
+__global__ void __launch_bounds__(kThreads)
+    middle_sums_kernel(const double *__restrict__ F, int64_t ldF, int cols, int n, int64_t T,
+                       const double *__restrict__ WB, const double *__restrict__ WA,
+                       int64_t wstride, int dim, int C, double *fsum, unsigned char *mark,
+                       unsigned char *big, double2 *__restrict__ mid)
+{
+    __shared__ double2 red[2][kThreads];
+    __shared__ int over[kThreads];
+    const int c = threadIdx.x % C, r = threadIdx.x / C, R = kThreads / C;
+    const int col = blockIdx.x * C + c;
+    const bool act = col < cols;
+    const int64_t S = T - 2;
+    auto tree = [&](int kinds) {  // over the R threads of a column, in a fixed order
+        for (int off = R / 2; off > 0; off >>= 1) {
+            __syncthreads();
+            if (r < off)
+                for (int k = 0; k < kinds; ++k) {
+                    double2 x = red[k][threadIdx.x];
+                    const double2 y = red[k][threadIdx.x + off * C];
+                    comp_add(x.x, x.y, y.x);
+                    x.y += y.y;
+                    red[k][threadIdx.x] = x;
+                }
+        }
+        __syncthreads();
+    };
+    if (r == 0) over[c] = 0;
+    __syncthreads();
+    auto column_sum = [&](double sc) {  // true if a value is of at least 2^900
+        double t = 0.0, e = 0.0;
+        bool ov = false;
+        for (int j = r; act && j < n; j += R) {
+            double f = F[(S * n + j) * ldF + col];
+            ov = ov || (__double2hiint(f) & 0x7fffffff) >= kBigHi;
+            if (sc != 1.0) f *= sc;
+            comp_add(t, e, f);
+        }
+        red[0][threadIdx.x] = make_double2(t, e);
+        return ov;
+    };
+    if (column_sum(1.0)) over[c] = 1;
+    __syncthreads();
+    if (over[c]) column_sum(kDown);
+    tree(1);
+    if (r == 0 && act) {
+        fsum[S * cols + col] = red[0][c].x + red[0][c].y;
+        mark[S * cols + col] = over[c] != 0;
+        big[S * cols + col] = over[c] || (S > 0 && big[(S - 1) * cols + col]);
+    }
+    __syncthreads();
+    double t[2] = {0.0, 0.0}, e[2] = {0.0, 0.0};
+    if (act) {
+        const bool scaled = big[S * cols + col];
+        const double *W[2] = {WB + (col % dim) * wstride, WA + (col % dim) * wstride};
+        for (int64_t q = r; q <= S; q += R) {
+            double f = fsum[q * cols + col];
+            if (scaled && !mark[q * cols + col]) f *= kDown;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const double w = W[k][n * (T - q) + 1], v = w * f;
+                e[k] += fma(w, f, -v);
+                comp_add(t[k], e[k], v);
+            }
+        }
+    }
+    red[0][threadIdx.x] = make_double2(t[0], e[0]);
+    red[1][threadIdx.x] = make_double2(t[1], e[1]);
+    tree(2);
+    if (r == 0 && act) mid[col] = red[0][c], mid[cols + col] = red[1][c];
+}
 
 // Spectrum of segment S (points nS .. nS+n-1) of column blockIdx.x.
 __global__ void __launch_bounds__(kThreads)
     segment_spectrum_kernel(const double *__restrict__ F, int64_t ldF, int cols, int64_t rows, int n,
-                            int64_t S, const double2 *__restrict__ tw, double2 *__restrict__ Fhat,
-                            unsigned char *__restrict__ mark, unsigned char *__restrict__ big)
+                            int64_t S, const double2 *__restrict__ tw,
+                            const unsigned char *__restrict__ mark, double2 *__restrict__ Fhat)
 {
     extern __shared__ double2 s[];
     const int M = 2 * n, col = blockIdx.x;
-    bool over = false;
+    const double sc = mark[S * cols + col] ? kDown : 1.0;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const int64_t k = S * n + j;
-        const double f = k < rows ? F[k * ldF + col] : 0.0;
-        over = over || fabs(f) > kBig;
-        s[j] = make_double2(f, 0.0);
+        s[j] = make_double2(k < rows ? F[k * ldF + col] * sc : 0.0, 0.0);
         s[j + n] = make_double2(0.0, 0.0);
     }
-    over = __syncthreads_or(over);
-    if (over) {
-        for (int j = threadIdx.x; j < n; j += blockDim.x) s[j].x *= kDown;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        mark[S * cols + col] = over;
-        big[S * cols + col] = over || (S > 0 && big[(S - 1) * cols + col]);
-    }
+    __syncthreads();
     fft_forward(s, M, tw);
     double2 *out = Fhat + (S * cols + col) * M;
     for (int u = threadIdx.x; u < M; u += blockDim.x) out[u] = s[u];
@@ -202,11 +288,12 @@ __global__ void product_kernel(const double2 *__restrict__ Fhat, const double2 *
     acc[(blockIdx.y * (int64_t)cols + col) * M + u] = r;
 }
 
-// G[kind][a][col], a < n: the sums of the chunks in order, transformed back.
+// G[kind][a][col], a < n: the sums of the chunks in order, transformed back,
+// plus the middle weights times the segments' sums (mid).
 __global__ void __launch_bounds__(kThreads)
-    inverse_kernel(const double2 *__restrict__ acc, const unsigned char *__restrict__ big, int chunks,
-                   int cols, int n, int64_t T, const double2 *__restrict__ tw,
-                   double *__restrict__ G)
+    inverse_kernel(const double2 *__restrict__ acc, const double2 *__restrict__ mid,
+                   const unsigned char *__restrict__ big, int chunks, int cols, int n, int64_t T,
+                   const double2 *__restrict__ tw, double *__restrict__ G)
 {
     extern __shared__ double2 s[];
     const int M = 2 * n, col = blockIdx.x;
@@ -218,9 +305,10 @@ __global__ void __launch_bounds__(kThreads)
     __syncthreads();
     fft_backward(s, M, tw);
     const double up = big[(T - 2) * cols + col] ? 1.0 / kDown : 1.0;
+    const double2 mP = mid[col], mC = mid[cols + col];
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        G[(int64_t)j * cols + col] = s[j].x * up;
-        G[(int64_t)(n + j) * cols + col] = s[j].y * up;
+        G[(int64_t)j * cols + col] = (mP.x + (mP.y + s[j].x)) * up;
+        G[(int64_t)(n + j) * cols + col] = (mC.x + (mC.y + s[j].y)) * up;
     }
 }
 
@@ -239,16 +327,6 @@ cudaError_t launch_fft_weights(const DevWeights &w, int sets, int n, int g_max, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_fft_segment(const DevBatch &bt, int n, int64_t S, const double2 *tw,
-                               double2 *Fhat, unsigned char *mark, unsigned char *big,
-                               cudaStream_t st)
-{
-    const int M = 2 * n;
-    segment_spectrum_kernel<<<(unsigned)bt.cols, fft_threads(M), sizeof(double2) * M, st>>>(
-        bt.F, bt.ldF, bt.cols, bt.N + 1, n, S, tw, Fhat, mark, big);
-    return cudaGetLastError();
-}
-
 int fft_chunks(int n, int cols, int64_t T)
 {
     // enough CTAs of 128 threads to fill the FP64 units (four warps per SM
@@ -259,16 +337,28 @@ int fft_chunks(int n, int cols, int64_t T)
     return (int)(c < 1 ? 1 : (c > 16 ? 16 : c));
 }
 
+cudaError_t launch_fft_segment(const DevBatch &bt, const DevWeights &w, int n, int64_t T,
+                               const double2 *tw, const FarWork &f, cudaStream_t st)
+{
+    const int M = 2 * n;
+    int C = 1;
+    while (C < 8 && C < bt.cols) C *= 2;
+    middle_sums_kernel<<<(unsigned)((bt.cols + C - 1) / C), kThreads, 0, st>>>(
+        bt.F, bt.ldF, bt.cols, n, T, w.B, w.A, w.stride, bt.dim, C, f.fsum, f.mark, f.big, f.mid);
+    segment_spectrum_kernel<<<(unsigned)bt.cols, fft_threads(M), sizeof(double2) * M, st>>>(
+        bt.F, bt.ldF, bt.cols, bt.N + 1, n, T - 2, tw, f.mark, f.Fhat);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_fft_far(const DevBatch &bt, bool multi, int n, int g_max, int64_t T,
-                           const double2 *tw, const double2 *Fhat, const double2 *What,
-                           const unsigned char *mark, const unsigned char *big, double2 *acc,
-                           double *G, cudaStream_t st)
+                           const double2 *tw, const double2 *What, const FarWork &f, double *G,
+                           cudaStream_t st)
 {
     const int M = 2 * n, chunks = fft_chunks(n, bt.cols, T);
     product_kernel<<<dim3((unsigned)(M / 128), (unsigned)chunks, (unsigned)bt.cols), 128, 0, st>>>(
-        Fhat, What, mark, big, bt.cols, bt.dim, multi, M, g_max, T, acc);
+        f.Fhat, What, f.mark, f.big, bt.cols, bt.dim, multi, M, g_max, T, f.acc);
     inverse_kernel<<<(unsigned)bt.cols, fft_threads(M), sizeof(double2) * M, st>>>(
-        acc, big, chunks, bt.cols, n, T, tw, G);
+        f.acc, f.mid, f.big, chunks, bt.cols, n, T, tw, G);
     return cudaGetLastError();
 }
 

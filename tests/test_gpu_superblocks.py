@@ -24,7 +24,7 @@ def rel_err(got, ref):
     return float(np.max(np.abs(np.asarray(got) - ref) / scale))
 
 
-@pytest.mark.parametrize("N", [1023, 1024, 1025, 2047, 2049, 3072, 3073, 4127])
+@pytest.mark.parametrize("N", [511, 512, 513, 1024, 1025, 1536, 1537, 2063])
 def test_superblock_edges_scalar(gpu_lib, parity, N):
     w = ml_scalar(N)
     with gpu_lib.Solver(w.rhs, w.dim, w.alpha, w.h, w.N, w.params) as s:
