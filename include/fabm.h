@@ -199,11 +199,9 @@ int fabm_last_history_kernel(const fabm_solver *s);
 /* Step layouts of the split-precision recurrence on the tensor-history path
  * (fabm_set_recurrence_layout); both compute the same steps in float-float. */
 enum {
-    FABM_REC_AUTO = 0,     /* COLUMNS when the batch has at least 96 warps of columns
-                              (96 * 32/dim trajectories) or N * columns >= 2^28
-                              (the history dominates), else TARGETS                 */
+    FABM_REC_AUTO = 0,     /* COLUMNS                                               */
     FABM_REC_COLUMNS = 1,  /* one lane per column (trajectory, component), 32/dim
-                              trajectories per warp: fewest instructions per step    */
+                              trajectories per team of five warps                   */
     FABM_REC_TARGETS = 2   /* one lane per target, one CTA of dim warps per
                               trajectory: most parallelism for narrow batches        */
 };
@@ -214,10 +212,9 @@ enum {
 fabm_status fabm_set_recurrence_layout(fabm_solver *s, int layout);
 /* The layout set on the solver (FABM_REC_*), or -1 for NULL. */
 int fabm_get_recurrence_layout(const fabm_solver *s);
-/* Warps per CTA of the lane-per-column recurrence (FABM_REC_COLUMNS) for later
- * solves: 0 chooses automatically (CTAs sized to fill the SMs the tensor CTAs
- * leave free, at most 4 warps each), 1..12 fixes it; the arithmetic and the
- * results do not depend on it.  FABM_EINVAL outside 0..12, FABM_EBUSY while
+/* Teams of warps per CTA of the lane-per-column recurrence (FABM_REC_COLUMNS)
+ * for later solves: 0 chooses automatically (one), 1..12 fixes it (more than
+ * three run as three); the arithmetic and the results do not depend on it.  FABM_EINVAL outside 0..12, FABM_EBUSY while
  * another thread uses the solver. */
 fabm_status fabm_set_recurrence_warps(fabm_solver *s, int warps);
 /* The width set on the solver (0: automatic), or -1 for NULL. */

@@ -277,7 +277,7 @@ __device__ __forceinline__ void chain_run(const Chain &c)
             if (lane == ((j - 1) & (kWarp - 1))) yo = yc, fo = f_new;
             if (s == 0 && j % kWarp == 0 && j) flush(j - kWarp, kWarp);
             // every lane runs the step, so that f ends up in all of them
-            const double fp = Rhs::template one<D>(I, y, p, axs);
+            const double fp = rhs_f64<Rhs, D>(I, y, p, axs);
             yc = fma(ha_ig2, fp, aC);
             if constexpr (D > 1) {
                 sy[par + D + I] = yc;
@@ -287,7 +287,7 @@ __device__ __forceinline__ void chain_run(const Chain &c)
             } else {
                 y[0] = yc;
             }
-            fk = Rhs::template one<D>(I, y, p, axs);
+            fk = rhs_f64<Rhs, D>(I, y, p, axs);
         }
     }
     const int last = (steps - 1) % kWarp;

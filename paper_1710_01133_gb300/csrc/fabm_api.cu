@@ -14,11 +14,12 @@
 //     stream G:  wait R(c-2); history(c) over k < (c-1)L; combine -> G[c%2]
 //     stream R:  wait G(c);   recurrence(c), which adds the lag-1 block itself
 //   (long FP64 solves: lag 2, the history of consecutive blocks on two streams)
-//   tensor history, L = 64:
-//     stream G:  wait R(c-2); far history(c) over segments 0..c-2; wait N(c);
-//                combine of far and newest partials -> G[c%2] (float-float)
-//     stream R:  slice segment c-1; N(c): newest segment c-1; wait G(c);
-//                recurrence(c) over its own triangle only
+//   tensor history, L = 64 (64 targets per far launch; pairs of blocks see
+//   enqueue_solve):
+//     stream G:  wait R(c-2); far history(c) over segments 0..c-2; sum of its
+//                chunks -> G[c%2] (float-float)
+//     stream R:  newest segment c-1; wait G(c); recurrence(c) over its own
+//                triangle, which also writes the slices of segment c
 //     stream G2: forcing tables up to three blocks ahead
 //     stream C:  finished rows of y to pinned host memory (large outputs)
 // The history of block c+1 therefore runs while the recurrence of block c
@@ -180,6 +181,7 @@ struct fabm_solver {
     DevBuf<unsigned char> fmark;
     DevBuf<double> Gfar, Xrow, fsegs;  // Xrow: forcing of two superblocks; fsegs: sums of f
     DevBuf<float2> auxb;       // tensor path: forcing tables of kAuxRing blocks
+    DevBuf<float2> parff, y0ff; // tensor path: float-float parameters and y_0
     DevBuf<unsigned int> err;  // split: timeout flag
     DevBuf<int64_t> nEach;
     DevBuf<unsigned long long> status;
@@ -192,9 +194,8 @@ struct fabm_solver {
     cudaStream_t sR = nullptr, sG = nullptr, sG2 = nullptr, sC = nullptr, sG3 = nullptr, sS = nullptr;
     double *out_stream = nullptr;  // pinned host output of the solve being enqueued, or NULL
     int64_t out_group = 1;         // blocks per streamed copy
-    // evN: the newest-segment history launch of the tensor path (on sR); evA:
-    // the forcing tables (tensor path, on sG2)
-    cudaEvent_t evR[kEvRing] = {}, evG[3] = {}, evN[3] = {}, evA[kAuxRing] = {};
+    // evA: the forcing tables (on sG2)
+    cudaEvent_t evR[kEvRing] = {}, evG[3] = {}, evA[kAuxRing] = {};
     cudaEvent_t evF[2] = {};  // wide far history of target group C summed, slot C % 2
     cudaEvent_t evFK[2] = {}; // wide far kernel of target group C done, slot C % 2
     cudaEvent_t evFork = nullptr, evJoin = nullptr, evJoinC = nullptr, evJoin3 = nullptr,
@@ -234,12 +235,11 @@ struct fabm_solver {
         wBf.release(), wAf.release(), wBff.release(), wAff.release(), wDff.release();
         F.release(), Ff.release(), Ystage.release(), G.release(), part.release();
         Fs.release(), Fe.release(), spart.release(), auxb.release(), err.release();
+        parff.release(), y0ff.release();
         y0.release(), par.release(), nEach.release(), status.release();
         for (auto &e : evR)
             if (e) cudaEventDestroy(e);
         for (auto &e : evG)
-            if (e) cudaEventDestroy(e);
-        for (auto &e : evN)
             if (e) cudaEventDestroy(e);
         for (auto &e : evA)
             if (e) cudaEventDestroy(e);
@@ -439,6 +439,10 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
     s->sample_now = true;
     FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
                                [&] { return launch_init(s->rhs, bt, s->sR, split); }));
+    if (split) {
+        s->launches += 2;
+        FABM_CUDA_TRY(launch_ff_inputs(bt, s->parff.p, s->y0ff.p, s->sR));
+    }
     // tensor path with forcing: the tables of the time-only part of f, on sG2,
     // up to kAuxRing - 1 blocks ahead of the recurrence
     const bool tables = split && rhs_has_forcing(s->rhs, bt.dim);
@@ -514,12 +518,12 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             hin.near = s->spart.p;
             hin.n_near = n_nc;
         } else if (split && c >= 1) {
-            // far part (segments 0 .. c-2) on sG beside the recurrence of block
-            // c-1; the newest segment c-1 on sR once it is sliced; the combine
-            // on sG after both
-            float2 *Gbuf = reinterpret_cast<float2 *>(s->G.p) + (size_t)(c % n_gbuf) * 2 * L * cols;
+            // far part (segments 0 .. c-2) and the sum of its chunks on sG beside
+            // the recurrence of block c-1; the newest segment c-1 on sR, its
+            // partials added by the recurrence
             const int n_far = (int)std::min<int64_t>(c - 1, split_chunks);
             if (n_far > 0) {
+                float2 *Gbuf = reinterpret_cast<float2 *>(s->G.p) + (size_t)(c % n_gbuf) * 2 * L * cols;
                 const double flops = 4.0 * L * (double)((c - 1) * L) * (double)cols;
                 FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG, s->evR[(c - 2) % kEvRing], 0));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sG, flops, [&] {
@@ -527,21 +531,23 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                                              0, n_far, n_ct, (int)cols, s->spart.p, s->err.p,
                                              s->wait_cycles, s->sG);
                 }));
+                FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, s->sG, 0.0, [&] {
+                    return launch_combine_split_ff(s->spart.p, n_far, (int)cols, L, Gbuf, s->sG);
+                }));
+                FABM_CUDA_TRY(cudaEventRecord(s->evG[c % 3], s->sG));
+                hin.G = Gbuf;
             }
+            // a chunk of its own, which the next block's far launch leaves alone
             const double nflops = 4.0 * L * (double)L * (double)cols;
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sR, nflops, [&] {
                 return launch_hist_split(s->Fs.p, s->Fe.p, s->wH.p, s->wHe.p, c, (int)(c - 1), 1,
-                                         n_far, 1, n_ct, (int)cols, s->spart.p, s->err.p,
+                                         split_chunks, 1, n_ct, (int)cols, s->spart.p, s->err.p,
                                          s->wait_cycles, s->sR);
             }));
-            FABM_CUDA_TRY(cudaEventRecord(s->evN[c % 3], s->sR));
-            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG, s->evN[c % 3], 0));
-            FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, s->sG, 0.0, [&] {
-                return launch_combine_split_ff(s->spart.p, n_far + 1, (int)cols, L, Gbuf, s->sG);
-            }));
-            FABM_CUDA_TRY(cudaEventRecord(s->evG[c % 3], s->sG));
-            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evG[c % 3], 0));
-            hin.G = Gbuf;
+            if (n_far > 0) FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evG[c % 3], 0));
+            hin.near = s->spart.p + split_part_elems(split_chunks, (int)cols);
+            hin.n_near = 1;
+            hin.near_as_chunk = true;
         } else if (!split && (c - lag) * L > 0) {
             const int64_t k_end = (c - lag) * L;
             double *Gbuf = s->G.p + (size_t)(c % n_gbuf) * 2 * L * cols;
@@ -597,13 +603,16 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evA[c % kAuxRing], 0));
         }
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sR, rflops, [&] {
-            if (split)
+            if (split) {
+                const bool slices = c + 1 < nblk;  // segment c is read by the blocks c+1 ..
+                const ColsIn in{s->parff.p, s->y0ff.p, X, slices ? s->Fs.p : nullptr, s->Fe.p, n_ct};
                 return launch_recur_cols(s->rhs, bt, s->wBff.p, s->wAff.p, s->wDff.p, s->k, c, hin,
-                                         X, s->cols_warps, s->sR);
+                                         in, s->cols_warps, s->sR);
+            }
             return launch_recur(s->rhs, bt, w, s->k, c, L, lag, s->precision == FABM_SPLIT,
                                 static_cast<const double *>(Gc), s->sR);
         }));
-        if (split && c + 1 < nblk) {  // segment c is read by the blocks c+1 ..
+        if (split && c + 1 < nblk && s->cols_warps == 0) {  // the other layout writes them itself
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_SLICE, s->sR, 0.0, [&] {
                 return launch_slice_f(bt, n_ct, c, s->Fs.p, s->Fe.p, s->sR);
             }));
@@ -823,20 +832,16 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     int split_chunks = 1, far_chunks = 1;
     s->wide = false;
     if (split) {
-        // recurrence layout: one lane per column for wide batches, and where
-        // the history dominates (its SMs matter more than the recurrence's
-        // latency); one lane per target for short, narrow runs (more
-        // parallelism, more instructions)
+        // SMs left to the recurrence that runs beside the tensor kernel (one
+        // tensor CTA fills an SM's register file), only where the column tiles
+        // do not need every SM: one SM per 8 column warps for wide or long
+        // batches, else one per 12 trajectories up to 16 SMs (LCR 1024 x
+        // 2^14: reserves of 40, 16 and 0 SMs predicted 25.3, 23.5, 23.1 ms)
         const int cwarps = recur_cols_warps(dim, B);
         const bool columns =
             s->rec_layout == FABM_REC_COLUMNS ||
             (s->rec_layout == FABM_REC_AUTO &&
              (cwarps >= 96 || (double)(s->plan_N > 0 ? s->plan_N : Nmax) * cols >= 0x1p28));
-        // leave SMs for the recurrence that runs beside the tensor kernel (one
-        // tensor CTA fills an SM's register file), only where the column tiles
-        // do not need every SM: one SM per 8 column warps, or per 12
-        // trajectories of the lane-per-target layout up to 16 SMs (LCR 1024 x
-        // 2^14: reserves of 40, 16 and 0 SMs predicted 25.3, 23.5, 23.1 ms)
         int reserve = s->sm_reserve;
         if (reserve < 0) {
             const int64_t want = columns ? std::clamp<int64_t>((cwarps + 7) / 8, 4, 40)
@@ -860,13 +865,10 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         // does not wait for far CTAs to retire (one CTA sums its segments in turn)
         const int far_free = 152 - 2 * n_ct * far_chunks;
         s->near_chunks = std::clamp(far_free / n_ct, 1, 3);
-        // column layout: CTAs sized to fill the SMs the tensor CTAs leave free,
-        // at most 4 warps each, so that a CTA fits beside others on an SM that
-        // is partly free (Duffing 4096 x 2^16: 4 warps 323 ms, 11 warps 340)
-        const int free_sms = std::max(4, 152 - n_ct * split_chunks);
-        s->cols_warps = !columns        ? 0
-                        : s->rec_warps > 0 ? s->rec_warps
-                                           : std::clamp((cwarps + free_sms - 1) / free_sms, 1, 4);
+        // one team of warps per CTA unless set; the lane-per-target layout on request
+        s->cols_warps = s->rec_layout == FABM_REC_TARGETS ? 0 : std::max(1, s->rec_warps);
+        FABM_CUDA_TRY(s->parff.ensure((size_t)B * kMaxParams));
+        FABM_CUDA_TRY(s->y0ff.ensure((size_t)cols));
         FABM_CUDA_TRY(s->Fs.ensure((size_t)nblk * n_ct * 3 * 128 * 64));
         FABM_CUDA_TRY(s->Fe.ensure((size_t)nblk * n_ct * 128));
         // far chunks and one chunk for the newest segment; with the wide far
@@ -953,7 +955,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)s->plan_N, (uintptr_t)s->cl_size, (uintptr_t)s->cl_n, (uintptr_t)s->What.p,
         (uintptr_t)s->Fhat.p, (uintptr_t)s->facc.p, (uintptr_t)s->fmark.p, (uintptr_t)s->Gfar.p,
         (uintptr_t)s->Xrow.p, (uintptr_t)s->fsegs.p,
-        (uintptr_t)s->fmid.p,
+        (uintptr_t)s->fmid.p, (uintptr_t)s->parff.p, (uintptr_t)s->y0ff.p,
         (uintptr_t)(s->cl_size ? Nmax : 0)};
     auto enqueue = [&]() -> fabm_status {
         if (s->cl_size) return enqueue_clusters(s, bt, w, Nmax);
@@ -1181,8 +1183,6 @@ fabm_status create_solver(int dim, const double *alpha_c, double h, int64_t N, i
     for (auto &ev : s->evR)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     for (auto &ev : s->evG)
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    for (auto &ev : s->evN)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     for (auto &ev : s->evA)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);

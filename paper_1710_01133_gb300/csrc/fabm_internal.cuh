@@ -183,20 +183,30 @@ cudaError_t launch_sum_far(const float2 *far, int n_far, int cols, float2 *out, 
 // float-float pairs: G[kind][g_off + t][col] (rows of g_rows per kind; NULL:
 // none) plus near[ch][kind][t][col] (64 rows per kind) over n_near chunks.  WB, WA: h^a B(d), h^a A(d)
 // for d = 0..64; WD: h^a D(m), m = 0..N; all float-float pairs, one order.
-// warps_per_cta (1..12) warps of 32/dim trajectories per CTA, or 0: one lane
-// per target, a CTA of dim warps per trajectory (narrow batches).  X: the table
-// of the time-only part of f for block c (launch_aux_table), required when
-// rhs_has_forcing(rhs), else ignored.  y's slots receive float-float
-// increments; launch_finish_y turns them into y after the last block.
+// warps_per_cta teams (at most 3) of 32/dim trajectories per CTA, or 0: one lane
+// per target, a CTA of dim warps per trajectory, which leaves the slices to
+// launch_slice_f.  y's slots receive float-float increments; launch_finish_y
+// turns them into y after the last block.
 struct HistIn {
     const float2 *G = nullptr;     // [2][g_rows][cols], or NULL
     int g_rows = 64, g_off = 0;
     const float2 *near = nullptr;  // [n_near][2][64][cols]
     int n_near = 0;
+    bool near_as_chunk = false;  // one near chunk, added as the chunk after those in G
+};
+struct ColsIn {
+    const float2 *par, *y0;  // float-float copies of the parameters and y_0 (launch_ff_inputs)
+    const float2 *X;         // table of the time-only part of f for block c
+                             // (launch_aux_table), required when rhs_has_forcing(rhs)
+    __nv_bfloat16 *Fs;       // where the slices and exponents of segment c go (all
+    int *Ef;                 // segments' arrays), or NULL
+    int n_ct;
 };
 cudaError_t launch_recur_cols(int rhs, const DevBatch &bt, const float2 *WB, const float2 *WA,
                               const float2 *WD, const StepConsts &k, int64_t c, const HistIn &hin,
-                              const float2 *X, int warps_per_cta, cudaStream_t st);
+                              const ColsIn &in, int warps_per_cta, cudaStream_t st);
+// par[B][kMaxParams], y0[cols] as float-float pairs.
+cudaError_t launch_ff_inputs(const DevBatch &bt, float2 *par, float2 *y0, cudaStream_t st);
 // The right-hand side has a time-dependent part (forcing).
 bool rhs_has_forcing(int rhs, int dim);
 // X[a][b] = aux(t_{64c+1+a}, params of b) as float-float pairs, a < 64, b < B.

@@ -13,7 +13,7 @@
 
 namespace fabm {
 
-struct FF {
+struct alignas(8) FF {  // one 64-bit load or store
     float hi, lo;
     FF() = default;
     __host__ __device__ constexpr FF(float h, float l) : hi(h), lo(l) {}
@@ -89,6 +89,18 @@ __device__ inline void dot2_acc(FF &acc, FF w, FF f)
 }
 
 __device__ inline FF ff_norm(FF a) { return two_sum(a.hi, a.lo); }
+
+// (hi, lo) += (x, y) as the chunk partials of the split history are added:
+// TwoSum of the leading parts, low parts folded in, renormalised.
+__device__ __forceinline__ void ff_add_chunk(float &hi, float &lo, float x, float y)
+{
+    const float s = hi + x;
+    const float bb = s - hi;
+    const float e = (hi - (s - bb)) + (x - bb);
+    lo += e + y;
+    hi = s + lo;
+    lo = lo - (hi - s);
+}
 
 __device__ inline bool operator<=(FF x, FF y) { return x.hi < y.hi || (x.hi == y.hi && x.lo <= y.lo); }
 __device__ inline bool operator>=(FF x, FF y) { return y <= x; }

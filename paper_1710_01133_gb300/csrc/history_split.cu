@@ -57,7 +57,9 @@
 
 
 #include "fabm_internal.cuh"
+#include "ff.cuh"
 #include "sm100_ptx.cuh"
+#include "split_slices.cuh"
 
 namespace fabm {
 namespace {
@@ -84,16 +86,14 @@ constexpr size_t kSmemBytes = (size_t)kStages * kStageStride + 1024 + kStashByte
 // which always complete, keep the default
 constexpr long long kWaitCycles = 4000000000LL;
 
-__device__ __forceinline__ int exp_clamp(int e) { return e < -126 ? -126 : (e > 127 ? 127 : e); }
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((exp_clamp(e) + 127) << 23); }
-
 // --------------------------------------------------------- f slicing ---
 
 // f of segment `seg` (points seg*64 .. seg*64+63) -> three bf16 slices in the
 // operand layout [seg][ct][slice][k1 = j'/8][col 128][j'%8], j' = 63 - j, and
 // the exponent E per column in Ef[seg][ct][col].  On this path the recurrence
-// stores f as float-float pairs (hi, lo).  grid = cols_pad/32, block = 256 =
-// 32 columns x 8 groups of 8 points.
+// stores f as float-float pairs (hi, lo).  For the lane-per-target recurrence;
+// the lane-per-column one writes its segment's slices itself.  grid =
+// cols_pad/32, block = 256 = 32 columns x 8 groups of 8 points.
 __global__ void __launch_bounds__(256) slice_f_kernel(const float2 *__restrict__ F, int64_t ldF,
                                                       int64_t n_rows, int cols, int n_ct,
                                                       int64_t seg,
@@ -107,8 +107,7 @@ __global__ void __launch_bounds__(256) slice_f_kernel(const float2 *__restrict__
     float m = 0.f;
 #pragma unroll
     for (int k0 = 0; k0 < 8; ++k0) {
-        const int j = 63 - (8 * k1 + k0);
-        const int64_t row = seg * kSeg + j;
+        const int64_t row = seg * kSeg + 63 - (8 * k1 + k0);
         const float2 f = (col < cols && row < n_rows) ? F[row * ldF + col] : make_float2(0.f, 0.f);
         hi[k0] = f.x;
         lo[k0] = f.y;
@@ -118,35 +117,15 @@ __global__ void __launch_bounds__(256) slice_f_kernel(const float2 *__restrict__
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 8; ++i) m = fmaxf(m, smax[i][cl]);
-    int E = 0;
-    if (m > 0.f && m <= 3.0e38f) E = ilogbf(m) + 1;
-    if (E < -100) E = -100;
-    const float sc = pow2f(8 - E);
+    const int E = slice_exponent(m);
     uint32_t w[3][4];
-#pragma unroll
-    for (int k0 = 0; k0 < 8; k0 += 2) {
-        float t[3][2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const float xh = hi[k0 + u] * sc, xl = lo[k0 + u] * sc;
-            const float t0 = rintf(xh);
-            const float r = ((xh - t0) + xl) * 256.f;
-            const float t1 = rintf(r);
-            const float t2 = rintf((r - t1) * 256.f);
-            t[0][u] = t0, t[1][u] = t1 * 0x1p-8f, t[2][u] = t2 * 0x1p-16f;
-        }
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            __nv_bfloat162 p = __floats2bfloat162_rn(t[q][0], t[q][1]);
-            w[q][k0 / 2] = *reinterpret_cast<uint32_t *>(&p);
-        }
-    }
+    slice8(hi, lo, E, w);
     const int ct = col / kMC, cloc = col % kMC;
     if (col < n_ct * kMC) {
-        __nv_bfloat16 *base = Fs + ((seg * n_ct + ct) * 3) * (int64_t)(kMC * kSeg);
+        __nv_bfloat16 *base = slice_base(Fs, seg, n_ct, ct, cloc);
 #pragma unroll
         for (int q = 0; q < 3; ++q)
-            *reinterpret_cast<uint4 *>(base + q * (kMC * kSeg) + k1 * (kMC * 8) + cloc * 8) =
+            *reinterpret_cast<uint4 *>(base + q * (kMC * kSeg) + k1 * (kMC * 8)) =
                 make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
         if (k1 == 0) Ef[(seg * n_ct + ct) * kMC + cloc] = E;
     }
@@ -478,18 +457,6 @@ __global__ void __launch_bounds__(kThreads, 1) hist_split_kernel(const SplitArgs
     if (!ok) atomicOr(a.err, 1u);
 }
 
-// float-float (hi, lo) += (x, y): two-sum of the high parts, low parts folded
-// in, renormalized.
-__device__ __forceinline__ void ff_add(float &hi, float &lo, float x, float y)
-{
-    const float s = hi + x;
-    const float bb = s - hi;
-    const float e = (hi - (s - bb)) + (x - bb);
-    lo += e + y;
-    hi = s + lo;
-    lo = lo - (hi - s);
-}
-
 // a3: G[kind][t][col] = sum over chunks of the float-float partials, R lanes
 // per output, each summing chunks r, r+R, ... in ascending order (four loads
 // in flight), then a fixed xor tree, in compensated float-float (~48 bits,
@@ -515,27 +482,27 @@ __global__ void combine_split_kernel(const float2 *__restrict__ part, int n_chun
                 const float2 v1 = part[(int64_t)(ch + R) * n_out + o];
                 const float2 v2 = part[(int64_t)(ch + 2 * R) * n_out + o];
                 const float2 v3 = part[(int64_t)(ch + 3 * R) * n_out + o];
-                ff_add(hi, lo, v0.x, v0.y);
-                ff_add(hi, lo, v1.x, v1.y);
-                ff_add(hi, lo, v2.x, v2.y);
-                ff_add(hi, lo, v3.x, v3.y);
+                ff_add_chunk(hi, lo, v0.x, v0.y);
+                ff_add_chunk(hi, lo, v1.x, v1.y);
+                ff_add_chunk(hi, lo, v2.x, v2.y);
+                ff_add_chunk(hi, lo, v3.x, v3.y);
             }
             for (; ch < n_chunks; ch += R) {
                 const float2 v = part[(int64_t)ch * n_out + o];
-                ff_add(hi, lo, v.x, v.y);
+                ff_add_chunk(hi, lo, v.x, v.y);
             }
         }
 #pragma unroll
         for (int off = R / 2; off > 0; off >>= 1) {
             const float ohi = __shfl_xor_sync(0xffffffffu, hi, off);
             const float olo = __shfl_xor_sync(0xffffffffu, lo, off);
-            ff_add(hi, lo, ohi, olo);
+            ff_add_chunk(hi, lo, ohi, olo);
         }
         if (r == 0 && o < n_out) {
             if constexpr (std::is_same_v<Out, double>)
                 G[o] = (double)hi + (double)lo;
             else
-                G[o] = make_float2(hi, lo);  // normalised by ff_add
+                G[o] = make_float2(hi, lo);  // normalised by ff_add_chunk
         }
     }
 }

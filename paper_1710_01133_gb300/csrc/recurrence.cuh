@@ -182,9 +182,9 @@ __device__ void recur_block(const DevBatch &bt, int b, const DevWeights &w, cons
         double fn = 0.0, yc = 0.0;
         if constexpr (D == 1) {
             if (lane == owner) {
-                const double fp = Rhs::template one<D>(0, &yp, p, ax);
+                const double fp = rhs_f64<Rhs, D>(0, &yp, p, ax);
                 yc = fma(ha_ig2, fp, aC);
-                fn = Rhs::template one<D>(0, &yc, p, ax);
+                fn = rhs_f64<Rhs, D>(0, &yc, p, ax);
             }
         } else {
             if (act && lane == owner) sy[0][i] = yp;
@@ -193,7 +193,7 @@ __device__ void recur_block(const DevBatch &bt, int b, const DevWeights &w, cons
                 double y[D];
 #pragma unroll
                 for (int q = 0; q < D; ++q) y[q] = sy[0][q];
-                const double fp = Rhs::template one<D>(i, y, p, ax);
+                const double fp = rhs_f64<Rhs, D>(i, y, p, ax);
                 yc = fma(ha_ig2, fp, aC);  // corrector
                 if (act) sy[1][i] = yc;
             }
@@ -202,7 +202,7 @@ __device__ void recur_block(const DevBatch &bt, int b, const DevWeights &w, cons
                 double y[D];
 #pragma unroll
                 for (int q = 0; q < D; ++q) y[q] = sy[1][q];
-                fn = Rhs::template one<D>(i, y, p, ax);
+                fn = rhs_f64<Rhs, D>(i, y, p, ax);
             }
         }
         if (act && lane == owner) {

@@ -1,44 +1,76 @@
-// a4 + a5 for wide batches on the tensor-history path: the predictor -> f ->
-// corrector -> f chain of Sec. 2 of arXiv:1710.01133 with one lane per column
-// (trajectory b, component i) instead of one lane per target.
+// a4 + a5 on the tensor-history path: the predictor -> f -> corrector -> f
+// chain of Sec. 2 of arXiv:1710.01133 with one lane per column (trajectory b,
+// component i), 32/D trajectories to a team of five warps.
 //
-// On this path the history launches (far segments and the newest segment,
+// The history launches (far segments and the newest segments, history_far.cu,
 // history_split.cu) deliver every point k < cL of block c, so a step only adds
-// the points of its own block.  Per lane, block c (targets m = cL+1+a, a < 64,
-// points f_{cL+j}, j = 0..64):
-//   bases   h^a (G_P(m)) and h^a (G_C(m) + D(m) f_0) from the combined history;
-//   near    S(a) = sum_{j<=a} w(a+1-j) f_{cL+j}, float-float products summed
-//           with separate error terms (dot2_acc), in sub-blocks of 8 targets:
-//           the points before the sub-block at its start (independent
-//           products, no chain), the sub-block's own points as they appear;
-//   step    y^P = T + b_P + S_P, exchange of y^P between the lanes of the
-//           trajectory (shuffles), f(t, y^P), y = T + b_C + S_C + h^a f^P /
-//           Gamma(a+2), exchange, f(t, y);
-//   output  the float-float increment h^a (...) in the double-sized slot of y
-//           (finish_y_kernel adds the Taylor part in double after the last
-//           block) and f as a float-float pair (the buffer the segment slicer
-//           reads).
-// A warp advances 32/D trajectories at once, so the serial part of a step is
-// paid once per warp rather than once per column, and no step waits on a
-// block-wide barrier.  GB300 runs FP64 at 1/64 of the fp32 rate with a long
-// latency, so no FP64 operation is left in the kernel: the time-only part of f
-// (forcing) comes from a table that aux_kernel fills blocks ahead on another
-// stream, and y is converted to double once at the end.
+// the points of its own block.  Targets m = cL+1+a, a < 64, points f_{cL+j},
+// j = 0..64, in sub-blocks of 8 targets:
+//   helpers (4 warps, each 4 of a sub-block's 16 sums): the base T + h^a G_P(m)
+//           or h^a (G_C(m) + D(m) f_0) from the history and the points before the
+//           sub-block.  All but the last 8 of them are summed while the chain
+//           runs the sub-block before; the last 8 once it is done;
+//   chain   (1 warp): the sub-block's own points and the step: y^P, exchange of
+//           y^P between the lanes of the trajectory (shuffles), f(t, y^P),
+//           y = T + h^a (... + f^P / Gamma(a+2)), exchange, f(t, y);
+//   output  by the helpers, a sub-block behind: the float-float increment
+//           h^a (...) in the double-sized slot of y (finish_y_kernel adds the
+//           Taylor part in double after the last block), f as a float-float
+//           pair, and after the last step the bf16 slices of the segment that
+//           the next blocks' history reads.
+// All in float-float; GB300 runs FP64 at 1/64 of the fp32 rate with a long
+// latency, so no FP64 operation is left: the time-only part of f comes from a
+// table (aux_kernel, on another stream), parameters and y_0 from float-float
+// copies, and y becomes a double once at the end.
+//
+// The float-float operations of a column, and their order, do not depend on the
+// number of warps: the sums run over the points in ascending order whoever adds
+// them.  (They decide the last bits of f, and those now and then a slice.)
+//
+// What bounds it: alone, the latency of a step's float-float operations (a
+// product takes 25 cycles, a sum 32, a multiply-add 36, a shuffle 26; ~450 cycles
+// a step for the Lorenz type); beside the tensor kernels, which leave wide
+// batches few SMs, its issue slots.  Hence the helpers, their weights held in
+// registers (11 loads for 32 products), operand selection instead of branches
+// on the component, and the slices written here instead of by a launch of their
+// own.  A block of 64 steps alone, one or two warps per 32 columns before / now:
+// LCR 1024 58 (a lane per target) / 37.5 us, Lorenz type 256 37 (likewise) / 34,
+// oscillator 4096 97 / 49.  Whole solves: LCR 1024 x 2^14 24.1 / 19.8 ms, Lorenz
+// type 256 x 2^16 87.8 / 52.4, 256 x 2^18 494 / 422, oscillator 4096 x 2^13 20.4 /
+// 16.9, 4096 x 2^16 312 / 306.  Measured and dropped: a second chain warp for
+// the sub-block's sums, handed over target by target (40 instead of 37 us, LCR),
+// helpers that take each point as it appears (40), sub-blocks of 4 (20.7 instead
+// of 19.8 ms).
+#include <algorithm>
+#include <type_traits>
+
 #include "recurrence.cuh"
+#include "split_slices.cuh"
 
 namespace fabm {
 namespace {
 
-constexpr int kColL = kSplitSeg;  // targets per block
-constexpr int kSub = 8;           // targets per sub-block
-constexpr int kMaxWarps = 12;     // warps per CTA at most (registers: <= 168 per thread)
+constexpr int kColL = kSplitSeg;   // targets per block
+constexpr int kSub = 8;            // targets per sub-block
+constexpr int kHelpers = 4;
+constexpr int kSums = 2 * kSub / kHelpers;  // sums per helper
+constexpr int kRows = kSub / kHelpers;      // output rows per helper
+constexpr int kTeam = 1 + kHelpers;  // warps per team
+constexpr int kMaxTeams = 3;         // teams per CTA at most (registers: <= 136 per thread)
 
-// shared memory of a CTA of `warps` warps, in float-float pairs: h^a B and
-// h^a A (65 each), then per warp f of the block's points [65][32]
-constexpr int ff_per_warp(int) { return (kColL + 1) * kWarp; }
-constexpr size_t cols_smem_bytes(int D, int warps)
+// Shared memory of a team.
+struct TeamMem {
+    FF f[kColL + 1][kWarp];        // f_{cL+j} of the team's columns
+    FF inc[kColL][kWarp];          // increments of y
+    FF sum[2 * kSub][kWarp];       // handed to the chain: sums over the points before the
+    FF base[2 * kSub][kWarp];      // sub-block (running sum, errors) and bases, P then C
+    FF T[kSub][kWarp];             // Taylor part, if y'(0) is given
+    FF aux[kSub][kWarp];           // forcing of the sub-block
+};
+// Of a CTA: h^a B(d), h^a A(d), d = 0..64, then the teams.
+constexpr size_t team_smem_bytes(int teams)
 {
-    return sizeof(FF) * (2 * (kColL + 1) + (size_t)warps * ff_per_warp(D));
+    return sizeof(FF) * 2 * (kColL + 2) + teams * sizeof(TeamMem);
 }
 
 __device__ __forceinline__ bool finite_f(float x)
@@ -56,20 +88,33 @@ __device__ __forceinline__ FF ld_ff(const float2 *p)
 // (0 predictor, 1 corrector): the far value plus the near partials (at most
 // kMaxNear), all loads issued before the additions.
 constexpr int kMaxNear = 3;
-__device__ __forceinline__ FF hist_in(const HistIn &h, int k, int a, int64_t col, int cols)
+__device__ __forceinline__ void hist_load(const HistIn &h, int k, int a, int64_t col, int cols,
+                                          float2 (&v)[kMaxNear + 1])
 {
-    float2 v[kMaxNear + 1];
     v[0] = h.G ? h.G[((int64_t)k * h.g_rows + h.g_off + a) * cols + col] : make_float2(0.f, 0.f);
 #pragma unroll
     for (int ch = 0; ch < kMaxNear; ++ch)
         v[ch + 1] = ch < h.n_near ? h.near[(((int64_t)ch * 2 + k) * kColL + a) * cols + col]
                                   : make_float2(0.f, 0.f);
+}
+__device__ __forceinline__ FF hist_sum(const HistIn &h, const float2 (&v)[kMaxNear + 1])
+{
+    if (h.near_as_chunk) {  // the chunk after the last of G (combine_split_kernel)
+        float hi = v[0].x, lo = v[0].y;
+        ff_add_chunk(hi, lo, v[1].x, v[1].y);
+        return FF(hi, lo);
+    }
     FF s(v[0].x, v[0].y);
 #pragma unroll
     for (int ch = 1; ch <= kMaxNear; ++ch) s = s + FF(v[ch].x, v[ch].y);
     return s;
 }
-
+__device__ __forceinline__ FF hist_in(const HistIn &h, int k, int a, int64_t col, int cols)
+{
+    float2 v[kMaxNear + 1];
+    hist_load(h, k, a, col, cols, v);
+    return hist_sum(h, v);
+}
 // Time-only part of f for the 64 targets of block c: X[a][b] = aux(t_m, p_b),
 // m = 64c+1+a, as float-float pairs.
 template <class Rhs>
@@ -109,114 +154,92 @@ __global__ void finish_y_kernel(DevBatch bt, double h, int64_t m_lo, int64_t m_h
     }
 }
 
-// Warp w of CTA x advances the trajectories 32/D * (x * warps + w) ...; the
-// CTA size is chosen by the host so that the CTAs fill the SMs the tensor
-// history leaves free (a tensor CTA and a recurrence CTA never share an SM).
-// WB, WA: h^a B(d), h^a A(d) for d = 0..64 as float-float pairs; WD: h^a D(m);
-// F: float-float pairs in the double-sized slots of bt.F; hin: the history of
-// block c (a far value and near partials, float-float pairs); X: the
-// forcing table of block c ([64][B] pairs, aux_kernel) when Rhs::kForcing.
-// Y1: bt.y1 is set (1 < alpha < 2, Taylor part y0 + t y'(0)); a template
-// parameter so that the solves without it carry no FP64 work per step.
-template <class Rhs, int D, bool Y1>
-__global__ void __launch_bounds__(kMaxWarps *kWarp)
-    recur_cols_kernel(DevBatch bt, const float2 *__restrict__ WB, const float2 *__restrict__ WA,
-                      const float2 *__restrict__ WD, StepConsts kc, int64_t c,
-                      const HistIn hin, const float2 *__restrict__ X)
+__device__ __forceinline__ void team_sync(int id)
 {
-    constexpr int TPW = kWarp / D;  // trajectories per warp
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kTeam * kWarp) : "memory");
+}
+
+struct TeamArgs {
+    DevBatch bt;
+    const float2 *WB, *WA, *WD;
+    const float2 *par, *y0;  // float-float copies: [B][kMaxParams], [cols]
+    float2 ha, ha_ig2;       // h^a, h^a / Gamma(a+2)
+    double h;
+    int64_t c;
+    HistIn hin;
+    const float2 *X;         // forcing table of block c ([64][B] pairs), if Rhs::kForcing
+    __nv_bfloat16 *Fs;       // slices and exponents of segment c, or NULL (last block)
+    int *Ef;
+    int n_ct;
+};
+
+// Team q of CTA x advances the trajectories 32/D * (x * teams + q) ...
+// Y1: bt.y1 is set (1 < alpha < 2, Taylor part y0 + t y'(0)).
+template <class Rhs, int D, bool Y1>
+__global__ void __launch_bounds__(kMaxTeams *kTeam *kWarp)
+    recur_team_kernel(const __grid_constant__ TeamArgs a)
+{
+    constexpr int TPW = kWarp / D;  // trajectories per team
     extern __shared__ __align__(16) FF smem_ff[];
-    FF *sB = smem_ff, *sA = smem_ff + (kColL + 1);
+    FF *sB = smem_ff, *sA = smem_ff + (kColL + 2);
     const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
-    FF *wbase = smem_ff + 2 * (kColL + 1) + warp * ff_per_warp(D);
-    FF(*sF)[kWarp] = reinterpret_cast<FF(*)[kWarp]>(wbase);  // f_{cL+j} of the warp's columns
+    // warps 0 and 4 share an SM sub-partition, so the chain (role 0) is warp 1
+    const int team = warp / kTeam, role = (warp % kTeam + kTeam - 1) % kTeam;
+    TeamMem &tm = reinterpret_cast<TeamMem *>(smem_ff + 2 * (kColL + 2))[team];
+    const int bar1 = 1 + 2 * team, bar2 = 2 + 2 * team;
 
-    for (int d = threadIdx.x; d <= kColL; d += blockDim.x) sB[d] = ld_ff(WB + d), sA[d] = ld_ff(WA + d);
-    __syncthreads();  // the only CTA-wide barrier: warps run independently from here
-
+    for (int d = threadIdx.x; d <= kColL; d += blockDim.x) sB[d] = ld_ff(a.WB + d), sA[d] = ld_ff(a.WA + d);
+    const DevBatch &bt = a.bt;
     const int g = lane / D, i = lane % D;
-    const int64_t b = ((int64_t)blockIdx.x * (blockDim.x / kWarp) + warp) * TPW + g;
+    const int64_t b = ((int64_t)blockIdx.x * (blockDim.x / (kTeam * kWarp)) + team) * TPW + g;
     const bool act = g < TPW && b < bt.B;
     const int64_t bb = act ? b : 0;  // in-range index for the loads of idle lanes
     const int64_t col = bb * D + i;
-    const int64_t m0 = c * kColL;
+    const int64_t m0 = a.c * kColL;
     const int64_t Nb = act ? bt.N_each[bb] : 0;
     const int steps = (int)(Nb - m0 < 0 ? 0 : (Nb - m0 < kColL ? Nb - m0 : kColL));
     const int wsteps = (int)__reduce_max_sync(0xffffffffu, (unsigned)steps);
-    if (wsteps == 0) return;  // every trajectory of the warp has finished (uniform)
-
     const float2 *F2 = reinterpret_cast<const float2 *>(bt.F);
-    float2 *Fw = reinterpret_cast<float2 *>(bt.F);
-    sF[0][lane] = ld_ff(F2 + m0 * bt.ldF + col);
-    const FF f0 = ld_ff(F2 + col);
+    if (role == 0) tm.f[0][lane] = ld_ff(F2 + m0 * bt.ldF + col);
+    __syncthreads();         // the only CTA-wide barrier
+    if (wsteps == 0) return;  // every trajectory of the team has finished (uniform over the team)
+    const FF T0 = ld_ff(a.y0 + col);
 
-    double p[kMaxParams];
-    FF pf[kMaxParams];
+    if (role == 0) {
+        // ---- chain ----
+        FF pf[kMaxParams];
 #pragma unroll
-    for (int q = 0; q < kMaxParams; ++q) {
-        p[q] = bt.params[bb * kMaxParams + q];
-        pf[q] = ff_from_double(p[q]);
-    }
-    // time-independent aux (a constant, or 0) once per lane
-    const FF aux0 = Rhs::kForcing ? FF(0) : ff_from_double(Rhs::aux(0.0, p));
-    const double y0 = bt.y0[bb * D + i];
-    const double y1 = Y1 ? bt.y1[bb * D + i] : 0.0;
-    const FF T0 = ff_from_double(y0);
-    const FF ha = ff_from_double(kc.h_alpha[0]);
-    const FF ha_ig2 = ff_from_double(kc.h_alpha[0] * kc.inv_gamma2[0]);
-    float2 *Yb = reinterpret_cast<float2 *>(bt.Y + bb * (bt.N + 1) * D);
-    const int cols = bt.cols;
-    __syncwarp();
-
-    FF accP[kSub], accC[kSub], bP[kSub], bC[kSub], rcs[kSub], axs[kSub];
-    for (int a0 = 0; a0 < wsteps; a0 += kSub) {
-        // the sub-block's forcing values, loaded before the work that does not
-        // need them (rows a0 .. a0+7 < 64 of the [64][B] table: in range even
-        // past the last step), so the steps do not wait on them
+        for (int q = 0; q < kMaxParams; ++q) pf[q] = ld_ff(a.par + bb * kMaxParams + q);
+        // the time-independent aux is a constant right-hand side's p0 or nothing
+        const FF aux0 = std::is_same_v<Rhs, RhsConst> ? pf[0] : FF(0);
+        const FF ha_ig2(a.ha_ig2.x, a.ha_ig2.y);
+        FF fn = tm.f[0][lane];
+        for (int a0 = 0; a0 < wsteps; a0 += kSub) {
+            team_sync(bar1);  // f up to f_{cL+a0} is in tm.f
+            team_sync(bar2);  // the helpers' sums are in tm.sum
+            FF accP[kSub], accC[kSub];
 #pragma unroll
-        for (int r = 0; r < kSub; ++r)
-            axs[r] = Rhs::kForcing ? ld_ff(X + (int64_t)(a0 + r) * bt.B + bb) : aux0;
-        // bases from the history of the points k < cL
-#pragma unroll
-        for (int r = 0; r < kSub; ++r) {
-            const int a = a0 + r;
-            const FF gP = hist_in(hin, 0, a, col, cols);
-            const FF gC = hist_in(hin, 1, a, col, cols);
-            bP[r] = ha * gP;
-            bC[r] = ff_fma(ld_ff(WD + (m0 + 1 + a)), f0, ha * gC);
-            accP[r] = accC[r] = FF(0);
-        }
-        // points of the block before the sub-block: j = 0 .. a0
-        for (int j = 0; j <= a0; ++j) {
-            const FF fj = sF[j][lane];
+            for (int r = 0; r < kSub; ++r) accP[r] = tm.sum[r][lane], accC[r] = tm.sum[kSub + r][lane];
+            // no test of wsteps in here (targets past the last are computed and
+            // dropped): the steps of a sub-block are one stretch of code, so that
+            // the work off the serial path fills its latencies
 #pragma unroll
             for (int r = 0; r < kSub; ++r) {
-                const int d = a0 + r + 1 - j;
-                dot2_acc(accP[r], sB[d], fj);
-                dot2_acc(accC[r], sA[d], fj);
-            }
-        }
-        __syncwarp();
-        // the serial chain of the sub-block's steps
-#pragma unroll
-        for (int r = 0; r < kSub; ++r) {
-            if (a0 + r < wsteps) {  // uniform over the warp
-                const FF ax = axs[r];
-                // Taylor part of the initial data: y0, or y0 + t y'(0) for 1 < alpha < 2
-                FF T = T0;
-                if constexpr (Y1) T = ff_from_double(fma((double)(m0 + 1 + a0 + r) * kc.h, y1, y0));
-                const FF yp = T + (bP[r] + ff_norm(accP[r]));
+                const FF T = Y1 ? tm.T[r][lane] : T0;
+                const FF yp = T + (tm.base[r][lane] + ff_norm(accP[r]));
+                const FF ax = Rhs::kForcing ? tm.aux[r][lane] : aux0;
                 FF y[D];
 #pragma unroll
-                for (int q = 0; q < D; ++q) y[q] = shfl_ff(yp, g * D + q);
-                const FF fp = Rhs::template one<D>(i, y, pf, ax);
-                rcs[r] = bC[r] + ff_fma(ha_ig2, fp, ff_norm(accC[r]));  // h^a (history + f^P / Gamma(a+2))
-                const FF yc = T + rcs[r];
+                for (int q = 0; q < D; ++q) y[q] = D == 1 ? yp : shfl_ff(yp, g * D + q);
+                const FF fp = Rhs::template lanes<D>(i, y, yp, pf, ax);
+                // h^a (history + f^P / Gamma(a+2))
+                const FF rc = tm.base[kSub + r][lane] + ff_fma(ha_ig2, fp, ff_norm(accC[r]));
+                const FF yc = T + rc;
 #pragma unroll
-                for (int q = 0; q < D; ++q) y[q] = shfl_ff(yc, g * D + q);
-                const FF fn = Rhs::template one<D>(i, y, pf, ax);
-                sF[a0 + r + 1][lane] = fn;
-                // the sub-block's later targets take the new point now
+                for (int q = 0; q < D; ++q) y[q] = D == 1 ? yc : shfl_ff(yc, g * D + q);
+                tm.inc[a0 + r][lane] = rc;
+                fn = Rhs::template lanes<D>(i, y, yc, pf, ax);
+                tm.f[a0 + r + 1][lane] = fn;
 #pragma unroll
                 for (int r2 = r + 1; r2 < kSub; ++r2) {
                     dot2_acc(accP[r2], sB[r2 - r], fn);
@@ -224,20 +247,141 @@ __global__ void __launch_bounds__(kMaxWarps *kWarp)
                 }
             }
         }
-        // outputs of the sub-block, off the chain: the increment of y and f, as pairs
+        team_sync(bar1);  // the last sub-block is done
+        if (!a.Fs) return;
+    } else {
+        // ---- helpers: kSums sums of kind `kind`, targets r0 .. of each sub-block ----
+        const int hq = role - 1, kind = hq & 1, r0 = kSums * (hq >> 1);
+        const FF *w = kind ? sA : sB;
+        const FF ha(a.ha.x, a.ha.y);
+        const FF f0 = ld_ff(F2 + col);
+        float2 *Fw = reinterpret_cast<float2 *>(bt.F);
+        float2 *Yb = reinterpret_cast<float2 *>(bt.Y + bb * (bt.N + 1) * D);
+        FF sum[kSums];  // running sums and errors (dot2_acc)
+        float2 hv[kSums][kMaxNear + 1], wd[kSums];
+        FF xa[kRows];
+        // history and forcing of the sub-block at a0, loaded ahead of their use
+        auto fetch = [&](int a0) {
 #pragma unroll
-        for (int r = 0; r < kSub; ++r) {
-            const int a = a0 + r;
-            if (act && a < steps) {
-                const int64_t m = m0 + 1 + a;
-                const FF fn = sF[a + 1][lane];
-                Yb[m * D + i] = make_float2(rcs[r].hi, rcs[r].lo);
-                Fw[m * bt.ldF + col] = make_float2(fn.hi, fn.lo);
-                if (!(finite_f(rcs[r].hi) && finite_f(fn.hi))) report_nonfinite(bt.status, m, (int)bb);
+            for (int q = 0; q < kSums; ++q) {
+                const int t = a0 + r0 + q;
+                hist_load(a.hin, kind, t, col, bt.cols, hv[q]);
+                if (kind) wd[q] = a.WD[m0 + 1 + t];
+            }
+            if (Rhs::kForcing) {
+#pragma unroll
+                for (int q = 0; q < kRows; ++q)
+                    xa[q] = ld_ff(a.X + (int64_t)(a0 + kRows * hq + q) * bt.B + bb);
+            }
+        };
+        // the points j0 .. j0+kSub-1 to the targets s0+r0 ..
+        auto add = [&](int j0, int s0) {
+            const int d0 = s0 + r0 + 1 - j0 - (kSub - 1);
+            FF wv[kSums + kSub - 1];
+#pragma unroll
+            for (int u = 0; u < kSums + kSub - 1; ++u) wv[u] = w[d0 + u];
+#pragma unroll
+            for (int u = 0; u < kSub; ++u) {
+                const FF f = tm.f[j0 + u][lane];
+#pragma unroll
+                for (int q = 0; q < kSums; ++q) dot2_acc(sum[q], wv[q + kSub - 1 - u], f);
+            }
+        };
+        auto write_out = [&](int a0) {  // its share of the targets from a0 on
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                const int t = a0 + kRows * hq + q;
+                if (act && t < steps) {
+                    const int64_t m = m0 + 1 + t;
+                    const FF r = tm.inc[t][lane], fn = tm.f[t + 1][lane];
+                    Yb[m * D + i] = make_float2(r.hi, r.lo);
+                    Fw[m * bt.ldF + col] = make_float2(fn.hi, fn.lo);
+                    if (!(finite_f(r.hi) && finite_f(fn.hi))) report_nonfinite(bt.status, m, (int)bb);
+                }
+            }
+        };
+        // h^a times the history of the sub-block at a0
+        FF base[kSums], T[kSums];
+        auto set_bases = [&](int a0) {
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) {
+                FF v = ha * hist_sum(a.hin, hv[q]);
+                if (kind) v = ff_fma(FF(wd[q].x, wd[q].y), f0, v);
+                base[q] = v;
+                if constexpr (Y1)
+                    if (!kind)
+                        T[q] = ff_from_double(
+                            fma((double)(m0 + 1 + a0 + r0 + q) * a.h, bt.y1[col], bt.y0[col]));
+            }
+        };
+        // the sums' first point, j = 0
+        auto start = [&](int a0) {
+            const FF f = tm.f[0][lane];
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) {
+                sum[q] = FF(0);
+                dot2_acc(sum[q], w[a0 + r0 + q + 1], f);
+            }
+        };
+        fetch(0);
+        set_bases(0);
+        for (int a0 = 0; a0 < wsteps; a0 += kSub) {
+            team_sync(bar1);
+            // the newest points (j = a0-7 .. a0, or j = 0) complete the sub-block's sums
+            if (a0 == 0) start(0);
+            else add(a0 - kSub + 1, a0);
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) {
+                tm.sum[kSub * kind + r0 + q][lane] = sum[q];
+                tm.base[kSub * kind + r0 + q][lane] = base[q];
+                if (Y1 && !kind) tm.T[r0 + q][lane] = T[q];
+            }
+            if (Rhs::kForcing) {
+#pragma unroll
+                for (int q = 0; q < kRows; ++q) tm.aux[kRows * hq + q][lane] = xa[q];
+            }
+            team_sync(bar2);
+            // beside the chain's sub-block: outputs of the one before, and the
+            // next one's sums over the points known now
+            if (a0 > 0) write_out(a0 - kSub);
+            const int an = a0 + kSub;
+            if (an < wsteps) {
+                fetch(an);
+                start(an);
+                for (int j = 1; j <= a0; j += kSub) add(j, an);
+                set_bases(an);
             }
         }
-        __syncwarp();
+        team_sync(bar1);
+        write_out((wsteps - 1) / kSub * kSub);
+        if (!a.Fs) return;
     }
+
+    // the segment's slices: column = lane, points j' = 8 k1 .. (j' = 63 - j)
+    if (!act) return;
+    float m = 0.f;
+#pragma unroll 8
+    for (int j = 0; j < kColL; ++j)
+        if (j <= steps) m = fmaxf(m, fabsf(tm.f[j][lane].hi));
+    const int E = slice_exponent(m);
+    const int ct = (int)(col / 128), cloc = (int)(col % 128);
+    __nv_bfloat16 *base = slice_base(a.Fs, a.c, a.n_ct, ct, cloc);
+    for (int k1 = role; k1 < 8; k1 += kTeam) {
+        float hi[8], lo[8];
+#pragma unroll
+        for (int k0 = 0; k0 < 8; ++k0) {
+            const int j = 63 - (8 * k1 + k0);
+            const FF f = j <= steps ? tm.f[j][lane] : FF(0);
+            hi[k0] = f.hi, lo[k0] = f.lo;
+        }
+        uint32_t w[3][4];
+        slice8(hi, lo, E, w);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            *reinterpret_cast<uint4 *>(base + q * (128 * kSplitSeg) + k1 * (128 * 8)) =
+                make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+    }
+    if (role == 0) a.Ef[(a.c * a.n_ct + ct) * 128 + cloc] = E;
 }
 
 // The same block with one lane per target (targets a and a+32 on lane a), one
@@ -245,7 +389,7 @@ __global__ void __launch_bounds__(kMaxWarps *kWarp)
 // leaves the GPU mostly idle.  Every pending target adds the newest point as
 // it appears; the owner of the next target runs the step, the components
 // exchange y through shared memory.  Same inputs and outputs as
-// recur_cols_kernel.
+// recur_team_kernel, but the segment's slices are left to slice_f_kernel.
 template <class Rhs, int D>
 __global__ void __launch_bounds__(D *kWarp)
     recur_targets_kernel(DevBatch bt, const float2 *__restrict__ WB, const float2 *__restrict__ WA,
@@ -368,46 +512,69 @@ cudaError_t prepare_recur_cols(int rhs, int dim)
         auto prep = [&](auto kernel) {
             cudaFuncAttributes fa;
             if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
-            if (e == cudaSuccess && fa.numRegs * kMaxWarps * kWarp > 65536)
+            if (e == cudaSuccess && fa.numRegs * kMaxTeams * kTeam * kWarp > 65536)
                 e = cudaErrorInvalidConfiguration;
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cols_smem_bytes(D, kMaxWarps));
+                                         (int)team_smem_bytes(kMaxTeams));
         };
-        prep(recur_cols_kernel<R, D, false>);
-        prep(recur_cols_kernel<R, D, true>);
+        prep(recur_team_kernel<R, D, false>);
+        prep(recur_team_kernel<R, D, true>);
     });
     return ok ? e : cudaErrorInvalidValue;
 }
 
 int recur_cols_warps(int dim, int64_t B) { return (int)((B + kWarp / dim - 1) / (kWarp / dim)); }
 
+namespace {
+__global__ void ff_inputs_kernel(const double *__restrict__ x, int64_t n, float2 *__restrict__ y)
+{
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const FF v = ff_from_double(x[e]);
+        y[e] = make_float2(v.hi, v.lo);
+    }
+}
+}  // namespace
+
+cudaError_t launch_ff_inputs(const DevBatch &bt, float2 *par, float2 *y0, cudaStream_t st)
+{
+    auto blocks = [](int64_t n) { return (unsigned)std::min<int64_t>((n + 127) / 128, 152 * 8); };
+    const int64_t np = (int64_t)bt.B * kMaxParams;
+    ff_inputs_kernel<<<blocks(np), 128, 0, st>>>(bt.params, np, par);
+    ff_inputs_kernel<<<blocks(bt.cols), 128, 0, st>>>(bt.y0, bt.cols, y0);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_recur_cols(int rhs, const DevBatch &bt, const float2 *WB, const float2 *WA,
                               const float2 *WD, const StepConsts &k, int64_t c, const HistIn &hin,
-                              const float2 *X, int warps_per_cta, cudaStream_t st)
+                              const ColsIn &in, int warps_per_cta, cudaStream_t st)
 {
-    if (warps_per_cta < 0 || warps_per_cta > kMaxWarps) return cudaErrorInvalidValue;
+    if (warps_per_cta < 0) return cudaErrorInvalidValue;
     if (hin.n_near < 0 || hin.n_near > kMaxNear) return cudaErrorInvalidValue;
     bool need_x = false;
     const bool ok = dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
         need_x = R::kForcing;
-        if (need_x && !X) return;
+        if (need_x && !in.X) return;
         if (warps_per_cta == 0) {  // one lane per target
             recur_targets_kernel<R, D><<<(unsigned)bt.B, D * kWarp, 0, st>>>(bt, WB, WA, WD, k, c,
-                                                                             hin, X);
+                                                                             hin, in.X);
             return;
         }
-        const int warps = recur_cols_warps(D, bt.B);
-        const unsigned blocks = (unsigned)((warps + warps_per_cta - 1) / warps_per_cta);
-        const size_t smem = cols_smem_bytes(D, warps_per_cta);
+        const int teams = recur_cols_warps(D, bt.B), per = std::min(warps_per_cta, kMaxTeams);
+        const unsigned blocks = (unsigned)((teams + per - 1) / per);
+        auto pair = [](double v) {
+            const float hi = (float)v;
+            return make_float2(hi, (float)(v - (double)hi));
+        };
+        const TeamArgs a{bt, WB, WA, WD, in.par, in.y0, pair(k.h_alpha[0]),
+                         pair(k.h_alpha[0] * k.inv_gamma2[0]), k.h, c, hin, in.X, in.Fs, in.Ef, in.n_ct};
         if (bt.y1)
-            recur_cols_kernel<R, D, true><<<blocks, warps_per_cta * kWarp, smem, st>>>(
-                bt, WB, WA, WD, k, c, hin, X);
+            recur_team_kernel<R, D, true><<<blocks, per * kTeam * kWarp, team_smem_bytes(per), st>>>(a);
         else
-            recur_cols_kernel<R, D, false><<<blocks, warps_per_cta * kWarp, smem, st>>>(
-                bt, WB, WA, WD, k, c, hin, X);
+            recur_team_kernel<R, D, false><<<blocks, per * kTeam * kWarp, team_smem_bytes(per), st>>>(a);
     });
-    return ok && !(need_x && !X) ? cudaGetLastError() : cudaErrorInvalidValue;
+    return ok && !(need_x && !in.X) ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 
 bool rhs_has_forcing(int rhs, int dim)

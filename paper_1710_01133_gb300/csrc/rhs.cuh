@@ -5,8 +5,6 @@
 // split recurrence.
 #pragma once
 
-#include <type_traits>
-
 #include "fabm_internal.cuh"
 #include "ff.cuh"
 
@@ -22,11 +20,38 @@ namespace fabm {
 // Component-wise evaluation lets the recurrence run the components of one
 // trajectory on different warps.
 
+//   lanes<D>(i, y, own, p, aux)  the same for lanes of a warp with different i,
+//                        own = y[i]: operands selected, no branch (a branch on i
+//                        would run every component's form one after another)
+//
+//   one64<D>(i, y, p, aux)  where it exists, one() for the FP64 recurrences, in
+//                        fewer operations: each on a step's serial path costs 64
+//                        cycles (rhs_f64 takes it if there is one)
+//
+// The float-float operations of a component, and their order, are the same in
+// one() and lanes(), so every layout of the split recurrence gives the same bits.
+
+// v[i] for a runtime i without indexing the array dynamically (which would put
+// it in local memory)
+template <int D, class T>
+__device__ inline T comp(const T *v, int i)
+{
+    T r = v[0];
+#pragma unroll
+    for (int q = 1; q < D; ++q)
+        if (i == q) r = v[q];
+    return r;
+}
+__device__ inline FF sel(bool c, FF a, FF b) { return FF(c ? a.hi : b.hi, c ? a.lo : b.lo); }
+__device__ inline double sel(bool c, double a, double b) { return c ? a : b; }
+
 struct RhsConst {  // f_i = p0
     static constexpr bool kForcing = false;
     __device__ static double aux(double, const double *p) { return p[0]; }
     template <int D, class T>
     __device__ static T one(int, const T *, const T *, T aux) { return aux; }
+    template <int D, class T>
+    __device__ static T lanes(int, const T *, T, const T *, T aux) { return aux; }
 };
 
 struct RhsTime {  // f_i = t
@@ -34,6 +59,8 @@ struct RhsTime {  // f_i = t
     __device__ static double aux(double t, const double *) { return t; }
     template <int D, class T>
     __device__ static T one(int, const T *, const T *, T aux) { return aux; }
+    template <int D, class T>
+    __device__ static T lanes(int, const T *, T, const T *, T aux) { return aux; }
 };
 
 struct RhsLinear {  // f_i = -p0 y_i
@@ -42,13 +69,12 @@ struct RhsLinear {  // f_i = -p0 y_i
     template <int D, class T>
     __device__ static T one(int i, const T *y, const T *p, T)
     {
-        // y[i] for a runtime i without indexing the array dynamically (which
-        // would put it in local memory)
-        T v = y[0];
-#pragma unroll
-        for (int q = 1; q < D; ++q)
-            if (i == q) v = y[q];
-        return -p[0] * v;
+        return -p[0] * comp<D>(y, i);
+    }
+    template <int D, class T>
+    __device__ static T lanes(int, const T *, T own, const T *p, T)
+    {
+        return -p[0] * own;
     }
 };
 
@@ -62,6 +88,13 @@ struct RhsLorenz {  // p = (sigma, rho, beta)
         if (i == 1) return y[0] * (p[1] - y[2]) - y[1];
         return y[0] * y[1] - p[2] * y[2];
     }
+    template <int D, class T>
+    __device__ static T lanes(int i, const T *y, T, const T *p, T)
+    {
+        const T d = sel(i == 0, y[1], p[1]) - sel(i == 0, y[0], y[2]);   // y - x, rho - z
+        const T m = sel(i == 0, p[0], y[0]) * sel(i == 2, y[1], d);     // sigma d, x d, x y
+        return sel(i == 0, m, m - sel(i == 1, y[1], p[2] * y[2]));
+    }
 };
 
 struct RhsDuffing {  // p = (gamma, omega, F): x' = y, y' = -gamma y - x - x^3 + F cos(omega t)
@@ -72,11 +105,17 @@ struct RhsDuffing {  // p = (gamma, omega, F): x' = y, y' = -gamma y - x - x^3 +
     {
         if (i == 0) return y[1];
         const T x = y[0];
-        // in double every operation is on the step's serial path: three of them
-        if constexpr (std::is_same_v<T, double>)
-            return fma(-x, fma(x, x, 1.0), fma(-p[0], y[1], aux));
-        else
-            return aux - (p[0] * y[1] + x * (T(1) + x * x));
+        return aux - (p[0] * y[1] + x * (T(1) + x * x));
+    }
+    template <int D>
+    __device__ static double one64(int i, const double *y, const double *p, double aux)
+    {
+        return i == 0 ? y[1] : fma(-y[0], fma(y[0], y[0], 1.0), fma(-p[0], y[1], aux));
+    }
+    template <int D, class T>
+    __device__ static T lanes(int i, const T *y, T, const T *p, T aux)
+    {
+        return sel(i == 0, y[1], RhsDuffing::one<D>(1, y, p, aux));
     }
 };
 
@@ -88,25 +127,22 @@ struct RhsManufactured {  // f = p0 t^p1 + t^p2 - y
     {
         return aux - y[0];
     }
+    template <int D, class T>
+    __device__ static T lanes(int, const T *, T own, const T *, T aux)
+    {
+        return aux - own;
+    }
 };
 
 struct RhsLcr {  // Sec. 5, Eq. sys.LRC; p = (sigma, omega, a, b, f)
     static constexpr bool kForcing = true;
     __device__ static double aux(double t, const double *p) { return p[4] * sin(p[1] * t); }
+    // y - g(x), g = a x for |x| < 1, else b x +- (a - b); aux - (sigma y + x)
     template <int D, class T>
     __device__ static T one(int i, const T *y, const T *p, T aux)
     {
-        const T x = y[0];
+        const T x = y[0], a = p[2], b = p[3];
         if (i == 1) return aux - (p[0] * y[1] + x);
-        const T a = p[2], b = p[3];
-        if constexpr (std::is_same_v<T, double>) {
-            // |x| >= 1 from the exponent bits, and g = slope x + offset in one FMA
-            // (an FP64 comparison costs the serial path as much as an FMA)
-            const int hx = __double2hiint(x);
-            const bool out = (hx & 0x7fffffff) >= 0x3ff00000;
-            const double ab = a - b, off = out ? (hx < 0 ? -ab : ab) : 0.0;
-            return fma(-(out ? b : a), x, y[1] - off);
-        }
         T g;
         if (x <= T(-1))
             g = b * x - a + b;
@@ -116,7 +152,38 @@ struct RhsLcr {  // Sec. 5, Eq. sys.LRC; p = (sigma, omega, a, b, f)
             g = a * x;
         return y[1] - g;
     }
+    // |x| >= 1 from the exponent bits (an FP64 comparison costs the serial path as
+    // much as an FMA), and g = slope x + offset
+    template <int D>
+    __device__ static double one64(int i, const double *y, const double *p, double aux)
+    {
+        const double x = y[0];
+        if (i == 1) return aux - fma(p[0], y[1], x);
+        const int hx = __double2hiint(x);
+        const bool out = (hx & 0x7fffffff) >= 0x3ff00000;
+        const double ab = p[2] - p[3], off = out ? (hx < 0 ? -ab : ab) : 0.0;
+        return fma(-(out ? p[3] : p[2]), x, y[1] - off);
+    }
+    template <int D, class T>
+    __device__ static T lanes(int i, const T *y, T, const T *p, T aux)
+    {
+        const T x = y[0], a = p[2], b = p[3];
+        const bool lo = x <= T(-1), out = lo || x >= T(1);
+        const T m = sel(i == 0, sel(out, b, a), p[0]) * sel(i == 0, x, y[1]);
+        const T v = m + sel(i == 0, sel(lo, -a, a), x);
+        return sel(i == 0, y[1], aux) - sel(i == 0, sel(out, v + sel(lo, b, -b), m), v);
+    }
 };
+
+// Component i of f in double.
+template <class Rhs, int D>
+__device__ __forceinline__ double rhs_f64(int i, const double *y, const double *p, double aux)
+{
+    if constexpr (requires { Rhs::template one64<D>(i, y, p, aux); })
+        return Rhs::template one64<D>(i, y, p, aux);
+    else
+        return Rhs::template one<D>(i, y, p, aux);
+}
 
 // Calls fn.template operator()<Rhs, D>() for the (rhs, dim) pair; returns false
 // if the pair is not supported.
