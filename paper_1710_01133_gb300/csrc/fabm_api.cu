@@ -435,6 +435,16 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
     const int64_t cols = bt.cols;
     const bool split = hk == FABM_HIST_TENSOR;
     const int lag = history_lag(hk, s->plan_N > 0 ? s->plan_N : Nmax, cols);
+    // compensated fp32, one history launch at a time: history and steps on SMs of
+    // their own, if every block's history leaves enough
+    bool alone = false;
+    if (hk == FABM_HIST_FP32C && lag == 1) {
+        int n_chunks;
+        int64_t kc;
+        plan_chunks(std::max<int64_t>(nblk - lag, 1) * L, (int)cols, max_chunks,
+                    s->chunk_ctas > 0 ? s->chunk_ctas : auto_chunk_ctas(hk, cols), &n_chunks, &kc);
+        alone = fp32c_alone(n_chunks, (int)cols, bt.B);
+    }
     const int n_gbuf = lag + 1;  // G of block c is read by R(c) until H(c + lag + 1) starts
     s->sample_now = true;
     FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
@@ -574,7 +584,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             } else if (hk == FABM_HIST_FP32C) {
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, gs, flops, [&] {
                     return launch_hist_fp32c(bt, s->wBf.p, s->wAf.p, w.stride, c, lag, n_chunks,
-                                             kc, s->spart.p + poff, gs);
+                                             kc, alone, s->spart.p + poff, gs);
                 }));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, gs, 0.0, [&] {
                     return launch_combine_split(s->spart.p + poff, n_chunks, (int)cols, L, Gbuf, gs);
@@ -609,7 +619,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                 return launch_recur_cols(s->rhs, bt, s->wBff.p, s->wAff.p, s->wDff.p, s->k, c, hin,
                                          in, s->cols_warps, s->sR);
             }
-            return launch_recur(s->rhs, bt, w, s->k, c, L, lag, s->precision == FABM_SPLIT,
+            return launch_recur(s->rhs, bt, w, s->k, c, L, lag, s->precision == FABM_SPLIT, alone,
                                 static_cast<const double *>(Gc), s->sR);
         }));
         if (split && c + 1 < nblk && s->cols_warps == 0) {  // the other layout writes them itself

@@ -97,8 +97,10 @@ cudaError_t launch_hist_reduce(const double *part, int n_chunks, int L, int cols
 // NULL when c <= lag; the lag blocks (lag 1 or 2) before block c are summed by
 // the recurrence.  split = false: all in double; split = true: FP64 bases and
 // corrector update, short-range sums and f in float-float (recur_block_split).
+// alone: no other CTA on its SM (split only).
 cudaError_t launch_recur(int rhs, const DevBatch &bt, const DevWeights &w, const StepConsts &k,
-                         int64_t c, int L, int lag, bool split, const double *G, cudaStream_t st);
+                         int64_t c, int L, int lag, bool split, bool alone, const double *G,
+                         cudaStream_t st);
 
 // Message returned by fabm_last_error() on the calling thread.
 void set_last_error(const char *msg);
@@ -314,11 +316,16 @@ cudaError_t launch_reduce_x2(const double2 *part, int n_chunks, int cols, double
 // y[i] = (float)x[i], i < n.
 cudaError_t launch_to_float(const double *x, int64_t n, float *y, cudaStream_t st);
 
+// Dynamic shared memory that keeps a second CTA of the same kind off an SM.
+constexpr size_t kAloneSmem = 116 * 1024;
+// A history launch of n_chunks chunks leaves an SM to each of B trajectories'
+// recurrences (both are then launched one CTA per SM).
+bool fp32c_alone(int n_chunks, int cols, int B);
 // Far history of block c (32 targets) over k < (c-lag)*32 in compensated fp32;
 // partials as float2 (sum, -compensation), n_chunks x 2 x 32 x cols.
 // wstride > 0: one order per component (weights of component i at WBf + i*wstride).
 cudaError_t launch_hist_fp32c(const DevBatch &bt, const float *WBf, const float *WAf,
                               int64_t wstride, int64_t c, int lag, int n_chunks, int64_t kc,
-                              float2 *part, cudaStream_t st);
+                              bool alone, float2 *part, cudaStream_t st);
 
 }  // namespace fabm

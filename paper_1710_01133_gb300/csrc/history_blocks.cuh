@@ -119,30 +119,38 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v)
     sum = t;
 }
 
-// One CTA of 32 * kHistCols threads: chunk `chunk` of the far history of
-// block c for the columns col0 .. col0+3, in compensated fp32.  Ff: f rounded
+// Shared memory of a group of 32 * kColsPerCta threads.
+template <bool MULTI>
+struct Tiles {
+    static constexpr int NW = MULTI ? kColsPerCta : 1;  // weight windows
+    float F[kTile * kColsPerCta];
+    float B[NW][kTile + kL], A[NW][kTile + kL];
+};
+
+// A group of 32 * kColsPerCta threads (tid among them, synchronised by sync()):
+// chunk `chunk` of the far history of block c for the columns col0 .. col0+3, in
+// compensated fp32.  Ff: f rounded
 // to float (same layout as F), read instead of converting F when not NULL.
 // The next tile's f and weights are loaded into registers while the current
 // tile is summed, so the staging latency hides behind the arithmetic.
 // MULTI as for hist_fp64_block.
-template <bool MULTI = false>
-__device__ inline void hist_fp32c_block(const double *__restrict__ F, const float *__restrict__ Ff,
+template <bool MULTI, class Sync>
+__device__ inline void hist_fp32c_chunk(const double *__restrict__ F, const float *__restrict__ Ff,
                                         int64_t ldF, int cols, const float *__restrict__ WB,
                                         const float *__restrict__ WA, int64_t c, int64_t kc,
                                         int64_t k_end, float2 *__restrict__ part, int64_t chunk,
-                                        int col0, int64_t wstride = 0, int dim = 1)
+                                        int col0, int64_t wstride, int dim, int tid, Tiles<MULTI> &tl, Sync sync)
 {
     constexpr int NW = MULTI ? kColsPerCta : 1;  // weight windows
     constexpr int kThreads = kWarp * kColsPerCta;
     constexpr int kRF = kTile * kColsPerCta / kThreads;            // f values per thread
     constexpr int kRW = (NW * (kTile + kL) + kThreads - 1) / kThreads;  // weights per thread and kind
-    __shared__ float sF[kTile * kColsPerCta];
-    __shared__ float sB[NW][kTile + kL], sA[NW][kTile + kL];
+    float *sF = tl.F, (*sB)[kTile + kL] = tl.B, (*sA)[kTile + kL] = tl.A;
     const int64_t k0 = chunk * kc;
     const int64_t k1 = k0 + kc < k_end ? k0 + kc : k_end;
     const int ncol = min(kColsPerCta, cols - col0);
-    const int w = threadIdx.x / kWarp;
-    const int a = threadIdx.x % kWarp;  // target m = cL+1+a
+    const int w = tid / kWarp;
+    const int a = tid % kWarp;  // target m = cL+1+a
     float sp = 0.f, cp = 0.f, sc = 0.f, cc = 0.f;
     float rf[kRF], rb[kRW], ra[kRW];
 
@@ -153,7 +161,7 @@ __device__ inline void hist_fp32c_block(const double *__restrict__ F, const floa
         const int64_t d_min = c * kL + 2 - t1;
 #pragma unroll
         for (int u = 0; u < kRW; ++u) {
-            const int i = threadIdx.x + u * kThreads;
+            const int i = tid + u * kThreads;
             const int v = MULTI ? i / nwin : 0, ii = MULTI ? i % nwin : i;
             const bool in = MULTI ? i < NW * nwin : i < nwin;
             const int64_t o = MULTI ? (int64_t)((col0 + v) % dim) * wstride : 0;
@@ -162,7 +170,7 @@ __device__ inline void hist_fp32c_block(const double *__restrict__ F, const floa
         }
 #pragma unroll
         for (int u = 0; u < kRF; ++u) {
-            const int i = threadIdx.x + u * kThreads;
+            const int i = tid + u * kThreads;
             const int k = i / kColsPerCta, j = i % kColsPerCta;
             float f = 0.f;
             if (k < nk && j < ncol)
@@ -177,7 +185,7 @@ __device__ inline void hist_fp32c_block(const double *__restrict__ F, const floa
         const int nk = (int)(t1 - t0), nwin = nk + kL - 1;
 #pragma unroll
         for (int u = 0; u < kRW; ++u) {
-            const int i = threadIdx.x + u * kThreads;
+            const int i = tid + u * kThreads;
             if (MULTI ? i < NW * nwin : i < nwin) {
                 const int v = MULTI ? i / nwin : 0, ii = MULTI ? i % nwin : i;
                 sB[v][ii] = rb[u];
@@ -185,8 +193,8 @@ __device__ inline void hist_fp32c_block(const double *__restrict__ F, const floa
             }
         }
 #pragma unroll
-        for (int u = 0; u < kRF; ++u) sF[threadIdx.x + u * kThreads] = rf[u];
-        __syncthreads();
+        for (int u = 0; u < kRF; ++u) sF[tid + u * kThreads] = rf[u];
+        sync();
         if (t1 < k1) fetch(t1);  // next tile in flight during the sums below
         if (w < ncol) {
             const float *fb = sF + w;
@@ -213,7 +221,7 @@ __device__ inline void hist_fp32c_block(const double *__restrict__ F, const floa
             kahan_add(sp, cp, gp);
             kahan_add(sc, cc, gc);
         }
-        __syncthreads();
+        sync();
     }
     if (w < ncol) {
         float2 *out = part + ((chunk * 2) * kL + a) * (int64_t)cols + col0 + w;

@@ -17,16 +17,24 @@
 namespace fabm {
 namespace {
 
-// grid = (n_chunks, ceil(cols / kColsPerCta)); block = 32 * kColsPerCta.
+// grid = (ceil(n_chunks / pack), ceil(cols / kColsPerCta)); block = pack groups of
+// 32 * kColsPerCta threads, one chunk each.
+constexpr int kGroup = kWarp * hist::kColsPerCta;
+constexpr int kPack = 3;  // groups per CTA where the launch leaves SMs free
 template <bool MULTI>
-__global__ void __launch_bounds__(kWarp *hist::kColsPerCta)
+__global__ void __launch_bounds__(kPack *kGroup)
     hist_fp32c_kernel(const double *__restrict__ F, const float *__restrict__ Ff, int64_t ldF,
                       int cols, const float *__restrict__ WB, const float *__restrict__ WA,
-                      int64_t c, int64_t kc, int64_t k_end, float2 *__restrict__ part,
+                      int64_t c, int64_t kc, int64_t k_end, int n_chunks, float2 *__restrict__ part,
                       int64_t wstride, int dim)
 {
-    hist::f32c::hist_fp32c_block<MULTI>(F, Ff, ldF, cols, WB, WA, c, kc, k_end, part, blockIdx.x,
-                                        blockIdx.y * hist::kColsPerCta, wstride, dim);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int g = threadIdx.x / kGroup, chunk = blockIdx.x * (blockDim.x / kGroup) + g;
+    if (chunk >= n_chunks) return;
+    hist::f32c::hist_fp32c_chunk<MULTI>(
+        F, Ff, ldF, cols, WB, WA, c, kc, k_end, part, chunk, blockIdx.y * hist::kColsPerCta, wstride,
+        dim, threadIdx.x % kGroup, reinterpret_cast<hist::f32c::Tiles<MULTI> *>(smem)[g],
+        [g] { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroup) : "memory"); });
 }
 
 __global__ void to_float_kernel(const double *__restrict__ x, int64_t n, float *__restrict__ y)
@@ -48,19 +56,39 @@ cudaError_t launch_to_float(const double *x, int64_t n, float *y, cudaStream_t s
 
 cudaError_t launch_hist_fp32c(const DevBatch &bt, const float *WBf, const float *WAf,
                               int64_t wstride, int64_t c, int lag, int n_chunks, int64_t kc,
-                              float2 *part, cudaStream_t st)
+                              bool alone, float2 *part, cudaStream_t st)
 {
     const int64_t k_end = (c - lag) * hist::kL;
     if (lag < 1) return cudaErrorInvalidValue;
     if (k_end <= 0) return cudaSuccess;
-    dim3 grid((unsigned)n_chunks, (unsigned)((bt.cols + hist::kColsPerCta - 1) / hist::kColsPerCta));
-    if (wstride)
-        hist_fp32c_kernel<true><<<grid, kWarp * hist::kColsPerCta, 0, st>>>(
-            bt.F, bt.Ff, bt.ldF, bt.cols, WBf, WAf, c, kc, k_end, part, wstride, bt.dim);
-    else
-        hist_fp32c_kernel<false><<<grid, kWarp * hist::kColsPerCta, 0, st>>>(
-            bt.F, bt.Ff, bt.ldF, bt.cols, WBf, WAf, c, kc, k_end, part, 0, 1);
-    return cudaGetLastError();
+    // The recurrence of the block before runs beside this launch on an SM per
+    // trajectory, and a step's latency grows by a third where history warps share
+    // its SM (Lorenz type 2^16: 724 cycles a step against 550 alone).  So where
+    // three chunks per CTA leave SMs free (fp32c_alone), each CTA takes an SM of
+    // its own, and so does the recurrence.  The chunks and their sums stay as
+    // they are.
+    const int groups = (bt.cols + hist::kColsPerCta - 1) / hist::kColsPerCta;
+    const int pack = alone ? kPack : 1;
+    auto run = [&](auto kernel, size_t tiles, int64_t stride, int dim) -> cudaError_t {
+        size_t smem = tiles * pack;
+        if (alone) smem = smem > kAloneSmem ? smem : kAloneSmem;
+        if (smem > 48 * 1024) {
+            const cudaError_t e =
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        kernel<<<dim3((unsigned)((n_chunks + pack - 1) / pack), (unsigned)groups), pack * kGroup, smem, st>>>(
+            bt.F, bt.Ff, bt.ldF, bt.cols, WBf, WAf, c, kc, k_end, n_chunks, part, stride, dim);
+        return cudaGetLastError();
+    };
+    if (wstride) return run(hist_fp32c_kernel<true>, sizeof(hist::f32c::Tiles<true>), wstride, bt.dim);
+    return run(hist_fp32c_kernel<false>, sizeof(hist::f32c::Tiles<false>), 0, 1);
+}
+
+bool fp32c_alone(int n_chunks, int cols, int B)
+{
+    const int groups = (cols + hist::kColsPerCta - 1) / hist::kColsPerCta;
+    return (n_chunks + kPack - 1) / kPack * groups + B <= 148;
 }
 
 }  // namespace fabm

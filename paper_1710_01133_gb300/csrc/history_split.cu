@@ -458,8 +458,8 @@ __global__ void __launch_bounds__(kThreads, 1) hist_split_kernel(const SplitArgs
 }
 
 // a3: G[kind][t][col] = sum over chunks of the float-float partials, R lanes
-// per output, each summing chunks r, r+R, ... in ascending order (four loads
-// in flight), then a fixed xor tree, in compensated float-float (~48 bits,
+// per output, each summing chunks r, r+R, ... in ascending order (up to 16 loads
+// in flight: the launch is a few CTAs waiting for L2), then a fixed xor tree, in compensated float-float (~48 bits,
 // 2^24 finer than the fp32 partials).  Out = float2 (tensor path) keeps the
 // pair; Out = double (compensated-fp32 history) rounds hi + lo once.  The
 // combine sits on the serial chain of every block and FP64 issues at 1/64 of
@@ -477,20 +477,18 @@ __global__ void combine_split_kernel(const float2 *__restrict__ part, int n_chun
         float hi = 0.f, lo = 0.f;
         if (o < n_out) {
             int ch = r;
-            for (; ch + 3 * R < n_chunks; ch += 4 * R) {
-                const float2 v0 = part[(int64_t)ch * n_out + o];
-                const float2 v1 = part[(int64_t)(ch + R) * n_out + o];
-                const float2 v2 = part[(int64_t)(ch + 2 * R) * n_out + o];
-                const float2 v3 = part[(int64_t)(ch + 3 * R) * n_out + o];
-                ff_add_chunk(hi, lo, v0.x, v0.y);
-                ff_add_chunk(hi, lo, v1.x, v1.y);
-                ff_add_chunk(hi, lo, v2.x, v2.y);
-                ff_add_chunk(hi, lo, v3.x, v3.y);
-            }
-            for (; ch < n_chunks; ch += R) {
-                const float2 v = part[(int64_t)ch * n_out + o];
-                ff_add_chunk(hi, lo, v.x, v.y);
-            }
+            auto batch = [&]<int U>() {  // U loads in flight
+                for (; ch + (U - 1) * R < n_chunks; ch += U * R) {
+                    float2 v[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) v[u] = part[(int64_t)(ch + u * R) * n_out + o];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) ff_add_chunk(hi, lo, v[u].x, v[u].y);
+                }
+            };
+            batch.template operator()<16>();
+            batch.template operator()<4>();
+            batch.template operator()<1>();
         }
 #pragma unroll
         for (int off = R / 2; off > 0; off >>= 1) {

@@ -12,12 +12,13 @@ __global__ void init_kernel(DevBatch bt, bool f_pairs)
 }
 
 template <class Rhs, int D, int TPL, bool SPLIT, int LAG>
-__global__ void __launch_bounds__(D *kWarp)
+__global__ void __launch_bounds__((D + 1) * kWarp)
     recur_kernel(DevBatch bt, DevWeights w, StepConsts kc, int64_t c, const double *G)
 {
     if constexpr (SPLIT) {
-        __shared__ __align__(16) float smem_f[recur_split_smem_floats<D, TPL, LAG>()];
-        recur_block_split<Rhs, D, TPL, LAG>(bt, blockIdx.x, w, kc, c, G, smem_f);
+        static_assert(TPL == 1);
+        __shared__ __align__(16) float smem_f[recur_split_smem_floats<D, LAG>()];
+        recur_block_split<Rhs, D, LAG>(bt, blockIdx.x, w, kc, c, G, smem_f);
     } else {
         __shared__ double smem[recur_smem_doubles<D, TPL, LAG>()];
         recur_block<Rhs, D, TPL, LAG>(bt, blockIdx.x, w, kc, c, G, smem);
@@ -26,11 +27,19 @@ __global__ void __launch_bounds__(D *kWarp)
 
 template <int TPL, bool SPLIT, int LAG>
 bool launch_recur_t(int rhs, const DevBatch &bt, const DevWeights &w, const StepConsts &k,
-                    int64_t c, const double *G, cudaStream_t st)
+                    int64_t c, bool alone, const double *G, cudaStream_t st)
 {
-    return dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
-        recur_kernel<R, D, TPL, SPLIT, LAG><<<(unsigned)bt.B, D * kWarp, 0, st>>>(bt, w, k, c, G);
+    bool set = true;
+    const bool ok = dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
+        constexpr int warps = SPLIT ? recur_split_warps<R, D>() : D;
+        auto kernel = recur_kernel<R, D, TPL, SPLIT, LAG>;
+        const size_t smem = alone ? kAloneSmem : 0;
+        if (alone)
+            set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem) == cudaSuccess;
+        if (set) kernel<<<(unsigned)bt.B, warps * kWarp, smem, st>>>(bt, w, k, c, G);
     });
+    return ok && set;
 }
 
 }  // namespace
@@ -46,15 +55,16 @@ cudaError_t launch_init(int rhs, const DevBatch &bt, cudaStream_t st, bool f_pai
 }
 
 cudaError_t launch_recur(int rhs, const DevBatch &bt, const DevWeights &w, const StepConsts &k,
-                         int64_t c, int L, int lag, bool split, const double *G, cudaStream_t st)
+                         int64_t c, int L, int lag, bool split, bool alone, const double *G,
+                         cudaStream_t st)
 {
     bool ok = false;
     if (L == kWarp && lag == 1)
-        ok = split ? launch_recur_t<1, true, 1>(rhs, bt, w, k, c, G, st)
-                   : launch_recur_t<1, false, 1>(rhs, bt, w, k, c, G, st);
+        ok = split ? launch_recur_t<1, true, 1>(rhs, bt, w, k, c, alone, G, st)
+                   : launch_recur_t<1, false, 1>(rhs, bt, w, k, c, false, G, st);
     else if (L == kWarp && lag == 2)
-        ok = split ? launch_recur_t<1, true, 2>(rhs, bt, w, k, c, G, st)
-                   : launch_recur_t<1, false, 2>(rhs, bt, w, k, c, G, st);
+        ok = split ? launch_recur_t<1, true, 2>(rhs, bt, w, k, c, alone, G, st)
+                   : launch_recur_t<1, false, 2>(rhs, bt, w, k, c, false, G, st);
     return ok ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 

@@ -218,13 +218,13 @@ __device__ void recur_block(const DevBatch &bt, int b, const DevWeights &w, cons
 // ---- split precision ----
 //
 // The same block of steps for the split path with no FP64 operation on the
-// serial chain of a step.  Per target (lane a, slot t):
+// serial chain of a step.  Per target (lane a):
 //   base    y0 + h^alpha (far part + D(m) f_0), FP64, at block start;
-//   near    the lag-1 block and the in-block points, h^alpha w(d) f_k summed
-//           in float-float (ff.cuh, ~48 bits) as the points become known;
-//   step    the owner forms, in float-float,
-//             y^P = base_P + near_P,  inc = near_C + h^alpha/Gamma(alpha+2) f(t, y^P),
-//           evaluates f(t, base_C + inc), and keeps inc and f;
+//   near    the lag blocks and the in-block points, h^alpha w(d) f_k summed in
+//           float-float (ff.cuh, ~48 bits) as the points become known;
+//   step    y^P = base_P + near_P,  inc = near_C + h^alpha/Gamma(alpha+2) f(t, y^P),
+//           then f(t, base_C + inc), all in float-float; the owner of the target
+//           keeps inc and f;
 //   end     y = base_C + inc (the FP64 corrector update) and f_k are written
 //           as doubles, one target per lane, for the whole block at once.
 // Float-float carries ~48 bits, so the recurrence adds rounding far below
@@ -232,152 +232,201 @@ __device__ void recur_block(const DevBatch &bt, int b, const DevWeights &w, cons
 // and a float-float operation completes in fewer cycles than one FP64
 // operation, so the chain is shorter and wide batches no longer saturate the
 // FP64 pipe.
-template <int D, int TPL, int LAG = 1>
+//
+// What bounds it: the latency of a step's operations (~450 cycles for the
+// Lorenz type).  Every lane runs the step on values that the owner puts into
+// shared memory, so f ends up in all of them without another shuffle and no lane
+// diverges; a component's code is compiled for it, so a warp converts and
+// branches on nothing it does not use; the forcing is evaluated by a warp of its
+// own beside the lag blocks; all global loads of a block are issued together.
+// Whole solves: Lorenz type 2^16 35.7 -> 25.8 ms (of that 5 ms from SMs of its own,
+// history_fp32c.cu), scalar 10^4 3.43 -> 2.92, oscillator 20 x 2^13 5.8 -> 4.0.
+template <int D, int LAG = 1>
 __host__ __device__ constexpr int recur_split_smem_floats()
 {
-    return 4 * ((LAG + 1) * kWarp * TPL + 1) * D + 4 * D + 2 * (LAG * kWarp * TPL + 1) * D;
+    return 4 * ((LAG + 1) * kWarp + 1) * D + 8 * D + 2 * (LAG * kWarp + 1) * D + 2 * kWarp;
+}
+// Warps of a CTA for recur_block_split: one per component, and one for the forcing.
+template <class Rhs, int D>
+constexpr int recur_split_warps()
+{
+    return D + (Rhs::kForcing ? 1 : 0);
 }
 
-// smem: recur_split_smem_floats<D, TPL, LAG>() floats, 8-byte aligned; LAG as
-// for recur_block
-template <class Rhs, int D, int TPL, int LAG = 1>
-__device__ void recur_block_split(const DevBatch &bt, int b, const DevWeights &w,
-                                  const StepConsts &kc, int64_t c, const double *G, float *smem)
-{
-    constexpr int L = kWarp * TPL;
-    constexpr int W = (LAG + 1) * L + 1;
-    FF *sB = reinterpret_cast<FF *>(smem);  // [D][W]  h^alpha_i B_i(d)
-    FF *sA = sB + D * W;                    // [D][W]  h^alpha_i A_i(d)
-    FF(*sy)[D] = reinterpret_cast<FF(*)[D]>(sA + D * W);  // [2][D]
-    FF(*sF)[D] = sy + 2;                    // [LAG L + 1][D]: f of the lag blocks and f_{m0}
-    const bool act = threadIdx.x / kWarp < D;
-    const int i = act ? threadIdx.x / kWarp : 0;
-    const int lane = threadIdx.x % kWarp;
-    const int64_t Nb = bt.N_each[b];
-    const int64_t m0 = c * L;
-    if (m0 >= Nb) return;
-    const int nW = w.stride ? D : 1;  // one weight set per order
-    for (int j = threadIdx.x; j < nW * W; j += blockDim.x) {
-        const int q = j / W, jj = j % W;
-        const double hq = pick<D>(kc.h_alpha, q);
-        sB[j] = ff_from_double(hq * w.B[q * w.stride + jj]);
-        sA[j] = ff_from_double(hq * w.A[q * w.stride + jj]);
+template <int D, int LAG>
+struct SplitMem {
+    static constexpr int L = kWarp, W = (LAG + 1) * L + 1;  // distances 0 .. (LAG+1) L
+    FF *sB, *sA;      // [D or 1][W]  h^alpha_i B_i(d), A_i(d)
+    FF (*sy)[2 * D];  // [2 parities][predictor, corrector][D]
+    FF (*sF)[D];      // [LAG L + 1][D]: f of the lag blocks and f_{m0}
+    FF *aux;          // [L] forcing
+    __device__ explicit SplitMem(float *smem)
+    {
+        sB = reinterpret_cast<FF *>(smem);
+        sA = sB + D * W;
+        sy = reinterpret_cast<FF(*)[2 * D]>(sA + D * W);
+        sF = reinterpret_cast<FF(*)[D]>(sy + 2);
+        aux = reinterpret_cast<FF *>(sF + LAG * L + 1);
     }
-    for (int j = threadIdx.x; j < (LAG * L + 1) * D; j += blockDim.x) {
-        const int64_t row = m0 - LAG * L + j / D;
-        sF[j / D][j % D] =
-            ff_from_double(row >= 0 ? bt.F[row * bt.ldF + (int64_t)b * D + j % D] : 0.0);
-    }
-    __syncthreads();
+};
 
-    double p[kMaxParams];
+// What a component's warp reads from global memory, loaded before anything waits.
+struct SplitIn {
+    double p[kMaxParams], y0, y1, f0, wD, gP, gC;
+};
+
+// Component I's part, by one warp; barrier 1 joins the D component warps.
+template <class Rhs, int D, int LAG, int I>
+__device__ __forceinline__ void split_steps(const DevBatch &bt, int b, const DevWeights &w,
+                                            const StepConsts &kc, int64_t c, int64_t Nb,
+                                            const SplitIn &in0, const SplitMem<D, LAG> &m)
+{
+    constexpr int L = kWarp;
+    const int lane = threadIdx.x % kWarp;
+    const int64_t m0 = c * L, mt = m0 + 1 + lane;
+    const FF *sB = m.sB + (w.stride ? I * m.W : 0), *sA = m.sA + (w.stride ? I * m.W : 0);
     FF pf[kMaxParams];
 #pragma unroll
-    for (int q = 0; q < kMaxParams; ++q) {
-        p[q] = bt.params[(int64_t)b * kMaxParams + q];
-        pf[q] = ff_from_double(p[q]);
-    }
-    const double y0 = bt.y0[(int64_t)b * D + i];
-    const int64_t col = (int64_t)b * D + i;
-    const double ha = pick<D>(kc.h_alpha, i);
-    const FF ha_ig2 = ff_from_double(ha * pick<D>(kc.inv_gamma2, i));
-    const double f0 = bt.F[col];
-    const double *wD = w.D + i * w.stride;
-    if (w.stride) sB += i * W, sA += i * W;  // this warp's component's order
-
-    double baseC[TPL];
-    FF bP[TPL], bC[TPL], aux[TPL], nP[TPL], nC[TPL], inc[TPL], fo[TPL];
-    const double y1 = bt.y1 ? bt.y1[col] : 0.0;
-#pragma unroll
-    for (int t = 0; t < TPL; ++t) {
-        const int a = lane + kWarp * t;
-        const int64_t m = m0 + 1 + a;
-        aux[t] = ff_from_double(Rhs::aux((double)m * kc.h, p));
-        const double Tm = bt.y1 ? fma((double)m * kc.h, y1, y0) : y0;  // Taylor part at t_m
-        const double gP = G ? G[(int64_t)a * bt.cols + col] : 0.0;
-        const double gC = fma(wD[m], f0, G ? G[(int64_t)(L + a) * bt.cols + col] : 0.0);
-        baseC[t] = fma(ha, gC, Tm);
-        bP[t] = ff_from_double(fma(ha, gP, Tm));
-        bC[t] = ff_from_double(baseC[t]);
-        nP[t] = nC[t] = inc[t] = fo[t] = FF(0);
-    }
+    for (int q = 0; q < kMaxParams; ++q) pf[q] = ff_from_double(in0.p[q]);
+    const int64_t col = (int64_t)b * D + I;
+    const double ha = kc.h_alpha[I];
+    const FF ha_ig2 = ff_from_double(ha * kc.inv_gamma2[I]);
+    const double Tm = bt.y1 ? fma((double)mt * kc.h, in0.y1, in0.y0) : in0.y0;  // Taylor part at t_m
+    const double gP = in0.gP, gC = fma(in0.wD, in0.f0, in0.gC);
+    const double baseC = fma(ha, gC, Tm);
+    const FF bP = ff_from_double(fma(ha, gP, Tm)), bC = ff_from_double(baseC);
+    FF nP(0), nC(0), inc(0), fo(0);
     if (c >= 1) {  // lag blocks: k = m0-LAG*L+j, d = LAG*L+1+a-j in [2, (LAG+1)L]
+#pragma unroll 8
         for (int j = 0; j < LAG * L; ++j) {
-            const FF fk = sF[j][i];
-#pragma unroll
-            for (int t = 0; t < TPL; ++t) {
-                const int d = LAG * L + 1 + lane + kWarp * t - j;
-                nP[t] = ff_fma(sB[d], fk, nP[t]);
-                nC[t] = ff_fma(sA[d], fk, nC[t]);
-            }
+            const FF fk = m.sF[j][I];
+            const int d = LAG * L + 1 + lane - j;
+            nP = ff_fma(sB[d], fk, nP);
+            nC = ff_fma(sA[d], fk, nC);
         }
     }
+    FF ax(0);
+    if constexpr (Rhs::kForcing) {
+        asm volatile("bar.sync 2, %0;" ::"r"((D + 1) * kWarp) : "memory");
+        ax = m.aux[lane];
+    } else {
+        ax = ff_from_double(Rhs::aux((double)mt * kc.h, in0.p));
+    }
 
-    FF fk = sF[LAG * L][i];
+    FF fk = m.sF[LAG * L][I];
     const int steps = (int)(Nb - m0 < L ? Nb - m0 : L);
+    FF wB = sB[lane + 1], wA = sA[lane + 1];
     for (int s = 0; s < steps; ++s) {
-        // add the newest point k = m0+s to every pending target
+        // the newest point k = m0+s; done targets add B(0) = A(0) = 0
+        nP = ff_fma(wB, fk, nP);
+        nC = ff_fma(wA, fk, nC);
+        const int d = lane - s > 0 ? lane - s : 0;
+        wB = sB[d], wA = sA[d];
+        const FF yp = bP + nP;
+        FF y[D];
+        volatile float *sy = reinterpret_cast<volatile float *>(m.sy[s & 1]);
+        if constexpr (D > 1) {
+            if (lane == s) sy[2 * I] = yp.hi, sy[2 * I + 1] = yp.lo;
+            asm volatile("bar.sync 1, %0;" ::"r"(D * kWarp) : "memory");
 #pragma unroll
-        for (int t = 0; t < TPL; ++t) {
-            const int d = lane + kWarp * t - s + 1;
-            const int dd = d > 0 ? d : 0;  // done targets add B(0) = A(0) = 0
-            nP[t] = ff_fma(sB[dd], fk, nP[t]);
-            nC[t] = ff_fma(sA[dd], fk, nC[t]);
-        }
-        const int owner = s % kWarp, slot = s / kWarp;  // uniform over the CTA
-        FF yp(0), nc(0), bc(0), ax(0);
-#pragma unroll
-        for (int t = 0; t < TPL; ++t)
-            if (t == slot) yp = bP[t] + nP[t], nc = nC[t], bc = bC[t], ax = aux[t];
-        FF fn(0), in(0);
-        if constexpr (D == 1) {
-            if (lane == owner) {
-                const FF fp = Rhs::template one<D>(0, &yp, pf, ax);
-                in = ha_ig2 * fp + nc;
-                const FF yc = bc + in;
-                fn = Rhs::template one<D>(0, &yc, pf, ax);
-            }
+            for (int q = 0; q < D; ++q) y[q] = FF(sy[2 * q], sy[2 * q + 1]);
         } else {
-            if (act && lane == owner) sy[0][i] = yp;
-            __syncthreads();
-            if (lane == owner) {
-                FF y[D];
-#pragma unroll
-                for (int q = 0; q < D; ++q) y[q] = sy[0][q];
-                const FF fp = Rhs::template one<D>(i, y, pf, ax);
-                in = ha_ig2 * fp + nc;  // corrector increment
-                if (act) sy[1][i] = bc + in;
-            }
-            __syncthreads();
-            if (lane == owner) {
-                FF y[D];
-#pragma unroll
-                for (int q = 0; q < D; ++q) y[q] = sy[1][q];
-                fn = Rhs::template one<D>(i, y, pf, ax);
-            }
+            y[0] = shfl_ff(yp, s);
         }
+        const FF nc = shfl_ff(nC, s), bc = shfl_ff(bC, s);
+        const FF axs = Rhs::kForcing ? shfl_ff(ax, s) : ax;
+        const FF fp = Rhs::template one<D>(I, y, pf, axs);
+        const FF in = ha_ig2 * fp + nc;  // corrector increment
+        const FF yc = bc + in;
+        if constexpr (D > 1) {
+            if (lane == 0) sy[2 * D + 2 * I] = yc.hi, sy[2 * D + 2 * I + 1] = yc.lo;
+            asm volatile("bar.sync 1, %0;" ::"r"(D * kWarp) : "memory");
 #pragma unroll
-        for (int t = 0; t < TPL; ++t)
-            if (t == slot && lane == owner) inc[t] = in, fo[t] = fn;
-        fk = shfl_ff(fn, owner);
+            for (int q = 0; q < D; ++q) y[q] = FF(sy[2 * D + 2 * q], sy[2 * D + 2 * q + 1]);
+        } else {
+            y[0] = yc;
+        }
+        fk = Rhs::template one<D>(I, y, pf, axs);
+        if (lane == s) inc = in, fo = fk;
     }
 
     // FP64 corrector update and f of the block's targets, one per lane
-    if (act) {
-        double *Yb = bt.Y + (int64_t)b * (bt.N + 1) * D;
+    if (lane < steps) {
+        const double yc = baseC + ff_to_double(inc);
+        const double fd = ff_to_double(fo);
+        bt.Y[((int64_t)b * (bt.N + 1) + mt) * D + I] = yc;
+        bt.F[mt * bt.ldF + col] = fd;
+        if (bt.Ff) bt.Ff[mt * bt.ldF + col] = (float)fd;  // the fp32 history's input
+        if (!(finite_bits(yc) && finite_bits(fd))) report_nonfinite(bt.status, mt, b);
+    }
+}
+
+// smem: recur_split_smem_floats<D, LAG>() floats, 16-byte aligned; LAG as for
+// recur_block; a CTA of at least recur_split_warps<Rhs, D>() warps.
+template <class Rhs, int D, int LAG = 1>
+__device__ void recur_block_split(const DevBatch &bt, int b, const DevWeights &w,
+                                  const StepConsts &kc, int64_t c, const double *G, float *smem)
+{
+    constexpr int L = kWarp;
+    const SplitMem<D, LAG> m(smem);
+    const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
+    const int64_t m0 = c * L;
+    // every load that does not depend on another one, in flight together
+    const int64_t Nb = bt.N_each[b];
+    const int nW = w.stride ? D : 1;  // one weight set per order
+    const int tid = threadIdx.x, nthr = blockDim.x, nF = (LAG * L + 1) * D;
+    auto weight_index = [&](int j) { return (int64_t)(j / m.W) * w.stride + j % m.W; };
+    auto f_at = [&](int j) {
+        const int64_t row = m0 - LAG * L + j / D;
+        return row >= 0 ? bt.F[row * bt.ldF + (int64_t)b * D + j % D] : 0.0;
+    };
+    double wb[2] = {}, wa[2] = {}, f[2] = {};
 #pragma unroll
-        for (int t = 0; t < TPL; ++t) {
-            const int a = lane + kWarp * t;
-            if (a < steps) {
-                const int64_t mm = m0 + 1 + a;
-                const double yc = baseC[t] + ff_to_double(inc[t]);
-                const double fd = ff_to_double(fo[t]);
-                Yb[mm * D + i] = yc;
-                bt.F[mm * bt.ldF + col] = fd;
-                if (bt.Ff) bt.Ff[mm * bt.ldF + col] = (float)fd;  // the fp32 history's input
-                if (!(finite_bits(yc) && finite_bits(fd))) report_nonfinite(bt.status, mm, b);
-            }
+    for (int u = 0; u < 2; ++u) {
+        const int j = tid + u * nthr;
+        if (j < nW * m.W) wb[u] = w.B[weight_index(j)], wa[u] = w.A[weight_index(j)];
+        if (j < nF) f[u] = f_at(j);
+    }
+    SplitIn in{};
+    if (warp < D) {
+        const int64_t col = (int64_t)b * D + warp;
+#pragma unroll
+        for (int q = 0; q < kMaxParams; ++q) in.p[q] = bt.params[(int64_t)b * kMaxParams + q];
+        in.y0 = bt.y0[col];
+        if (bt.y1) in.y1 = bt.y1[col];
+        in.f0 = bt.F[col];
+        in.wD = w.D[warp * w.stride + m0 + 1 + lane];
+        if (G) in.gP = G[(int64_t)lane * bt.cols + col], in.gC = G[(int64_t)(L + lane) * bt.cols + col];
+    }
+    if (m0 >= Nb) return;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int j = tid + u * nthr;
+        if (j < nW * m.W) {
+            const double hq = pick<D>(kc.h_alpha, j / m.W);
+            m.sB[j] = ff_from_double(hq * wb[u]);
+            m.sA[j] = ff_from_double(hq * wa[u]);
         }
+        if (j < nF) m.sF[j / D][j % D] = ff_from_double(f[u]);
+    }
+    for (int j = tid + 2 * nthr; j < nW * m.W; j += nthr) {  // several orders
+        const double hq = pick<D>(kc.h_alpha, j / m.W);
+        m.sB[j] = ff_from_double(hq * w.B[weight_index(j)]);
+        m.sA[j] = ff_from_double(hq * w.A[weight_index(j)]);
+    }
+    for (int j = tid + 2 * nthr; j < nF; j += nthr) m.sF[j / D][j % D] = ff_from_double(f_at(j));
+    __syncthreads();
+    if (warp < D) {
+        if (D == 1 || warp == 0) split_steps<Rhs, D, LAG, 0>(bt, b, w, kc, c, Nb, in, m);
+        else if (D == 2 || warp == 1) split_steps<Rhs, D, LAG, D >= 2 ? 1 : 0>(bt, b, w, kc, c, Nb, in, m);
+        else if (D == 3 || warp == 2) split_steps<Rhs, D, LAG, D >= 3 ? 2 : 0>(bt, b, w, kc, c, Nb, in, m);
+        else split_steps<Rhs, D, LAG, D >= 4 ? 3 : 0>(bt, b, w, kc, c, Nb, in, m);
+    } else if (Rhs::kForcing && warp == D) {
+        double p[kMaxParams];
+#pragma unroll
+        for (int q = 0; q < kMaxParams; ++q) p[q] = bt.params[(int64_t)b * kMaxParams + q];
+        m.aux[lane] = ff_from_double(Rhs::aux((double)(m0 + 1 + lane) * kc.h, p));
+        asm volatile("bar.sync 2, %0;" ::"r"((D + 1) * kWarp) : "memory");
     }
 }
 

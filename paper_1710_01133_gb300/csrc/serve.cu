@@ -335,14 +335,16 @@ __global__ void combine_slots_kernel(const SlotDev *__restrict__ slots, const in
     }
 }
 
-// One CTA of 4 warps per slot: block cs[slot] of the recurrence (the split
+constexpr int kRecurWarps = FABM_MAX_DIM + 1;  // the components and the forcing
+
+// One CTA per slot: block cs[slot] of the recurrence (the split
 // recurrence for split slots).
-__global__ void __launch_bounds__(kWarp *FABM_MAX_DIM)
+__global__ void __launch_bounds__(kWarp *kRecurWarps)
     recur_slots_kernel(const SlotDev *__restrict__ slots, const int64_t *__restrict__ cs)
 {
-    static_assert(recur_split_smem_floats<FABM_MAX_DIM, 1>() <=
-                  2 * recur_smem_doubles<FABM_MAX_DIM, 1>());
-    __shared__ double smem[recur_smem_doubles<FABM_MAX_DIM, 1>()];
+    constexpr int kDoubles = std::max(recur_smem_doubles<FABM_MAX_DIM, 1>(),
+                                      (recur_split_smem_floats<FABM_MAX_DIM>() + 1) / 2);
+    __shared__ __align__(16) double smem[kDoubles];
     const SlotDev s = slots[blockIdx.x];
     const int64_t c = cs[blockIdx.x];  // the block this step runs; -1: none (new slot)
     if (c < 0) return;
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(kWarp *FABM_MAX_DIM)
     const bool split = s.hk == FABM_HIST_FP32C;
     slot_dispatch(s.rhs, s.dim, [&]<class R, int D>() {
         if (split)
-            recur_block_split<R, D, 1>(bt, 0, w, s.kc, c, G, reinterpret_cast<float *>(smem));
+            recur_block_split<R, D>(bt, 0, w, s.kc, c, G, reinterpret_cast<float *>(smem));
         else
             recur_block<R, D, 1>(bt, 0, w, s.kc, c, G, smem);
     });
@@ -674,7 +676,7 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
         SRV_TRY(cudaGetLastError());
         S->launches += 2;
     }
-    recur_slots_kernel<<<(unsigned)ns, kWarp * FABM_MAX_DIM, 0, S->sR>>>(S->d_slots, S->d_c);
+    recur_slots_kernel<<<(unsigned)ns, kWarp * kRecurWarps, 0, S->sR>>>(S->d_slots, S->d_c);
     SRV_TRY(cudaGetLastError());
     ++S->launches;
     SRV_TRY(cudaStreamSynchronize(S->sG));
