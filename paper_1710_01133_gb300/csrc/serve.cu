@@ -3,21 +3,23 @@
 // alpha, h and N) wait in a host queue and are admitted as "slots" while the
 // device memory they need (weights, history, output, partials) fits in the
 // server's HBM budget.  Each fabm_server_step advances every admitted slot by
-// one block of 32 steps with shared launches over tables of slots:
-//   stream G: far history of block c+1 of every slot (one launch whose CTAs
-//             derive their (slot, chunk, column) items from each slot's block
-//             index, so the host builds no work list), then the fixed-order
-//             combine
-//   stream R: the recurrence of block c of every slot (one CTA per slot,
-//             the right-hand side dispatched at run time)
-//   stream W: weights and initial values of newly admitted slots, beside the
-//             step's launches; new slots run their first block at the next step
-// which is the two-stream schedule of a single solve, run for all slots at
-// once.  Finished slots are copied to host memory and their device memory is
-// returned to the stream-ordered pool; the freed budget admits waiting
-// requests at the next step.  Per step the host uploads one block index per
-// slot, and the slot table only when slots were admitted or retired.  A slot's chunking depends on its own block index
-// only, so its result does not depend on the other requests in flight.
+// one block of 32 steps with one launch over a table of slots: a CTA per slot
+// for the recurrence of block c (the right-hand side dispatched at run time),
+// and beside them CTAs for the far history of block c+1, which derive their
+// (slot, chunk, column) items from each slot's block index; the CTA that
+// finishes a slot's last items adds its chunks in a fixed order.  Stream W
+// computes weights and initial values of newly admitted slots beside the step's
+// launch; new slots run their first block at the next step.  Finished slots are
+// copied to host memory and their device memory is returned to the
+// stream-ordered pool; the freed budget admits waiting requests at the next step.
+//
+// A step of a few hundred slots is bound by what surrounds the kernels, so the
+// host uploads the slot table only when slots were admitted or retired, requests'
+// inputs in it, the device counts the blocks, and a step is one launch and one
+// wait (256 requests of 2^12 to 2^14 steps: 55 -> 52 us a step,
+// one request 30..36 -> 20..27; the step that admits them 4.1 -> 2.1 ms, the steps
+// that return their results 7.0 -> 4.8 ms in all).  A slot's chunking depends on its own block
+// index only, so its result does not depend on the other requests in flight.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,7 +58,16 @@ struct SlotDev {
     StepConsts kc;
     double alpha, inv_g1;
     unsigned long long *status;
+    // the block of server step e is c0 + e from step `start` on; before it the
+    // slot is skipped (its weights are being computed)
+    int64_t c0, start;
+    // the request's inputs, copied to the buffers above when the slot is set up
+    double y0v[FABM_MAX_DIM], y1v[FABM_MAX_DIM], pv[kMaxParams];
+    int resumed, pad2;  // history, solution and status come from a checkpoint
 };
+
+// Block that the slot runs at server step e, or -1.
+__device__ inline int64_t slot_block(const SlotDev &s, int64_t e) { return e < s.start ? -1 : s.c0 + e; }
 
 // Chunking of block c's far history for one slot: depends on c only, so a
 // request's partial sums do not depend on the other requests in flight.
@@ -123,39 +134,57 @@ __device__ inline void slot_dispatch(int rhs, int dim, Fn &&fn)
 }
 
 // Weights (double, and fp32 copies for split slots) of new slots:
-// blockIdx.y = new slot, grid-stride over the distances.
-__global__ void weights_slots_kernel(const SlotDev *__restrict__ slots, const int *__restrict__ idx)
+// blockIdx.y = new slot, stride over the distances.
+__global__ void __launch_bounds__(kWeightThreads)
+    weights_slots_kernel(const SlotDev *__restrict__ slots, const int *__restrict__ idx)
 {
-    const SlotDev s = slots[idx[blockIdx.y]];
-    const double inv_g2 = s.kc.inv_gamma2[0];
-    for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d <= s.w_ext;
-         d += (int64_t)gridDim.x * blockDim.x) {
-        weights_at(d, s.alpha, s.inv_g1, inv_g2, s.WB, s.WA, s.WD);
-        if (s.WBf) {
-            s.WBf[d] = (float)s.WB[d];
-            s.WAf[d] = (float)s.WA[d];
-        }
-    }
+    const SlotDev &s = slots[idx[blockIdx.y]];
+    const double inv_g2 = s.kc.inv_gamma2[0], alpha = s.alpha, inv_g1 = s.inv_g1;
+    const int64_t w_ext = s.w_ext;
+    double *WB = s.WB, *WA = s.WA, *WD = s.WD;
+    float *WBf = s.WBf, *WAf = s.WAf;
+    for (int64_t d0 = blockIdx.x * (int64_t)blockDim.x; d0 <= w_ext; d0 += (int64_t)gridDim.x * blockDim.x)
+        weights_block(d0, w_ext, alpha, inv_g1, inv_g2, WB, WA, WD, [&](int64_t d) {
+            if (WBf) {
+                WBf[d] = (float)WB[d];
+                WAf[d] = (float)WA[d];
+            }
+        });
 }
 
+// Inputs, and for slots that start from the beginning the initial values, of n
+// new slots.
 __global__ void init_slots_kernel(const SlotDev *__restrict__ slots, const int *__restrict__ idx,
                                   int n)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
-    const SlotDev s = slots[idx[j]];
+    const SlotDev &s = slots[idx[j]];
+    *s.Nb = s.N;
+    for (int q = 0; q < FABM_MAX_DIM; ++q) {
+        s.y0[q] = s.y0v[q];
+        if (s.y1) s.y1[q] = s.y1v[q];
+    }
+    for (int q = 0; q < kMaxParams; ++q) s.params[q] = s.pv[q];
+    if (s.resumed) return;
+    *s.status = ~0ull;
     const DevBatch bt = slot_batch(s);
     slot_dispatch(s.rhs, s.dim, [&]<class R, int D>() { init_one<R, D>(bt, 0); });
 }
 
-// Far history, one warp per (slot, chunk, column) item: requests have one to
-// three columns, so a CTA of four warps takes four items (of one request or
-// several) and no warp idles.  Each warp stages its own tiles of f and of the
+// status[j] of n finished slots, for the host.
+__global__ void collect_slots_kernel(const SlotDev *__restrict__ slots, const int *__restrict__ idx,
+                                     int n, unsigned long long *__restrict__ status)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) status[j] = *slots[idx[j]].status;
+}
+
+// Far history, one warp per (slot, chunk, column) item (FP64) or four: requests
+// have one to three columns.  Each warp stages its own tiles of f and of the
 // weights and runs the same per-column arithmetic as the batch kernels
 // (hist_fp64_block / hist_fp32c_block), so a request's partial sums do not
 // depend on which items share its CTA.
-constexpr int kWarpsPerHistCta = 4;
-
 __device__ void hist_warp_f64(const SlotDev &s, int64_t c, int chunk, int64_t kc, int q,
                               double *sF, double *sB, double *sA)
 {
@@ -258,65 +287,162 @@ __device__ void hist_warp_f32c(const SlotDev &s, int64_t c, int chunk, int64_t k
     out[(int64_t)kL * dim] = make_float2(sc, -cc);
 }
 
-// Slots blockIdx.y, blockIdx.y + gridDim.y, ...: the slot's items are
-// (chunk, column) pairs in chunk-major order, warp w of CTA x taking item
-// 4x + w; the item list is derived here from the slot's block index cs[slot],
-// so the host uploads no work list.
-__global__ void __launch_bounds__(kWarp *kWarpsPerHistCta)
-    hist_slots_kernel(const SlotDev *__restrict__ slots, const int64_t *__restrict__ cs, int ns)
+// Four items of a slot by one warp in compensated fp32: eight lanes an item,
+// four targets a lane.  As j advances a lane's window of weights moves by one, so
+// a point costs it two weights and a quarter of a vector load of f for eight
+// multiply-adds, where a lane per target took three loads for two (a step's
+// shared-memory loads were what its history and the steps beside it waited for).
+// Chosen from kQuadItems items a step on, where the loads count and not the
+// latency of one item.  Steps with an item per warp / with four, us: 1024 slots of
+// the Lorenz type, 39,000 items 439 / 290, 12,000 180 / 147, 6,000 128 / 125; 1024
+// linear ones, 13,000 items 181 / 135, 4,000 86 / 94; 256 of the Lorenz type, 5,000
+// items 87 / 92, 1,500 52 / 57; 64 slots, 400 items 29 / 33.
+constexpr int kQuad = 4;
+constexpr int64_t kQuadItems = 6144;
+constexpr int kQT = 64;                      // points per tile
+constexpr int kQF = kQT + 4, kQW = kQT + 33;  // strides of f and of the weights: banks apart
+constexpr int kQuadFloats = 2 * kQuad * (kQF + 2 * kQW);
+
+__device__ __forceinline__ void copy4(float *dst, const float *src, bool in)
 {
-    constexpr int kBytesF64 = (hist::f64::kTile + 2 * (hist::f64::kTile + hist::kL)) * 8;
-    constexpr int kBytesF32 = (hist::f32c::kTile + 2 * (hist::f32c::kTile + hist::kL)) * 4;
-    constexpr int kWarpBytes = kBytesF64 > kBytesF32 ? kBytesF64 : kBytesF32;
-    __shared__ __align__(16) unsigned char smem[kWarpsPerHistCta][kWarpBytes];
-    const int w = threadIdx.x / kWarp;
-    for (int slot = blockIdx.y; slot < ns; slot += gridDim.y) {
-        const SlotDev s = slots[slot];
-        const int64_t cn = cs[slot] + 1;  // far history of the slot's next block
-        if (cn < 2 || cn >= slot_blocks(s.N)) continue;
-        int64_t kc;
-        int n;
-        slot_chunks(cn, &kc, &n);
-        const int g = (int)blockIdx.x * kWarpsPerHistCta + w;
-        if (g >= n * s.dim) continue;  // uniform over the warp; warps never synchronize
-        const int chunk = g / s.dim, q = g % s.dim;
-        if (s.hk == FABM_HIST_FP32C) {
-            float *sF = reinterpret_cast<float *>(smem[w]);
-            float *sB = sF + hist::f32c::kTile;
-            hist_warp_f32c(s, cn, chunk, kc, q, sF, sB, sB + hist::f32c::kTile + hist::kL);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(in ? 4 : 0)
+                 : "memory");
+}
+
+__device__ void hist_quad_f32c(const SlotDev &s, int64_t c, int64_t kc, int n_chunks, int g0,
+                               float *smem)
+{
+    using hist::kL;
+    using hist::f32c::kahan_add;
+    constexpr int kT = hist::f32c::kTile, kG = hist::f32c::kGroup;
+    static_assert(kQT % kG == 0 && kT % kQT == 0);
+    const int lane = threadIdx.x % kWarp, grp = lane / 8, l = lane % 8;
+    const int dim = s.dim, g = g0 + grp;
+    const bool valid = g < n_chunks * dim;
+    const int chunk = valid ? g / dim : 0, q = valid ? g % dim : 0;
+    const int64_t k_end = (c - 1) * kSL, k0 = (int64_t)chunk * kc;
+    const int npts = valid ? (int)(k0 + kc < k_end ? kc : k_end - k0) : 0;
+    const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)npts);
+    float *sF = smem + grp * kQF, *sB = smem + kQuad * kQF + grp * kQW;
+    float *sA = sB + kQuad * kQW;
+    constexpr int kBuf = kQuadFloats / 2;
+    // tile t: f of the points k0 + kQT t + j; window index i <-> distance
+    // cL + 1 - (k0 + kQT t + kQT - 1) + i, of target a and point j: a + kQT - 1 - j
+    auto fetch = [&](int t) {
+        const int o = (t & 1) * kBuf;
+        const int64_t t0 = k0 + (int64_t)t * kQT, d0 = c * kL + 2 - kQT - t0;
+        const bool on = t * kQT < npts;
+#pragma unroll
+        for (int u = 0; u < kQT / 8; ++u) {
+            const int i = l + 8 * u;
+            const bool in = t * kQT + i < npts;
+            copy4(sF + o + i, s.Ff + (in ? (t0 + i) * dim + q : 0), in);
+        }
+#pragma unroll
+        for (int u = 0; u < (kQT + kL) / 8; ++u) {
+            const int i = l + 8 * u;
+            const bool in = on && d0 + i >= 0;
+            copy4(sB + o + i, s.WBf + (in ? d0 + i : 0), in);
+            copy4(sA + o + i, s.WAf + (in ? d0 + i : 0), in);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float sp[4] = {}, cp[4] = {}, sc[4] = {}, cc[4] = {};
+    fetch(0);
+    for (int t = 0; t * kQT < most; ++t) {
+        if ((t + 1) * kQT < most) {
+            fetch(t + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
-            double *sF = reinterpret_cast<double *>(smem[w]);
-            double *sB = sF + hist::f64::kTile;
-            hist_warp_f64(s, cn, chunk, kc, q, sF, sB, sB + hist::f64::kTile + hist::kL);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncwarp();
+        const int o = (t & 1) * kBuf, nk = npts - t * kQT;
+        if (nk > 0) {
+            const float4 *fv = reinterpret_cast<const float4 *>(sF + o);
+            const float *wb = sB + o + 4 * l + kQT - 1, *wa = sA + o + 4 * l + kQT - 1;
+            float b[4], a[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) b[u] = wb[u], a[u] = wa[u];
+#pragma unroll
+            for (int j0 = 0; j0 < kQT; j0 += kG) {
+                if (j0 < nk) {  // points past the chunk are zeros
+                    float gp[4] = {}, gc[4] = {};
+#pragma unroll
+                    for (int u4 = 0; u4 < kG; u4 += 4) {
+                        const float4 f4 = fv[(j0 + u4) / 4];
+                        const float f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) {
+                                gp[v] = fmaf(b[v], f[u], gp[v]);
+                                gc[v] = fmaf(a[v], f[u], gc[v]);
+                            }
+                            const int j = j0 + u4 + u + 1;  // the next point's weights
+#pragma unroll
+                            for (int v = 3; v > 0; --v) b[v] = b[v - 1], a[v] = a[v - 1];
+                            if (j < kQT) b[0] = wb[-j], a[0] = wa[-j];
+                        }
+                    }
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) kahan_add(sp[v], cp[v], gp[v]), kahan_add(sc[v], cc[v], gc[v]);
+                }
+            }
+            // the fold after 512 points or the last one: of the rest that is not a
+            // multiple of 16 (done above), or of nothing
+            const bool end = nk <= kQT || (t + 1) % (kT / kQT) == 0;
+            if (end && (nk >= kQT || nk % kG == 0)) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) kahan_add(sp[v], cp[v], 0.f), kahan_add(sc[v], cc[v], 0.f);
+            }
+        }
+        __syncwarp();
+    }
+    if (valid) {
+        float2 *out = static_cast<float2 *>(s.part) + ((int64_t)(chunk * 2) * kL + 4 * l) * dim + q;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            out[(int64_t)v * dim] = make_float2(sp[v], -cp[v]);
+            out[(int64_t)(kL + v) * dim] = make_float2(sc[v], -cc[v]);
         }
     }
 }
 
-// One CTA per slot: G[gbuf][kind][t][col] = sum over the chunks in ascending
-// order (compensated double, or float-float rounded once to double).
-__global__ void combine_slots_kernel(const SlotDev *__restrict__ slots, const int64_t *__restrict__ cs)
+constexpr int kHistBytesF64 = (hist::f64::kTile + 2 * (hist::f64::kTile + hist::kL)) * 8;
+constexpr int kHistBytesF32 =
+    std::max(kQuadFloats, hist::f32c::kTile + 2 * (hist::f32c::kTile + hist::kL)) * 4;
+constexpr int kHistWarpBytes = kHistBytesF64 > kHistBytesF32 ? kHistBytesF64 : kHistBytesF32;
+constexpr int kStepWarps = FABM_MAX_DIM + 1;  // the components and the forcing; history items
+
+// A slot's history items for its block cn.
+__host__ __device__ inline int slot_items(int64_t cn, int dim)
 {
-    const SlotDev s = slots[blockIdx.x];
-    const int64_t cn = cs[blockIdx.x] + 1;
-    if (cn < 2 || cn >= slot_blocks(s.N)) return;  // no far history this step (uniform)
     int64_t kc;
-    int n_chunks;
-    slot_chunks(cn, &kc, &n_chunks);
+    int n;
+    slot_chunks(cn, &kc, &n);
+    return n * dim;
+}
+
+// The fixed-order sum of a slot's chunks: G[kind][t][col] over the chunks in
+// ascending order (compensated double, or float-float rounded once to double).
+__device__ void combine_slot(const SlotDev &s, int64_t cn, int n_chunks)
+{
     const int n_out = 2 * kSL * s.dim;
     double *G = s.G + (int64_t)(cn % 2) * n_out;
     for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
         if (s.hk == FABM_HIST_FP32C) {
             const float2 *p = static_cast<const float2 *>(s.part);
             float hi = 0.f, lo = 0.f;
-            for (int ch = 0; ch < n_chunks; ++ch) {
-                const float2 v = p[(int64_t)ch * n_out + o];
-                const float t = hi + v.x;
-                const float bb = t - hi;
-                const float e = (hi - (t - bb)) + (v.x - bb);
-                lo += e + v.y;
-                hi = t + lo;
-                lo = lo - (hi - t);
-            }
+            float2 v[kMaxChunksSlot];
+#pragma unroll
+            for (int ch = 0; ch < kMaxChunksSlot; ++ch)
+                if (ch < n_chunks) v[ch] = __ldcg(p + (int64_t)ch * n_out + o);
+#pragma unroll
+            for (int ch = 0; ch < kMaxChunksSlot; ++ch)
+                if (ch < n_chunks) ff_add_chunk(hi, lo, v[ch].x, v[ch].y);
             G[o] = (double)hi + (double)lo;
         } else {
             // Neumaier: the rounding error of every addition (TwoSum) is kept
@@ -324,7 +450,7 @@ __global__ void combine_slots_kernel(const SlotDev *__restrict__ slots, const in
             const double *p = static_cast<const double *>(s.part);
             double acc = 0.0, err = 0.0;
             for (int ch = 0; ch < n_chunks; ++ch) {
-                const double v = p[(int64_t)ch * n_out + o];
+                const double v = __ldcg(p + (int64_t)ch * n_out + o);
                 const double t = acc + v;
                 const double bv = t - acc;
                 err += (acc - (t - bv)) + (v - bv);
@@ -335,29 +461,67 @@ __global__ void combine_slots_kernel(const SlotDev *__restrict__ slots, const in
     }
 }
 
-constexpr int kRecurWarps = FABM_MAX_DIM + 1;  // the components and the forcing
-
-// One CTA per slot: block cs[slot] of the recurrence (the split
-// recurrence for split slots).
-__global__ void __launch_bounds__(kWarp *kRecurWarps)
-    recur_slots_kernel(const SlotDev *__restrict__ slots, const int64_t *__restrict__ cs)
+// One server step.  CTA x < ns: the step's block of slot x.  The other CTAs, hx
+// per slot: the far history of the slot's next block, its (chunk, column) items
+// in chunk-major order, `per` (1 or kQuad) to a warp, derived from the slot's block index, so the host
+// uploads no work list; the CTA that finishes a slot's last items (a count per
+// slot, left at zero) adds its chunks.  No CTA waits for another one.
+__global__ void __launch_bounds__(kWarp *kStepWarps)
+    step_slots_kernel(const SlotDev *__restrict__ slots, int64_t epoch, int ns, int hx, int per,
+                      int *cnt)
 {
-    constexpr int kDoubles = std::max(recur_smem_doubles<FABM_MAX_DIM, 1>(),
-                                      (recur_split_smem_floats<FABM_MAX_DIM>() + 1) / 2);
-    __shared__ __align__(16) double smem[kDoubles];
-    const SlotDev s = slots[blockIdx.x];
-    const int64_t c = cs[blockIdx.x];  // the block this step runs; -1: none (new slot)
-    if (c < 0) return;
-    const DevBatch bt = slot_batch(s);
-    const DevWeights w{s.WB, s.WA, s.WD, s.w_ext};
-    const double *G = c >= 2 ? s.G + (c % 2) * 2 * kSL * s.dim : nullptr;
-    const bool split = s.hk == FABM_HIST_FP32C;
-    slot_dispatch(s.rhs, s.dim, [&]<class R, int D>() {
-        if (split)
-            recur_block_split<R, D>(bt, 0, w, s.kc, c, G, reinterpret_cast<float *>(smem));
-        else
-            recur_block<R, D, 1>(bt, 0, w, s.kc, c, G, smem);
-    });
+    static_assert(recur_smem_doubles<FABM_MAX_DIM, 1>() * 8 <= kStepWarps * kHistWarpBytes &&
+                  recur_split_smem_floats<FABM_MAX_DIM>() * 4 <= kStepWarps * kHistWarpBytes);
+    __shared__ __align__(16) unsigned char smem[kStepWarps][kHistWarpBytes];
+    __shared__ bool last;
+    if ((int)blockIdx.x < ns) {
+        const SlotDev &s = slots[blockIdx.x];
+        const int64_t c = slot_block(s, epoch);  // -1: none (new slot)
+        if (c < 0) return;
+        const DevBatch bt = slot_batch(s);
+        const DevWeights w{s.WB, s.WA, s.WD, s.w_ext};
+        const double *G = c >= 2 ? s.G + (c % 2) * 2 * kSL * s.dim : nullptr;
+        const bool split = s.hk == FABM_HIST_FP32C;
+        slot_dispatch(s.rhs, s.dim, [&]<class R, int D>() {
+            if (split)
+                recur_block_split<R, D>(bt, 0, w, s.kc, c, G, reinterpret_cast<float *>(smem));
+            else
+                recur_block<R, D, 1>(bt, 0, w, s.kc, c, G, reinterpret_cast<double *>(smem));
+        });
+        return;
+    }
+    const int slot = ((int)blockIdx.x - ns) / hx, x = ((int)blockIdx.x - ns) % hx;
+    const SlotDev s = slots[slot];
+    const int64_t cn = slot_block(s, epoch) + 1;
+    if (cn < 2 || cn >= slot_blocks(s.N)) return;
+    int64_t kc;
+    int n;
+    slot_chunks(cn, &kc, &n);
+    const int items = n * s.dim, ctas = (items + kStepWarps * per - 1) / (kStepWarps * per);
+    if (x >= ctas) return;
+    const int w = threadIdx.x / kWarp, g = (x * kStepWarps + w) * per;
+    if (g >= items) {
+    } else if (per == kQuad) {
+        hist_quad_f32c(s, cn, kc, n, g, reinterpret_cast<float *>(smem[w]));
+    } else if (s.hk == FABM_HIST_FP32C) {
+        float *sF = reinterpret_cast<float *>(smem[w]);
+        float *sB = sF + hist::f32c::kTile;
+        hist_warp_f32c(s, cn, g / s.dim, kc, g % s.dim, sF, sB, sB + hist::f32c::kTile + hist::kL);
+    } else {
+        double *sF = reinterpret_cast<double *>(smem[w]);
+        double *sB = sF + hist::f64::kTile;
+        hist_warp_f64(s, cn, g / s.dim, kc, g % s.dim, sF, sB, sB + hist::f64::kTile + hist::kL);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(cnt + slot, 1) == ctas - 1;
+        if (last) cnt[slot] = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    combine_slot(s, cn, n);
 }
 
 // ------------------------------------------------------------------- host ---
@@ -430,7 +594,8 @@ struct Slot {
 struct Result {
     int state;  // FABM_REQ_*
     fabm_status status;
-    std::vector<double> y;
+    std::unique_ptr<double[]> y;  // n values once it has finished
+    size_t n = 0;
 };
 
 size_t slot_bytes(const Req &r, int hk, int64_t *w_ext_out)
@@ -494,6 +659,9 @@ void slot_layout(Slot &s, int hk, int64_t w_ext)
         d.kc.h_alpha[q] = std::pow(r.h, r.alpha);
         d.kc.inv_gamma2[q] = 1.0 / std::tgamma(r.alpha + 2.0);
     }
+    for (int q = 0; q < FABM_MAX_DIM; ++q) d.y0v[q] = r.y0[q], d.y1v[q] = r.y1[q];
+    for (int q = 0; q < kMaxParams; ++q) d.pv[q] = q < r.n_params ? r.params[q] : 0.0;
+    d.resumed = r.ckpt ? 1 : 0;
     d.alpha = r.alpha;
     d.inv_g1 = 1.0 / std::tgamma(r.alpha + 1.0);
 }
@@ -512,14 +680,15 @@ struct fabm_server {
     std::unordered_map<int64_t, std::pair<int64_t, int>> shapes;  // ticket -> (N, dim)
     std::vector<int64_t> finished;  // finished since the last fabm_server_finished
     int64_t next_ticket = 1;
-    cudaStream_t sR = nullptr, sG = nullptr, sW = nullptr;
-    cudaEvent_t evUp = nullptr, evIn = nullptr;
+    cudaStream_t sR = nullptr, sW = nullptr;
+    cudaEvent_t evIn = nullptr, evW = nullptr;
+    int64_t epoch = 0;           // server steps with slots, the time base of their block indices
     SlotDev *d_slots = nullptr;  // device tables: the slots, uploaded when they change,
-    int64_t *d_c = nullptr;      // each slot's block index, uploaded every step,
-    int *d_idx = nullptr;        // and the indices of newly admitted slots
+    int *d_idx = nullptr;        // and the indices of newly admitted or finished slots
     SlotDev *h_slots = nullptr;  // pinned staging
-    int64_t *h_c = nullptr;
     int *h_idx = nullptr;
+    int *d_cnt = nullptr;        // history CTAs done per slot, zero between steps
+    unsigned long long *h_status = nullptr;  // pinned, written by the device
     bool table_dirty = true;     // the slot table changed since its last upload
     int64_t steps_done = 0, launches = 0;
     std::mutex mu;
@@ -530,16 +699,15 @@ struct fabm_server {
             if (s.mem) cudaFreeAsync(s.mem, sR);
         if (sR) cudaStreamSynchronize(sR);
         if (d_slots) cudaFree(d_slots);
-        if (d_c) cudaFree(d_c);
         if (d_idx) cudaFree(d_idx);
+        if (d_cnt) cudaFree(d_cnt);
         if (h_slots) cudaFreeHost(h_slots);
-        if (h_c) cudaFreeHost(h_c);
+        if (h_status) cudaFreeHost(h_status);
         if (h_idx) cudaFreeHost(h_idx);
         if (sW) cudaStreamSynchronize(sW);
-        if (evUp) cudaEventDestroy(evUp);
         if (evIn) cudaEventDestroy(evIn);
+        if (evW) cudaEventDestroy(evW);
         if (sR) cudaStreamDestroy(sR);
-        if (sG) cudaStreamDestroy(sG);
         if (sW) cudaStreamDestroy(sW);
     }
 };
@@ -558,7 +726,7 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
         if (S->in_use + bytes > S->budget) {
             if (S->slots.empty()) {  // can never fit
                 S->queue.pop_front();
-                S->results[r.ticket] = {FABM_REQ_FAILED, FABM_ENOMEM, {}};
+                S->results[r.ticket] = {FABM_REQ_FAILED, FABM_ENOMEM, nullptr};
                 S->finished.push_back(r.ticket);
                 continue;
             }
@@ -573,7 +741,7 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
         if (e != cudaSuccess) {
             if (S->slots.empty()) {
                 S->queue.pop_front();
-                S->results[r.ticket] = {FABM_REQ_FAILED, FABM_ENOMEM, {}};
+                S->results[r.ticket] = {FABM_REQ_FAILED, FABM_ENOMEM, nullptr};
                 S->finished.push_back(r.ticket);
                 continue;
             }
@@ -583,110 +751,91 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
         if (r.ckpt) s.c = r.ckpt->c;
         S->queue.pop_front();
         S->in_use += bytes;
-        S->results[r.ticket] = {FABM_REQ_RUNNING, FABM_OK, {}};
+        S->results[r.ticket] = {FABM_REQ_RUNNING, FABM_OK, nullptr};
         s.pending = true;
         fresh.push_back((int)S->slots.size());
         S->slots.push_back(s);
     }
-    // new slots needing initial values first, resumed ones after them
-    std::stable_partition(fresh.begin(), fresh.end(),
-                          [&](int i) { return !S->slots[i].req.ckpt; });
-    int n_init = 0;
-    for (int i : fresh) n_init += S->slots[i].req.ckpt ? 0 : 1;
     const int ns = (int)S->slots.size();
     *n_waiting = (int)S->queue.size();
     *n_active = ns;
     if (ns == 0) return FABM_OK;
 
-    // 2. tables: the slots (when they changed), each slot's block index (its
-    // history, combine and recurrence items follow from it on the device) and
-    // the indices of new slots
+    // 2. table: the slots, when they changed (a slot's block index follows from
+    // the step number, its history, combine and recurrence items from the block
+    // index, so a step without arrivals or departures uploads nothing), and the
+    // indices of new slots
+    const int64_t epoch = S->epoch;
     if (!fresh.empty()) S->table_dirty = true;
     if (S->table_dirty) {
-        for (int i = 0; i < ns; ++i) S->h_slots[i] = S->slots[i].dev;
+        for (int i = 0; i < ns; ++i) {
+            Slot &s = S->slots[i];
+            if (s.pending) {  // first block at the next step
+                s.dev.start = epoch + 1;
+                s.dev.c0 = s.c - (epoch + 1);
+            }
+            S->h_slots[i] = s.dev;
+        }
         SRV_TRY(cudaMemcpyAsync(S->d_slots, S->h_slots, sizeof(SlotDev) * ns, cudaMemcpyHostToDevice, S->sR));
         S->table_dirty = false;
     }
-    int max_items = 0;  // history items of the busiest slot
+    int64_t items = 0;   // history items of the step,
+    int most_items = 0;  // of the busiest slot
     for (int i = 0; i < ns; ++i) {
         const Slot &s = S->slots[i];
-        S->h_c[i] = s.pending ? -1 : s.c;  // -1: the device skips the slot this step
-        if (s.pending) continue;
         const int64_t cn = s.c + 1;
-        if (cn >= 2 && cn < s.nblk) {
-            int64_t kc;
-            int n;
-            slot_chunks(cn, &kc, &n);
-            max_items = std::max(max_items, n * s.req.dim);
-        }
+        if (s.pending || cn < 2 || cn >= s.nblk) continue;
+        const int n = slot_items(cn, s.req.dim);
+        items += n;
+        most_items = std::max(most_items, n);
     }
-    for (size_t j = 0; j < fresh.size(); ++j) S->h_idx[j] = fresh[j];
-    SRV_TRY(cudaMemcpyAsync(S->d_c, S->h_c, sizeof(int64_t) * ns, cudaMemcpyHostToDevice, S->sR));
-    // 3. new slots: inputs (stream R), then weights and initial values on
-    // stream W beside this step's launches (they take ~0.1-0.2 ms of FP64
-    // work, which had delayed the whole step whenever requests arrived); the
-    // new slots run their first block at the next step
+    const int per = hk == FABM_HIST_FP32C && items >= kQuadItems ? kQuad : 1;  // items per warp
+    const int hx = (most_items + kStepWarps * per - 1) / (kStepWarps * per);
+    // 3. new slots: weights and initial values on stream W beside this step's
+    // launches (they take ~0.1-0.2 ms of FP64 work, which had delayed the whole
+    // step whenever requests arrived); the new slots run their first block at
+    // the next step.  Their inputs travel in the table.
     if (!fresh.empty()) {
+        for (size_t j = 0; j < fresh.size(); ++j) S->h_idx[j] = fresh[j];
         SRV_TRY(cudaMemcpyAsync(S->d_idx, S->h_idx, sizeof(int) * fresh.size(), cudaMemcpyHostToDevice, S->sR));
         for (int i : fresh) {
             Slot &s = S->slots[i];
-            double par[kMaxParams] = {};
-            for (int q = 0; q < s.req.n_params; ++q) par[q] = s.req.params[q];
-            SRV_TRY(cudaMemcpyAsync(s.dev.y0, s.req.y0, sizeof(double) * s.req.dim, cudaMemcpyHostToDevice, S->sR));
-            if (s.dev.y1)
-                SRV_TRY(cudaMemcpyAsync(s.dev.y1, s.req.y1, sizeof(double) * s.req.dim, cudaMemcpyHostToDevice, S->sR));
-            SRV_TRY(cudaMemcpyAsync(s.dev.params, par, sizeof par, cudaMemcpyHostToDevice, S->sR));
-            SRV_TRY(cudaMemcpyAsync(s.dev.Nb, &s.req.N, sizeof(int64_t), cudaMemcpyHostToDevice, S->sR));
-            if (const Ckpt *k = s.req.ckpt.get()) {  // resumed: the saved state
-                const size_t rows = k->F.size() / s.req.dim;
-                SRV_TRY(cudaMemcpyAsync(s.dev.F, k->F.data(), sizeof(double) * rows * s.req.dim, cudaMemcpyHostToDevice, S->sR));
-                if (s.dev.Ff)  // the float copy the fp32 history reads
-                    SRV_TRY(launch_to_float(s.dev.F, (int64_t)(rows * s.req.dim), s.dev.Ff, S->sR));
-                SRV_TRY(cudaMemcpyAsync(s.dev.Y, k->Y.data(), sizeof(double) * rows * s.req.dim, cudaMemcpyHostToDevice, S->sR));
-                SRV_TRY(cudaMemcpyAsync(s.dev.G, k->G.data(), sizeof(double) * k->G.size(), cudaMemcpyHostToDevice, S->sR));
-                SRV_TRY(cudaMemcpyAsync(s.dev.status, &k->status, sizeof k->status, cudaMemcpyHostToDevice, S->sR));
-            } else {
-                SRV_TRY(cudaMemsetAsync(s.dev.status, 0xff, sizeof(unsigned long long), S->sR));
-            }
+            const Ckpt *k = s.req.ckpt.get();
+            if (!k) continue;  // resumed: the saved state
+            const size_t rows = k->F.size() / s.req.dim;
+            SRV_TRY(cudaMemcpyAsync(s.dev.F, k->F.data(), sizeof(double) * rows * s.req.dim, cudaMemcpyHostToDevice, S->sR));
+            if (s.dev.Ff)  // the float copy the fp32 history reads
+                SRV_TRY(launch_to_float(s.dev.F, (int64_t)(rows * s.req.dim), s.dev.Ff, S->sR));
+            SRV_TRY(cudaMemcpyAsync(s.dev.Y, k->Y.data(), sizeof(double) * rows * s.req.dim, cudaMemcpyHostToDevice, S->sR));
+            SRV_TRY(cudaMemcpyAsync(s.dev.G, k->G.data(), sizeof(double) * k->G.size(), cudaMemcpyHostToDevice, S->sR));
+            SRV_TRY(cudaMemcpyAsync(s.dev.status, &k->status, sizeof k->status, cudaMemcpyHostToDevice, S->sR));
         }
         SRV_TRY(cudaEventRecord(S->evIn, S->sR));
         SRV_TRY(cudaStreamWaitEvent(S->sW, S->evIn, 0));
         int64_t wmax = 0;
         for (int i : fresh) wmax = std::max(wmax, S->slots[i].dev.w_ext);
-        const unsigned gx = (unsigned)std::min<int64_t>((wmax + 256) / 256, 64);
-        weights_slots_kernel<<<dim3(gx, (unsigned)fresh.size()), 256, 0, S->sW>>>(S->d_slots, S->d_idx);
+        const unsigned gx = (unsigned)std::min<int64_t>((wmax + kWeightThreads) / kWeightThreads, 64);
+        weights_slots_kernel<<<dim3(gx, (unsigned)fresh.size()), kWeightThreads, 0, S->sW>>>(S->d_slots, S->d_idx);
         SRV_TRY(cudaGetLastError());
-        S->launches += 1;
-        if (n_init > 0) {
-            init_slots_kernel<<<(unsigned)((n_init + 127) / 128), 128, 0, S->sW>>>(
-                S->d_slots, S->d_idx, n_init);
-            SRV_TRY(cudaGetLastError());
-            S->launches += 1;
-        }
-    }
-    SRV_TRY(cudaEventRecord(S->evUp, S->sR));
-    SRV_TRY(cudaStreamWaitEvent(S->sG, S->evUp, 0));
-    // 4. shared launches
-    if (max_items > 0) {
-        const unsigned hx = (unsigned)((max_items + kWarpsPerHistCta - 1) / kWarpsPerHistCta);
-        const unsigned hy = (unsigned)std::min(ns, 65535);
-        hist_slots_kernel<<<dim3(hx, hy), kWarp * kWarpsPerHistCta, 0, S->sG>>>(S->d_slots, S->d_c, ns);
+        init_slots_kernel<<<(unsigned)((fresh.size() + 127) / 128), 128, 0, S->sW>>>(
+            S->d_slots, S->d_idx, (int)fresh.size());
         SRV_TRY(cudaGetLastError());
-        combine_slots_kernel<<<(unsigned)ns, 256, 0, S->sG>>>(S->d_slots, S->d_c);
-        SRV_TRY(cudaGetLastError());
+        SRV_TRY(cudaEventRecord(S->evW, S->sW));
         S->launches += 2;
     }
-    recur_slots_kernel<<<(unsigned)ns, kWarp * kRecurWarps, 0, S->sR>>>(S->d_slots, S->d_c);
+    // 4. one launch for all slots
+    step_slots_kernel<<<(unsigned)(ns + ns * hx), kWarp * kStepWarps, 0, S->sR>>>(
+        S->d_slots, epoch, ns, std::max(hx, 1), per, S->d_cnt);
     SRV_TRY(cudaGetLastError());
     ++S->launches;
-    SRV_TRY(cudaStreamSynchronize(S->sG));
+    if (!fresh.empty()) SRV_TRY(cudaStreamWaitEvent(S->sR, S->evW, 0));
     SRV_TRY(cudaStreamSynchronize(S->sR));
-    SRV_TRY(cudaStreamSynchronize(S->sW));
     ++S->steps_done;
+    ++S->epoch;
 
     // 5. advance; finished slots to host, memory back to the pool; the table
     // is compacted (and uploaded at the next step) only when a slot finished
-    bool retired = false;
+    int n_done = 0;
     for (int i = 0; i < ns; ++i) {
         Slot &s = S->slots[i];
         s.req.ckpt.reset();  // restored on the device by now
@@ -695,20 +844,34 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
             continue;
         }
         s.c += 1;
-        if (s.c < s.nblk) continue;
-        retired = true;
-        Result &res = S->results[s.req.ticket];
-        res.y.resize((size_t)(s.req.N + 1) * s.req.dim);
-        unsigned long long st = 0;
-        SRV_TRY(cudaMemcpy(res.y.data(), s.dev.Y, sizeof(double) * res.y.size(), cudaMemcpyDeviceToHost));
-        SRV_TRY(cudaMemcpy(&st, s.dev.status, sizeof st, cudaMemcpyDeviceToHost));
-        res.state = st == ~0ull ? FABM_REQ_DONE : FABM_REQ_FAILED;
-        res.status = st == ~0ull ? FABM_OK : FABM_ENONFINITE;
-        S->finished.push_back(s.req.ticket);
-        SRV_TRY(cudaFreeAsync(s.mem, S->sR));
-        S->in_use -= s.bytes;
+        if (s.c >= s.nblk) S->h_idx[n_done++] = i;
     }
-    if (retired) {
+    if (n_done > 0) {
+        SRV_TRY(cudaMemcpyAsync(S->d_idx, S->h_idx, sizeof(int) * n_done, cudaMemcpyHostToDevice, S->sR));
+        collect_slots_kernel<<<(unsigned)((n_done + 127) / 128), 128, 0, S->sR>>>(
+            S->d_slots, S->d_idx, n_done, S->h_status);
+        SRV_TRY(cudaGetLastError());
+        ++S->launches;
+        for (int j = 0; j < n_done; ++j) {
+            Slot &s = S->slots[S->h_idx[j]];
+            Result &res = S->results[s.req.ticket];
+            res.n = (size_t)(s.req.N + 1) * s.req.dim;
+            res.y.reset(new (std::nothrow) double[res.n]());  // touched here: the copy engine
+                                                                // is slow on new pages
+            if (!res.y) return srv_fail(FABM_ENOMEM, "host memory for a result");
+            SRV_TRY(cudaMemcpyAsync(res.y.get(), s.dev.Y, sizeof(double) * res.n, cudaMemcpyDeviceToHost, S->sR));
+        }
+        SRV_TRY(cudaStreamSynchronize(S->sR));
+        for (int j = 0; j < n_done; ++j) {
+            Slot &s = S->slots[S->h_idx[j]];
+            Result &res = S->results[s.req.ticket];
+            const bool ok = S->h_status[j] == ~0ull;
+            res.state = ok ? FABM_REQ_DONE : FABM_REQ_FAILED;
+            res.status = ok ? FABM_OK : FABM_ENONFINITE;
+            S->finished.push_back(s.req.ticket);
+            SRV_TRY(cudaFreeAsync(s.mem, S->sR));
+            S->in_use -= s.bytes;
+        }
         S->slots.erase(std::remove_if(S->slots.begin(), S->slots.end(),
                                       [](const Slot &s) { return s.c >= s.nblk; }),
                        S->slots.end());
@@ -736,14 +899,14 @@ fabm_status fabm_server_create(size_t budget_bytes, int precision, int max_slots
     S->budget = budget_bytes, S->precision = precision, S->max_slots = max_slots;
     cudaError_t e = cudaGetDevice(&S->device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->sR, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->sG, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->sW, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->evUp, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->evIn, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&S->d_slots, sizeof(SlotDev) * max_slots);
     if (e == cudaSuccess) e = cudaMalloc(&S->d_idx, sizeof(int) * max_slots);
-    if (e == cudaSuccess) e = cudaMalloc(&S->d_c, sizeof(int64_t) * max_slots);
-    if (e == cudaSuccess) e = cudaMallocHost(&S->h_c, sizeof(int64_t) * max_slots);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->evW, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMalloc(&S->d_cnt, sizeof(int) * max_slots);
+    if (e == cudaSuccess) e = cudaMemset(S->d_cnt, 0, sizeof(int) * max_slots);
+    if (e == cudaSuccess) e = cudaMallocHost(&S->h_status, sizeof(unsigned long long) * max_slots);
     if (e == cudaSuccess) e = cudaMallocHost(&S->h_slots, sizeof(SlotDev) * max_slots);
     if (e == cudaSuccess) e = cudaMallocHost(&S->h_idx, sizeof(int) * max_slots);
     if (e != cudaSuccess) {
@@ -789,7 +952,7 @@ static fabm_status server_submit(fabm_server *S, const fabm_request *q, const do
     std::lock_guard<std::mutex> lk(S->mu);
     r.ticket = S->next_ticket++;
     S->queue.push_back(r);
-    S->results[r.ticket] = {FABM_REQ_WAITING, FABM_OK, {}};
+    S->results[r.ticket] = {FABM_REQ_WAITING, FABM_OK, nullptr};
     S->shapes[r.ticket] = {r.N, r.dim};
     *ticket = r.ticket;
     return FABM_OK;
@@ -844,7 +1007,7 @@ fabm_status fabm_server_result(fabm_server *S, int64_t ticket, double *out)
     if (r.state == FABM_REQ_WAITING || r.state == FABM_REQ_RUNNING)
         return srv_fail(FABM_EBUSY, "request %lld not finished", (long long)ticket);
     const fabm_status st = r.status;
-    if (!r.y.empty()) std::memcpy(out, r.y.data(), sizeof(double) * r.y.size());
+    if (r.y) std::memcpy(out, r.y.get(), sizeof(double) * r.n);
     S->results.erase(it);
     S->shapes.erase(ticket);
     if (st != FABM_OK)
@@ -960,7 +1123,7 @@ fabm_status fabm_server_resume(fabm_server *S, const void *buf, size_t size, int
     std::lock_guard<std::mutex> lk(S->mu);
     r.ticket = S->next_ticket++;
     S->queue.push_back(r);
-    S->results[r.ticket] = {FABM_REQ_WAITING, FABM_OK, {}};
+    S->results[r.ticket] = {FABM_REQ_WAITING, FABM_OK, nullptr};
     S->shapes[r.ticket] = {r.N, r.dim};
     *ticket = r.ticket;
     return FABM_OK;

@@ -5,19 +5,19 @@
 namespace fabm {
 namespace {
 
-__global__ void weights_kernel(double alpha, int64_t N, double inv_g1, double inv_g2, double *B,
-                               double *A, double *D)
+__global__ void __launch_bounds__(kWeightThreads)
+    weights_kernel(double alpha, int64_t N, double inv_g1, double inv_g2, double *B, double *A,
+                   double *D)
 {
-    for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d <= N;
-         d += (int64_t)gridDim.x * blockDim.x)
-        weights_at(d, alpha, inv_g1, inv_g2, B, A, D);
+    for (int64_t d0 = blockIdx.x * (int64_t)blockDim.x; d0 <= N; d0 += (int64_t)gridDim.x * blockDim.x)
+        weights_block(d0, N, alpha, inv_g1, inv_g2, B, A, D, [](int64_t) {});
 }
 
 }  // namespace
 cudaError_t launch_weights(double alpha, int64_t N, double inv_g1, double inv_g2, double *B,
                            double *A, double *D, cudaStream_t st)
 {
-    const int threads = 256;
+    const int threads = kWeightThreads;
     int64_t blocks = (N + 1 + threads - 1) / threads;
     if (blocks > 152 * 32) blocks = 152 * 32;
     weights_kernel<<<(unsigned)blocks, threads, 0, st>>>(alpha, N, inv_g1, inv_g2, B, A, D);
