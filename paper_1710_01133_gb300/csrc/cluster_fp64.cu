@@ -501,7 +501,8 @@ cudaError_t cluster_config(int B, int CS, int n, int nW, bool alone, cudaLaunchC
     const int warps = CS > 1 ? (kc > kHelpWarps + 1 ? kc : kHelpWarps + 1) : kc + kHelpWarps + 1;
     size_t smem = sizeof(double) * (size_t)layout(D, nW, n, CS).total;
     if (alone && smem < 120 * 1024) smem = 120 * 1024;  // one CTA per SM
-    if (smem > 226 * 1024) return cudaErrorInvalidConfiguration;
+    constexpr size_t kMaxSmem = 226 * 1024;
+    if (smem > kMaxSmem) return cudaErrorInvalidConfiguration;
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3((unsigned)(B * CS));
     cfg->blockDim = dim3((unsigned)(warps * kWarp));
@@ -511,7 +512,9 @@ cudaError_t cluster_config(int B, int CS, int n, int nW, bool alone, cudaLaunchC
     cfg->attrs = attr;
     cfg->numAttrs = 1;
     auto k = cluster_kernel<Rhs, D>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the same limit in every call: a solver on another thread may be about to launch
+    // this kernel with another size
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e == cudaSuccess && CS > 8)
         e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;

@@ -70,11 +70,13 @@ cudaError_t launch_hist_fp32c(const DevBatch &bt, const float *WBf, const float 
     const int groups = (bt.cols + hist::kColsPerCta - 1) / hist::kColsPerCta;
     const int pack = alone ? kPack : 1;
     auto run = [&](auto kernel, size_t tiles, int64_t stride, int dim) -> cudaError_t {
-        size_t smem = tiles * pack;
-        if (alone) smem = smem > kAloneSmem ? smem : kAloneSmem;
+        const size_t packed = tiles * kPack > kAloneSmem ? tiles * kPack : kAloneSmem;
+        const size_t smem = alone ? packed : tiles;
         if (smem > 48 * 1024) {
+            // the same limit in every call: a solver on another thread may be about
+            // to launch this kernel with the other size
             const cudaError_t e =
-                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)packed);
             if (e != cudaSuccess) return e;
         }
         kernel<<<dim3((unsigned)((n_chunks + pack - 1) / pack), (unsigned)groups), pack * kGroup, smem, st>>>(
