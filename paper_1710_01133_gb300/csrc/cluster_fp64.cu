@@ -537,14 +537,15 @@ int cluster_max_active(int rhs, int dim, bool multi, int CS, int n)
 }
 
 cudaError_t launch_cluster_fp64(int rhs, const DevBatch &bt, const DevWeights &w,
-                                const StepConsts &k, int64_t T, int n, int CS, const double *G,
+                                const StepConsts &k, int64_t T, int n, int CS, bool alone,
+                                const double *G,
                                 const double *X, unsigned *err, long long wait_cycles, cudaStream_t st)
 {
     cudaError_t e = cudaErrorInvalidValue;
     dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
-        e = cluster_config<R, D>(bt.B, CS, n, w.stride ? D : 1, CS > 1, &cfg, &attr);
+        e = cluster_config<R, D>(bt.B, CS, n, w.stride ? D : 1, alone, &cfg, &attr);
         if (e != cudaSuccess) return;
         cfg.stream = st;
         const Args a{bt, w, k, T, n, G, X, err, wait_cycles};

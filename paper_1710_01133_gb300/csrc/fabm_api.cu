@@ -95,6 +95,10 @@ struct DevBuf {
 };
 
 constexpr int kMaxBlockL = 1024;
+// FP64X2: up to kX2AloneMax trajectories step on SMs that the history leaves them
+// (Lorenz type 2^13, ms with / without: 8 trajectories 17.3 / 23.3, 16 36.1 / 38.2,
+// 24 54.7 / 53.6).
+constexpr int kX2AloneMax = 16;
 constexpr int kEvRing = 4;
 constexpr int kClusterChoices = 9;
 constexpr int kAuxRing = 4;  // forcing tables computed up to 3 blocks ahead
@@ -272,11 +276,11 @@ namespace {
 // CTAs): Lorenz 2^18 FP64, 3 columns: 499/381/419/710; 4 trajectories x 2^16,
 // 12 columns: 117/103/108/122; 16 x 2^15, 48 columns: 115/114/109/99; Duffing
 // 64 x 2^14, 128 columns: 106/106/94/83; LCR 256 x 2^13, 512 columns:
-// 256/173/107/68.  FP64X2 (10 FP64 operations per term) is best at 608 for 3
-// columns.
+// 256/173/107/68.  FP64X2 (four warps share a chunk; ms for 608/1216/2432 CTAs):
+// Lorenz-type 64 x 2^12 41/34/36, 256 x 2^12 152/124/125, 512 x 2^11 111/61/62.
 int auto_chunk_ctas(int hk, int64_t cols)
 {
-    if (hk == FABM_HIST_X2) return 152 * 4;
+    if (hk == FABM_HIST_X2) return 152 * 8;
     const int64_t col_tiles = (cols + 3) / 4;
     return col_tiles <= 4 ? 152 * 2 : (col_tiles >= 8 ? 152 * 8 : 152 * 4);
 }
@@ -415,12 +419,25 @@ int resolve_hist_kernel(const fabm_solver *s, int64_t cols)
 // Lag 2 pays where the history bounds the solve: N x cols at least 2^19 for
 // the FP64 kernel (its per-block work then exceeds the recurrence's ~30 us),
 // 2^25 for the compensated-fp32 kernel (64x the FP64 rate).  Below that the
-// extra lag block only lengthens the recurrence.
+// extra lag block only lengthens the recurrence.  FP64X2 keeps lag 1: its history
+// CTAs fill the FP64 units on their own, four warps per SM.
 int history_lag(int hk, int64_t N, int64_t cols)
 {
-    if (hk == FABM_HIST_FP64 || hk == FABM_HIST_X2) return N * cols >= (1LL << 19) ? 2 : 1;
+    if (hk == FABM_HIST_FP64) return N * cols >= (1LL << 19) ? 2 : 1;
     if (hk == FABM_HIST_FP32C) return N * cols >= (1LL << 25) ? 2 : 1;
     return 1;
+}
+
+// FP64X2: a CTA's four warps share a chunk of its four columns, so that chunks may
+// be short; at_most: no more than want_ctas CTAs (one wave of an SM each).
+void plan_chunks_x2(int64_t k_end, int cols, int64_t max_chunks, int want_ctas, bool at_most,
+                    int *n_chunks, int64_t *kc)
+{
+    const int col_tiles = (cols + 3) / 4;
+    const int64_t want = at_most ? want_ctas / col_tiles : (want_ctas + col_tiles - 1) / col_tiles;
+    const int64_t n = std::clamp<int64_t>(std::min<int64_t>(want, k_end / 16), 1, max_chunks);
+    *kc = ((k_end + n - 1) / n + 3) / 4 * 4;
+    *n_chunks = (int)((k_end + *kc - 1) / *kc);
 }
 
 // Enqueues one solve on the solver's streams (or records it into the graph
@@ -445,6 +462,12 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                     s->chunk_ctas > 0 ? s->chunk_ctas : auto_chunk_ctas(hk, cols), &n_chunks, &kc);
         alone = fp32c_alone(n_chunks, (int)cols, bt.B);
     }
+    const bool x2 = hk == FABM_HIST_X2;
+    // few trajectories: history and steps on SMs of their own here as well
+    const bool x2_alone = x2 && s->chunk_ctas == 0 && bt.B <= kX2AloneMax;
+    const int x2_ctas = s->chunk_ctas > 0 ? s->chunk_ctas
+                        : x2_alone        ? 152 - bt.B
+                                          : auto_chunk_ctas(hk, cols);
     const int n_gbuf = lag + 1;  // G of block c is read by R(c) until H(c + lag + 1) starts
     s->sample_now = true;
     FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
@@ -569,14 +592,17 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             // algorithmic work: 2 sums x L targets x k_end points x cols, 2 flops each
             const double flops = 4.0 * L * (double)k_end * (double)cols;
             FABM_CUDA_TRY(cudaStreamWaitEvent(gs, s->evR[(c - lag - 1) % kEvRing], 0));
-            plan_chunks(k_end, (int)cols, max_chunks,
-                        s->chunk_ctas > 0 ? s->chunk_ctas : auto_chunk_ctas(hk, cols), &n_chunks,
-                        &kc);
-            if (hk == FABM_HIST_X2) {
+            if (x2)
+                plan_chunks_x2(k_end, (int)cols, max_chunks, x2_ctas, x2_alone, &n_chunks, &kc);
+            else
+                plan_chunks(k_end, (int)cols, max_chunks,
+                            s->chunk_ctas > 0 ? s->chunk_ctas : auto_chunk_ctas(hk, cols), &n_chunks,
+                            &kc);
+            if (x2) {
                 double2 *xp = reinterpret_cast<double2 *>(s->part.p) + poff;
                 const DevWeightsLo wl{s->wBl.p, s->wAl.p, s->wDl.p};
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, gs, flops, [&] {
-                    return launch_hist_x2(bt, w, wl, c, lag, n_chunks, kc, xp, gs);
+                    return launch_hist_x2(bt, w, wl, c, lag, n_chunks, kc, x2_alone, xp, gs);
                 }));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, gs, 0.0, [&] {
                     return launch_reduce_x2(xp, n_chunks, (int)cols, Gbuf, gs);
@@ -612,6 +638,16 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             X = s->auxb.p + (size_t)(c % kAuxRing) * kSplitSeg * bt.B;
             FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evA[c % kAuxRing], 0));
         }
+        double *X64 = nullptr;
+        if (x2 && rhs_has_forcing(s->rhs, bt.dim)) {  // on sG2, a block ahead of the steps
+            X64 = s->Xrow.p + (size_t)(c & 1) * L * bt.B;
+            if (c >= 2) FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG2, s->evR[(c - 2) % kEvRing], 0));
+            FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sG2, 0.0, [&] {
+                return launch_aux_rows(s->rhs, bt, s->h, c, L, X64, s->sG2);
+            }));
+            FABM_CUDA_TRY(cudaEventRecord(s->evA[c % kAuxRing], s->sG2));
+            FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evA[c % kAuxRing], 0));
+        }
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sR, rflops, [&] {
             if (split) {
                 const bool slices = c + 1 < nblk;  // segment c is read by the blocks c+1 ..
@@ -619,6 +655,10 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                 return launch_recur_cols(s->rhs, bt, s->wBff.p, s->wAff.p, s->wDff.p, s->k, c, hin,
                                          in, s->cols_warps, s->sR);
             }
+            if (x2)
+                return launch_cluster_fp64(s->rhs, bt, w, s->k, c, L, 1, x2_alone,
+                                           static_cast<const double *>(Gc), X64, s->err.p,
+                                           s->wait_cycles, s->sR);
             return launch_recur(s->rhs, bt, w, s->k, c, L, lag, s->precision == FABM_SPLIT, alone,
                                 static_cast<const double *>(Gc), s->sR);
         }));
@@ -732,7 +772,8 @@ fabm_status enqueue_clusters(fabm_solver *s, const DevBatch &bt, const DevWeight
         const int64_t lo = T * n, hi = std::min<int64_t>((T + 1) * n, Nmax);
         const double near = (double)(T > 0 ? n : 0) + 0.5 * (double)(hi - lo + 1);
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sR, 4.0 * (double)(hi - lo) * near * cols, [&] {
-            return launch_cluster_fp64(s->rhs, bt, w, s->k, T, n, s->cl_size, G, X, s->err.p,
+            return launch_cluster_fp64(s->rhs, bt, w, s->k, T, n, s->cl_size, s->cl_size > 1, G, X,
+                                       s->err.p,
                                        s->wait_cycles, s->sR);
         }));
         FABM_CUDA_TRY(cudaEventRecord(s->evR[T % kEvRing], s->sR));
@@ -829,7 +870,15 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     if (!s->cl_size) FABM_CUDA_TRY(s->G.ensure((size_t)3 * 2 * L * cols));
     // two partial buffers: the history launches of blocks c and c+1 may overlap
     if (hk == FABM_HIST_FP64 && !s->cl_size) FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
-    if (hk == FABM_HIST_X2) FABM_CUDA_TRY(s->part.ensure((size_t)4 * max_chunks * part_per_chunk));
+    if (hk == FABM_HIST_X2) {
+        // pairs; the steps by the superblock kernel, a block of 32 targets per launch
+        // (the same 32 to 64 newest points in double as recur_block; Lorenz type,
+        // cold caches, 28.4 -> 20.5 us a block)
+        FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
+        if (rhs_has_forcing(s->rhs, dim)) FABM_CUDA_TRY(s->Xrow.ensure((size_t)2 * L * B));
+        FABM_CUDA_TRY(s->err.ensure(1));
+        FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
+    }
     if (hk == FABM_HIST_FP32C) {
         FABM_CUDA_TRY(s->spart.ensure((size_t)2 * max_chunks * part_per_chunk));
         FABM_CUDA_TRY(s->Ff.ensure(f_elems));
@@ -1074,7 +1123,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
 
     unsigned long long st = 0;
     FABM_CUDA_TRY(cudaMemcpy(&st, s->status.p, sizeof st, cudaMemcpyDeviceToHost));
-    if (split || s->cl_size) {  // bounded waits
+    if (split || s->cl_size || hk == FABM_HIST_X2) {  // bounded waits
         unsigned int tout = 0;
         FABM_CUDA_TRY(cudaMemcpy(&tout, s->err.p, sizeof tout, cudaMemcpyDeviceToHost));
         if (tout) return fail(FABM_ETIMEOUT, "a history kernel gave up waiting on a barrier");
@@ -1475,8 +1524,9 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
     // at most 8 candidates are reported
     if (s->precision == FABM_FP64 || s->precision == FABM_FP64X2) {
         const int k = s->precision == FABM_FP64 ? FABM_HIST_FP64 : FABM_HIST_X2;
-        if (s->precision == FABM_FP64) cands.push_back({k, 0});  // superblocks, the automatic choice
-        for (int c : ctas_opts) cands.push_back({k, c});
+        cands.push_back({k, 0});  // the automatic choice: superblocks; FP64X2: by the batch
+        for (int c : ctas_opts)
+            if (s->precision == FABM_FP64 || c > 152) cands.push_back({k, c});
         if (s->precision == FABM_FP64 && s->persist_ctas >= B + 8 && !s->multi)
             cands.push_back({FABM_HIST_FP64_PERSIST, s->persist_ctas});
     } else {

@@ -258,7 +258,8 @@ int cluster_max_active(int rhs, int dim, bool multi, int CS, int n);
 // k < n(T-1), or NULL for T < 2; X: the rows of launch_aux_rows (required when
 // rhs_has_forcing).  err: set when a wait gave up.
 cudaError_t launch_cluster_fp64(int rhs, const DevBatch &bt, const DevWeights &w,
-                                const StepConsts &k, int64_t T, int n, int CS, const double *G,
+                                const StepConsts &k, int64_t T, int n, int CS, bool alone,
+                                const double *G,
                                 const double *X, unsigned *err, long long wait_cycles, cudaStream_t st);
 // X[b][j] = the time-only part of f at t_m, m = nT+1+j, j < n.
 cudaError_t launch_aux_rows(int rhs, const DevBatch &bt, double h, int64_t T, int n, double *X,
@@ -304,9 +305,10 @@ cudaError_t launch_weights_x2(double alpha, int64_t n, double ig1_hi, double ig1
                               double *Al, double *Dh, double *Dl, cudaStream_t st);
 
 // a2 in double-double: partial far-history sums of target block c (32 targets)
-// over k < (c-lag)*32 as (hi, lo) pairs, n_chunks x 2 x 32 x cols.
+// over k < (c-lag)*32 as (hi, lo) pairs, n_chunks x 2 x 32 x cols; alone: one CTA
+// per SM.
 cudaError_t launch_hist_x2(const DevBatch &bt, const DevWeights &w, const DevWeightsLo &wl,
-                           int64_t c, int lag, int n_chunks, int64_t kc, double2 *part,
+                           int64_t c, int lag, int n_chunks, int64_t kc, bool alone, double2 *part,
                            cudaStream_t st);
 // a3: G = sum over chunks in double-double, rounded once to double.
 cudaError_t launch_reduce_x2(const double2 *part, int n_chunks, int cols, double *G, cudaStream_t st);
