@@ -162,11 +162,11 @@ class ClockSampler:
 # Sources each profiled kernel is built from; a committed ncu summary gives its
 # traffic only while the sha256 over these files (in this order) still matches.
 KERNEL_SOURCES = {
-    "history_fp64": ["history_fp64.cu", "history_blocks.cuh", "fabm_internal.cuh"],
+    "history_fp64": ["far_fft.cu", "fabm_internal.cuh"],
     "history_split": ["history_far.cu", "history_split.cu", "sm100_ptx.cuh", "fabm_internal.cuh"],
-    "recurrence": ["recurrence.cu", "recurrence.cuh", "rhs.cuh", "fabm_internal.cuh"],
-    "recurrence_split": ["recurrence_cols.cu", "recurrence.cuh", "rhs.cuh", "ff.cuh",
-                         "fabm_internal.cuh"],
+    "recurrence": ["cluster_fp64.cu", "recurrence.cuh", "rhs.cuh", "fabm_internal.cuh"],
+    "recurrence_split": ["recurrence_cols.cu", "split_slices.cuh", "recurrence.cuh", "rhs.cuh",
+                         "ff.cuh", "fabm_internal.cuh"],
     "history_served": ["serve.cu", "history_blocks.cuh", "recurrence.cuh", "fabm_internal.cuh"],
 }
 
@@ -270,8 +270,11 @@ def roofline(kind, ks, precision, clocks, workload, w=None, step_ms=None):
         note = ("FP64 FMA pipe: 2 DFMA/clk/SM x 152 SMs x max SM clock "
                 "(probe: 1.19 TFLOP/s at 1.96 GHz)")
         if precision == "fp64x2":
-            note += ("; achieved counts algorithmic multiply-adds, each of which costs ten "
-                     "FP64 operations in double-double")
+            note += ("; achieved counts algorithmic multiply-adds, each of which costs five "
+                     "FP64 instructions in double-double")
+        else:
+            note += ("; achieved counts the multiply-adds of direct sums, which the superblock "
+                     "schedule replaces by transforms, so it can exceed the peak")
         out.update({"bound": "alu", "peak_note": note})
     in_launch = mult * flops / (ms * 1e-3) / scale if ms > 0 else 0.0
     out["in_launch"] = {"launches_timed": n, "avg_launch_us": avg_us, "busy_ms": ms,
