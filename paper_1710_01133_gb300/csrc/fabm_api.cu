@@ -186,6 +186,7 @@ struct fabm_solver {
     DevBuf<double> Gfar, Xrow, fsegs;  // Xrow: forcing of two superblocks; fsegs: sums of f
     DevBuf<float2> auxb;       // tensor path: forcing tables of kAuxRing blocks
     DevBuf<float2> parff, y0ff; // tensor path: float-float parameters and y_0
+    bool cols_ready = false;  // tensor path: its recurrence kernels' limits are set
     DevBuf<unsigned int> err;  // split: timeout flag
     DevBuf<int64_t> nEach;
     DevBuf<unsigned long long> status;
@@ -926,6 +927,10 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         s->near_chunks = std::clamp(far_free / n_ct, 1, 3);
         // one team of warps per CTA unless set; the lane-per-target layout on request
         s->cols_warps = s->rec_layout == FABM_REC_TARGETS ? 0 : std::max(1, s->rec_warps);
+        if (!s->cols_ready) {  // here, as a narrow batch never needs it (0.1 ms)
+            FABM_CUDA_TRY(prepare_recur_cols(s->rhs, dim));
+            s->cols_ready = true;
+        }
         FABM_CUDA_TRY(s->parff.ensure((size_t)B * kMaxParams));
         FABM_CUDA_TRY(s->y0ff.ensure((size_t)cols));
         FABM_CUDA_TRY(s->Fs.ensure((size_t)nblk * n_ct * 3 * 128 * 64));
@@ -1306,8 +1311,7 @@ fabm_status create_solver(int dim, const double *alpha_c, double h, int64_t N, i
         }
         if (e == cudaSuccess && !multi) {
             const double ha = s->k.h_alpha[0];
-            e = prepare_recur_cols(rhs_id, dim);
-            if (e == cudaSuccess) e = s->wBff.ensure(kSplitSeg + 1);
+            e = s->wBff.ensure(kSplitSeg + 1);
             if (e == cudaSuccess) e = s->wAff.ensure(kSplitSeg + 1);
             if (e == cudaSuccess) e = s->wDff.ensure((size_t)s->w_ext + 1);
             if (e == cudaSuccess) e = launch_ff_weights(s->wB.p, ha, kSplitSeg + 1, s->wBff.p, s->sR);
