@@ -163,6 +163,7 @@ class ClockSampler:
 # traffic only while the sha256 over these files (in this order) still matches.
 KERNEL_SOURCES = {
     "history_fp64": ["far_fft.cu", "fabm_internal.cuh"],
+    "history_fp64x2": ["history_x2.cu", "fabm_internal.cuh"],
     "history_split": ["history_far.cu", "history_split.cu", "sm100_ptx.cuh", "fabm_internal.cuh"],
     "recurrence": ["cluster_fp64.cu", "recurrence.cuh", "rhs.cuh", "fabm_internal.cuh"],
     "recurrence_split": ["recurrence_cols.cu", "split_slices.cuh", "recurrence.cuh", "rhs.cuh",
@@ -292,7 +293,7 @@ def roofline(kind, ks, precision, clocks, workload, w=None, step_ms=None):
         out.update({"achieved": in_launch, "peak": peak, "unit": unit,
                     "frac": in_launch / peak if peak else None,
                     "achieved_over": out["in_launch"]["over"]})
-    key = {"history": f"history_{'split' if precision == 'split' else 'fp64'}",
+    key = {"history": f"history_{precision}",
            "recurrence": "recurrence_split" if precision == "split" else "recurrence"}.get(kind)
     # profiles/<kernel class>_<precision>_<workload>.md, e.g. history_fp64_lorenz-single.md
     traffic = _profile_traffic(key, f"{kind}_{precision}_{workload}") if key else None
