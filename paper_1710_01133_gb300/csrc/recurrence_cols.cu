@@ -35,12 +35,12 @@
 // on the component, and the slices written here instead of by a launch of their
 // own.  A block of 64 steps alone, one or two warps per 32 columns before / now:
 // LCR 1024 58 (a lane per target) / 37.5 us, Lorenz type 256 37 (likewise) / 34,
-// oscillator 4096 97 / 49.  Whole solves: LCR 1024 x 2^14 24.1 / 19.8 ms, Lorenz
-// type 256 x 2^16 87.8 / 52.4, 256 x 2^18 494 / 422, oscillator 4096 x 2^13 20.4 /
-// 16.9, 4096 x 2^16 312 / 306.  Measured and dropped: a second chain warp for
+// oscillator 4096 97 / 49.  Whole solves: LCR 1024 x 2^14 24.1 / 20.2 ms, Lorenz
+// type 256 x 2^16 87.8 / 52.4, 256 x 2^18 495 / 425, oscillator 4096 x 2^13 20.4 /
+// 16.9, 4096 x 2^16 317 / 308.  Measured and dropped: a second chain warp for
 // the sub-block's sums, handed over target by target (40 instead of 37 us, LCR),
 // helpers that take each point as it appears (40), sub-blocks of 4 (20.7 instead
-// of 19.8 ms).
+// of 19.8 ms, both on one box).
 #include <algorithm>
 #include <type_traits>
 
