@@ -136,6 +136,7 @@ __device__ __forceinline__ unsigned long long peek(const double *p)
     asm volatile("ld.relaxed.cluster.shared::cta.b64 %0, [%1];" : "=l"(u) : "r"(smem_u32(p)) : "memory");
     return u;
 }
+// The aligned form: the lanes of a warp have to arrive together.
 __device__ __forceinline__ void named_sync(int id, int threads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -408,6 +409,7 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
             }
 #pragma unroll
             for (int q = 0; q < C; ++q) sm[l.near + ((t & 1) * D + c0 + q) * kWarp + lane] = nxt[q];
+            __syncwarp();  // lanes leave their waits one by one; the barrier takes whole warps
             named_sync(2, (D + R::kPrev) * kWarp);
         }
     } else if (hr >= 0 && warp >= hw0 && warp < hw0 + kHelpWarps) {
@@ -452,6 +454,7 @@ __global__ void __launch_bounds__((Roles<D>::kChainWarps + kHelpWarps + 1) * kWa
                 reinterpret_cast<double(*)[D][kWarp]>(sm + l.red) + (t & 1) * kHelpWarps;
 #pragma unroll
             for (int q = 0; q < D; ++q) red[w][q][lane] = acc[q];
+            __syncwarp();  // as above
             named_sync(3, kHelpWarps * kWarp);
             if (w < D) {
                 // the slot's last rows, of block t-2, are used up once the chain has
