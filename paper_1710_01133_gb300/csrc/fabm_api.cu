@@ -1006,6 +1006,8 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     bt.status = s->status.p;
     DevWeights w{s->wB.p, s->wA.p, s->wD.p, s->w_ext, s->multi ? s->w_ext + 1 : 0};
 
+    // what a captured graph holds: every choice that shapes the launches and every
+    // buffer that a solve may allocate anew
     const std::vector<uintptr_t> key = {
         (uintptr_t)B, (uintptr_t)nblk, (uintptr_t)L, (uintptr_t)s->timing,
         (uintptr_t)s->timing_period, (uintptr_t)hk, (uintptr_t)s->chunk_ctas,
@@ -1018,7 +1020,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)s->fpart.p, (uintptr_t)s->fsum.p, (uintptr_t)s->near_chunks,
         (uintptr_t)s->plan_N, (uintptr_t)s->cl_size, (uintptr_t)s->cl_n, (uintptr_t)s->What.p,
         (uintptr_t)s->Fhat.p, (uintptr_t)s->facc.p, (uintptr_t)s->fmark.p, (uintptr_t)s->Gfar.p,
-        (uintptr_t)s->Xrow.p, (uintptr_t)s->fsegs.p,
+        (uintptr_t)s->Xrow.p, (uintptr_t)s->fsegs.p, (uintptr_t)s->tw.p,
         (uintptr_t)s->fmid.p, (uintptr_t)s->parff.p, (uintptr_t)s->y0ff.p,
         (uintptr_t)(s->cl_size ? Nmax : 0)};
     auto enqueue = [&]() -> fabm_status {

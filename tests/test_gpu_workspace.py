@@ -1,0 +1,34 @@
+"""A solver's work space and cached launch graph across solves of different
+shapes and failed allocations (needs a GPU).
+
+One solver used with several batch sizes allocates some buffers anew, and an
+allocation that fails (injected on the host) makes a solve take the schedule
+that needs less room.  A later solve of an earlier shape gives the same bits as
+before: the same launches on the same inputs.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from fabm_workloads import duffing_sweep, lorenz_long
+
+pytestmark = pytest.mark.gpu
+TOL_FP64 = 1e-12
+
+
+def rel_err(got, ref):
+    scale = np.max(np.abs(ref), axis=-2, keepdims=True)
+    return float(np.max(np.abs(got - ref) / np.where(scale == 0, 1.0, scale)))
+
+
+def test_graph_is_recorded_again_when_the_factors_move(gpu_lib):
+    """Superblocks of 512 targets need longer transforms than those of 128, so the
+    factors of the first solve's graph are freed by the second solve."""
+    w = duffing_sweep(256, 8192)
+    with gpu_lib.Solver(w.rhs, w.dim, w.alpha, w.h, w.N, w.params) as s:
+        first = s.solve_batch(w.y0, traj_params=w.traj_params)
+        s.set_graphs(False)
+        s.solve_batch(w.y0[:1], traj_params=w.traj_params[:1])
+        s.set_graphs(True)
+        again = s.solve_batch(w.y0, traj_params=w.traj_params)
+    assert np.array_equal(first, again)
