@@ -180,7 +180,7 @@ struct fabm_solver {
     // partial spectra, marks of large segments, far history of two superblocks
     int cl_size = 0, cl_n = 0;
     std::vector<int> cl_fit = std::vector<int>(kClusterChoices, -1);
-    int what_n = 0;  // superblock length the weight spectra are for
+    int what_n = 0;  // superblock length tw and What are for
     DevBuf<double2> tw, What, Fhat, facc, fmid;
     DevBuf<unsigned char> fmark;
     DevBuf<double> Gfar, Xrow, fsegs;  // Xrow: forcing of two superblocks; fsegs: sums of f
@@ -846,11 +846,11 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
             if (e == cudaSuccess) e = s->fsegs.ensure((size_t)nsb * cols);
             if (e == cudaSuccess) e = s->facc.ensure((size_t)16 * cols * 2 * n);
             if (e == cudaSuccess) e = s->Gfar.ensure((size_t)2 * 2 * n * cols);
-            if (e == cudaSuccess) e = s->tw.ensure((size_t)2 * n);
             const int64_t g_max = (N + n - 1) / n - 1;
             if (e == cudaSuccess && s->what_n != n) {
-                s->what_n = 0;
-                e = s->What.ensure((size_t)sets * (g_max + 1) * 2 * n);
+                s->what_n = 0;  // until both the factors and the spectra are those of n
+                e = s->tw.ensure((size_t)2 * n);
+                if (e == cudaSuccess) e = s->What.ensure((size_t)sets * (g_max + 1) * 2 * n);
                 if (e == cudaSuccess) {
                     const DevWeights w{s->wB.p, s->wA.p, s->wD.p, s->w_ext, s->multi ? s->w_ext + 1 : 0};
                     FABM_CUDA_TRY(launch_fft_weights(w, sets, n, (int)g_max, s->tw.p, s->What.p, s->sR));

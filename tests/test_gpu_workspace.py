@@ -32,3 +32,20 @@ def test_graph_is_recorded_again_when_the_factors_move(gpu_lib):
         s.set_graphs(True)
         again = s.solve_batch(w.y0, traj_params=w.traj_params)
     assert np.array_equal(first, again)
+
+
+def test_failed_allocation_of_the_factors(gpu_lib):
+    """The factors for 512 targets cannot be allocated (every other buffer fits):
+    that solve takes the block schedule, and the next one of the first shape
+    computes its factors again."""
+    w = lorenz_long(30, 4000)  # superblocks of 256 targets
+    with gpu_lib.Solver(w.rhs, w.dim, w.alpha, w.h, w.N, w.params) as s:
+        first = s.solve_batch(w.y0)
+        gpu_lib.fabm_inject_alloc_failures(1)
+        try:
+            s.solve_batch(w.y0[:1])
+        finally:
+            gpu_lib.fabm_inject_alloc_failures(0)
+        assert s.last_launch_count > 200  # one launch per kernel and block of 32
+        again = s.solve_batch(w.y0)
+    assert np.array_equal(first, again)
