@@ -1016,7 +1016,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)s->Fe.p, (uintptr_t)s->spart.p, (uintptr_t)s->y0.p, (uintptr_t)s->par.p,
         (uintptr_t)s->nEach.p, (uintptr_t)s->status.p, (uintptr_t)s->err.p, (uintptr_t)s->auxb.p,
         (uintptr_t)s->out_stream, (uintptr_t)s->out_group, (uintptr_t)s->wait_cycles,
-        (uintptr_t)s->wide, (uintptr_t)far_chunks, (uintptr_t)s->Fs2.p, (uintptr_t)s->Fe2.p,
+        (uintptr_t)s->wide, (uintptr_t)split_chunks, (uintptr_t)far_chunks, (uintptr_t)s->Fs2.p, (uintptr_t)s->Fe2.p,
         (uintptr_t)s->fpart.p, (uintptr_t)s->fsum.p, (uintptr_t)s->near_chunks,
         (uintptr_t)s->plan_N, (uintptr_t)s->cl_size, (uintptr_t)s->cl_n, (uintptr_t)s->What.p,
         (uintptr_t)s->Fhat.p, (uintptr_t)s->facc.p, (uintptr_t)s->fmark.p, (uintptr_t)s->Gfar.p,

@@ -49,3 +49,22 @@ def test_failed_allocation_of_the_factors(gpu_lib):
         assert s.last_launch_count > 200  # one launch per kernel and block of 32
         again = s.solve_batch(w.y0)
     assert np.array_equal(first, again)
+
+
+def test_graph_is_recorded_again_for_another_layout(gpu_lib):
+    """At nine column tiles the layouts asked for leave other numbers of SMs to the
+    recurrence, so the far history has 14 chunks automatically and 15 with
+    "columns", in both layouts by the same kernels."""
+    w = duffing_sweep(576, 2500)
+
+    def solver(layout):
+        return gpu_lib.Solver(w.rhs, w.dim, w.alpha, w.h, w.N, w.params, precision="split", history="tensor",
+                              recurrence=layout)
+
+    with solver("columns") as s:
+        want = s.solve_batch(w.y0, traj_params=w.traj_params)
+    with solver("auto") as s:
+        s.solve_batch(w.y0, traj_params=w.traj_params)
+        gpu_lib.fabm_set_recurrence_layout(s.handle, "columns")
+        got = s.solve_batch(w.y0, traj_params=w.traj_params)
+    assert np.array_equal(want, got)
