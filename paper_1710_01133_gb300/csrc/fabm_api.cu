@@ -844,7 +844,9 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
             if (e == cudaSuccess) e = s->fmark.ensure((size_t)2 * nsb * cols);
             if (e == cudaSuccess) e = s->fmid.ensure((size_t)2 * cols);
             if (e == cudaSuccess) e = s->fsegs.ensure((size_t)nsb * cols);
-            if (e == cudaSuccess) e = s->facc.ensure((size_t)16 * cols * 2 * n);
+            // the last superblock's sums have the most chunks
+            if (e == cudaSuccess)
+                e = s->facc.ensure((size_t)fft_chunks(n, (int)cols, nsb - 1) * cols * 2 * n);
             if (e == cudaSuccess) e = s->Gfar.ensure((size_t)2 * 2 * n * cols);
             const int64_t g_max = (N + n - 1) / n - 1;
             if (e == cudaSuccess && s->what_n != n) {

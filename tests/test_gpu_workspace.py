@@ -68,3 +68,19 @@ def test_graph_is_recorded_again_for_another_layout(gpu_lib):
         gpu_lib.fabm_set_recurrence_layout(s.handle, "columns")
         got = s.solve_batch(w.y0, traj_params=w.traj_params)
     assert np.array_equal(want, got)
+
+
+def test_partial_spectra_are_sized_by_their_chunks(gpu_lib):
+    """A wide batch's sums over segments have one chunk: 4 KB a column, where 16
+    would be 1.3 GB.  All other buffers of the solve are below 0.4 GB."""
+    torch = pytest.importorskip("torch")
+    B, N = 20000, 400  # superblocks of 128 targets, two of them with a far history
+    out = torch.empty((B, N + 1, 1), dtype=torch.float64, device="cuda")
+    with gpu_lib.Solver("linear", 1, 0.9, 1e-3, N, [1.0]) as s:
+        s.solve_batch(np.ones((B, 1)), N_each=np.full(B, 10), out=out)
+        free = torch.cuda.mem_get_info()[0]
+        s.solve_batch(np.ones((B, 1)), out=out)
+        assert s.last_launch_count < 30  # superblocks
+        assert free - torch.cuda.mem_get_info()[0] < 0.5e9
+    ref = oracle.solve("linear", 0.9, 1e-3, N, [1.0], params=[1.0])
+    assert rel_err(out[-1].cpu().numpy(), ref) <= TOL_FP64
