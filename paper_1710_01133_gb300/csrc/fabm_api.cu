@@ -229,13 +229,22 @@ struct fabm_solver {
     double k_flops[FABM_KERNEL_KINDS] = {};
     double k_busy[FABM_KERNEL_KINDS] = {};  // union of the timed launches' intervals
 
+    // Frees what only superblocks use; true if there was any.
+    bool release_superblocks()
+    {
+        const bool held = Fhat.p || facc.p || What.p || tw.p || Gfar.p || fmid.p || fmark.p || fsegs.p;
+        tw.release(), What.release(), Fhat.release(), facc.release(), fmid.release(), fmark.release(), Gfar.release(),
+            fsegs.release();
+        what_n = 0;
+        return held;
+    }
+
     ~fabm_solver()
     {
         wB.release(), wA.release(), wD.release(), wH.release(), wHe.release();
         wH2.release(), wHe2.release(), Fs2.release(), Fe2.release(), fpart.release(), fsum.release();
         ppart.release(), pspart.release(), psg.release(), pdone.release(), prdone.release();
-        tw.release(), What.release(), Fhat.release(), facc.release(), fmid.release(), fmark.release(), Gfar.release(),
-            Xrow.release(), fsegs.release();
+        release_superblocks(), Xrow.release();
         wBl.release(), wAl.release(), wDl.release();
         wBf.release(), wAf.release(), wBff.release(), wAff.release(), wDff.release();
         F.release(), Ff.release(), Ystage.release(), G.release(), part.release();
@@ -832,15 +841,32 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     const int64_t part_per_chunk = 2LL * L * cols;
     int64_t max_chunks = std::max<int64_t>(1, (int64_t)(64ull << 20) / (part_per_chunk * 8));
     max_chunks = std::min<int64_t>(max_chunks, 4096);
-    FABM_CUDA_TRY(s->F.ensure(f_elems));
+    // What every schedule needs comes first, and takes the room of superblock
+    // buffers that an earlier solve left if there is no other.
+    auto need = [&](auto &buf, size_t n) {
+        cudaError_t e = buf.ensure(n);
+        if (e == cudaErrorMemoryAllocation && s->release_superblocks()) {
+            cudaGetLastError();
+            e = buf.ensure(n);
+        }
+        return e;
+    };
+    FABM_CUDA_TRY(need(s->F, f_elems));
+    if (!out_on_device) FABM_CUDA_TRY(need(s->Ystage, (size_t)B * (N + 1) * dim));
+    FABM_CUDA_TRY(need(s->y0, (size_t)B * dim * 2));  // y0, then y1
+    FABM_CUDA_TRY(need(s->par, (size_t)B * kMaxParams));
+    FABM_CUDA_TRY(need(s->nEach, (size_t)B));
+    FABM_CUDA_TRY(need(s->status, 1));
     s->cl_size = 0;
     if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0) {
         plan_cluster(s, B, cols, s->plan_N > 0 ? s->plan_N : N);
         const int n = s->cl_n;
         const int64_t nsb = (Nmax + n - 1) / n;
+        cudaError_t e = cudaSuccess;
+        if (s->cl_size && rhs_has_forcing(s->rhs, dim)) e = s->Xrow.ensure((size_t)2 * n * B);
         if (s->cl_size && nsb > 2) {  // superblocks with a far history
             const int sets = s->multi ? dim : 1;
-            cudaError_t e = s->Fhat.ensure((size_t)(nsb - 2) * cols * 2 * n);
+            if (e == cudaSuccess) e = s->Fhat.ensure((size_t)(nsb - 2) * cols * 2 * n);
             if (e == cudaSuccess) e = s->fmark.ensure((size_t)2 * nsb * cols);
             if (e == cudaSuccess) e = s->fmid.ensure((size_t)2 * cols);
             if (e == cudaSuccess) e = s->fsegs.ensure((size_t)nsb * cols);
@@ -859,20 +885,20 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
                     s->what_n = n;
                 }
             }
-            if (e != cudaSuccess) {  // no room for the spectra: the block schedule
-                cudaGetLastError();
-                s->cl_size = 0;
-            }
+        }
+        if (e != cudaSuccess) {  // no room for them: the block schedule, which may need theirs
+            cudaGetLastError();
+            s->release_superblocks();
+            s->cl_size = 0;
         }
         if (s->cl_size) {
-            if (rhs_has_forcing(s->rhs, dim)) FABM_CUDA_TRY(s->Xrow.ensure((size_t)2 * n * B));
-            FABM_CUDA_TRY(s->err.ensure(1));
+            FABM_CUDA_TRY(need(s->err, 1));
             FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
         }
     }
-    if (!s->cl_size) FABM_CUDA_TRY(s->G.ensure((size_t)3 * 2 * L * cols));
+    if (!s->cl_size) FABM_CUDA_TRY(need(s->G, (size_t)3 * 2 * L * cols));
     // two partial buffers: the history launches of blocks c and c+1 may overlap
-    if (hk == FABM_HIST_FP64 && !s->cl_size) FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
+    if (hk == FABM_HIST_FP64 && !s->cl_size) FABM_CUDA_TRY(need(s->part, (size_t)2 * max_chunks * part_per_chunk));
     if (hk == FABM_HIST_X2) {
         // pairs; the steps by the superblock kernel, a block of 32 targets per launch
         // (the same 32 to 64 newest points in double as recur_block; Lorenz type,
@@ -886,10 +912,6 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         FABM_CUDA_TRY(s->spart.ensure((size_t)2 * max_chunks * part_per_chunk));
         FABM_CUDA_TRY(s->Ff.ensure(f_elems));
     }
-    FABM_CUDA_TRY(s->y0.ensure((size_t)B * dim * 2));  // y0, then y1
-    FABM_CUDA_TRY(s->par.ensure((size_t)B * kMaxParams));
-    FABM_CUDA_TRY(s->nEach.ensure((size_t)B));
-    FABM_CUDA_TRY(s->status.ensure(1));
     const int n_ct = (int)((cols + 127) / 128);
     int split_chunks = 1, far_chunks = 1;
     s->wide = false;
@@ -952,11 +974,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         FABM_CUDA_TRY(s->err.ensure(1));
         FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
     }
-    double *Y = out;
-    if (!out_on_device) {
-        FABM_CUDA_TRY(s->Ystage.ensure((size_t)B * (N + 1) * dim));
-        Y = s->Ystage.p;
-    }
+    double *Y = out_on_device ? out : s->Ystage.p;
     // a large output into pinned host memory, every trajectory to N: copied
     // block group by block group on sC while the solve goes on (a group is at
     // least 8 MB), instead of once at the end
@@ -1036,11 +1054,11 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         const int pchunks = persist_workers(grid, (int)B);
         const int ncg = (int)((cols + 3) / 4);
         const size_t n_sg = (size_t)nblk * ncg * persist_max_sg(pchunks);
-        FABM_CUDA_TRY(s->ppart.ensure(persist_part_elems(pchunks, (int)cols)));
-        FABM_CUDA_TRY(s->pspart.ensure(persist_spart_elems(pchunks, (int)cols)));
-        FABM_CUDA_TRY(s->psg.ensure(n_sg));
-        FABM_CUDA_TRY(s->pdone.ensure((size_t)nblk * ncg));
-        FABM_CUDA_TRY(s->prdone.ensure((size_t)B));
+        FABM_CUDA_TRY(need(s->ppart, persist_part_elems(pchunks, (int)cols)));
+        FABM_CUDA_TRY(need(s->pspart, persist_spart_elems(pchunks, (int)cols)));
+        FABM_CUDA_TRY(need(s->psg, n_sg));
+        FABM_CUDA_TRY(need(s->pdone, (size_t)nblk * ncg));
+        FABM_CUDA_TRY(need(s->prdone, (size_t)B));
         FABM_CUDA_TRY(s->err.ensure(1));
         s->recs.clear();
         FABM_CUDA_TRY(cudaMemsetAsync(s->psg.p, 0, sizeof(int) * n_sg, s->sR));
@@ -1550,7 +1568,12 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
     DeviceGuard g(s->device);
     double *dout = nullptr;
     {
-        cudaError_t e = cudaMalloc(&dout, sizeof(double) * (size_t)B * (s->N + 1) * s->dim);
+        const size_t bytes = sizeof(double) * (size_t)B * (s->N + 1) * s->dim;
+        cudaError_t e = cudaMalloc(&dout, bytes);
+        if (e == cudaErrorMemoryAllocation && s->release_superblocks()) {
+            cudaGetLastError();
+            e = cudaMalloc(&dout, bytes);
+        }
         if (e != cudaSuccess) return fail(FABM_ENOMEM, "autotune output: %s", cudaGetErrorString(e));
     }
     std::vector<int64_t> ne((size_t)B, n1);

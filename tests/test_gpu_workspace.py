@@ -84,3 +84,46 @@ def test_partial_spectra_are_sized_by_their_chunks(gpu_lib):
         assert free - torch.cuda.mem_get_info()[0] < 0.5e9
     ref = oracle.solve("linear", 0.9, 1e-3, N, [1.0], params=[1.0])
     assert rel_err(out[-1].cpu().numpy(), ref) <= TOL_FP64
+
+
+def test_spectra_make_way_for_what_every_schedule_needs(gpu_lib, parity):
+    """The spectra of an earlier solve are on the device when the staging buffer of
+    a host output cannot be allocated: they are given back and the solve goes on."""
+    torch = pytest.importorskip("torch")
+    w = duffing_sweep(3, 4000)
+    ref = oracle.solve_batch(w.rhs, w.alpha, w.h, w.N, w.y0, params=w.params, traj_params=w.traj_params)
+    with gpu_lib.Solver(w.rhs, w.dim, w.alpha, w.h, w.N, w.params) as s:
+        dev = torch.empty((w.B, w.N + 1, w.dim), dtype=torch.float64, device="cuda")
+        s.solve_batch(w.y0, traj_params=w.traj_params, out=dev)
+        gpu_lib.fabm_inject_alloc_failures(1)
+        try:
+            got = s.solve_batch(w.y0, traj_params=w.traj_params)
+        finally:
+            gpu_lib.fabm_inject_alloc_failures(0)
+    parity(rel_err(got, ref), TOL_FP64, "host")
+    assert np.array_equal(got, dev.cpu().numpy())
+
+
+def test_fallback_gives_the_spectra_back(gpu_lib):
+    """A wider batch one of whose superblock buffers cannot grow takes the block
+    schedule, whose own buffers are 0.13 GB here; the spectra of the solve before
+    it (0.44 GB) do not stay beside them."""
+    torch = pytest.importorskip("torch")
+    N, B = 20000, 700  # 32 bytes a point and column, one column
+    y0 = np.ones((B + 100, 1))
+    out = torch.empty((B + 100, N + 1, 1), dtype=torch.float64, device="cuda")
+    with gpu_lib.Solver("linear", 1, 0.9, 1e-3, N, [1.0]) as s:
+        # the buffers of the wider batch that do not depend on the schedule
+        s.solve_batch(y0, N_each=np.full(B + 100, 200), out=out)
+        before = torch.cuda.mem_get_info()[0]
+        s.solve_batch(y0[:B], out=out[:B])
+        assert before - torch.cuda.mem_get_info()[0] > 0.4e9
+        gpu_lib.fabm_inject_alloc_failures(1)
+        try:
+            s.solve_batch(y0, N_each=np.full(B + 100, 2000), out=out)
+        finally:
+            gpu_lib.fabm_inject_alloc_failures(0)
+        assert s.last_launch_count > 100  # one launch per kernel and block of 32
+        assert before - torch.cuda.mem_get_info()[0] < 0.3e9
+    ref = oracle.solve("linear", 0.9, 1e-3, 2000, [1.0], params=[1.0])
+    assert rel_err(out[-1, :2001].cpu().numpy(), ref) <= TOL_FP64
