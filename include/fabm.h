@@ -162,8 +162,8 @@ enum {
                               the last two superblocks of 128 to 512 steps summed
                               directly, older ones by transforms of a superblock's
                               points (32 bytes of device memory per step and column
-                              beyond two superblocks; without that room, every point
-                              is summed directly)                                    */
+                              beyond two superblocks; without that room, or after
+                              fabm_set_block(32), every point is summed directly)    */
     FABM_HIST_TENSOR = 2,  /* three-term bf16 split on tcgen05 tensor cores, exact
                               per 64-point segment, far history of each 64-step block
                               with 64 targets per MMA (split precision)              */
@@ -247,9 +247,11 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
                           int *ctas_report, int *n_report);
 
 /* Time-block length L of the last solve (or of the current choice before any
- * solve).  fabm_set_block accepts only the length of an allowed history
- * kernel (32 or 64) and selects that kernel; it changes the order of summation
- * only. */
+ * solve); 32 for FABM_FP64 solves by superblocks too.  fabm_set_block accepts
+ * only the length of an allowed history kernel (32 or 64) and selects that
+ * kernel; it changes the order of summation only.  On a FABM_FP64 solver 32
+ * asks for blocks of 32 steps with every point summed directly, without
+ * superblocks, until fabm_set_history_kernel or fabm_autotune chooses anew. */
 fabm_status fabm_set_block(fabm_solver *s, int L);
 int fabm_get_block(const fabm_solver *s);
 

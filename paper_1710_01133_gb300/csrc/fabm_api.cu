@@ -8,7 +8,8 @@
 //              segments 0 .. T-2
 //   stream G2: forcing of superblock T
 // Schedule of the other solves, block by block (and of FP64 solves whose
-// spectra do not fit or whose chunk count the autotuner has set):
+// spectra do not fit, whose chunk count the autotuner has set, or whose block
+// length is set):
 //   init                      y_0, f_0
 //   for each block c of L targets (CUDA-core history kernels, L = 32):
 //     stream G:  wait R(c-2); history(c) over k < (c-1)L; combine -> G[c%2]
@@ -131,6 +132,7 @@ struct fabm_solver {
     double params[kMaxParams] = {};
     int precision = FABM_FP64;
     int hist_kernel = FABM_HIST_AUTO;  // requested
+    bool direct = false;               // FP64: direct sums block by block (fabm_set_block)
     int last_hk = -1;                  // run by the last solve (fabm_last_history_kernel)
     int chunk_ctas = 0;                // split-k CTA target of the CUDA-core history kernels (0: auto)
     int sm_reserve = -1;               // SMs kept free of tensor-history CTAs (-1: automatic)
@@ -858,7 +860,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     FABM_CUDA_TRY(need(s->nEach, (size_t)B));
     FABM_CUDA_TRY(need(s->status, 1));
     s->cl_size = 0;
-    if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0) {
+    if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0 && !s->direct) {
         plan_cluster(s, B, cols, s->plan_N > 0 ? s->plan_N : N);
         const int n = s->cl_n;
         const int64_t nsb = (Nmax + n - 1) / n;
@@ -1439,6 +1441,7 @@ fabm_status fabm_set_block(fabm_solver *s, int L)
     std::unique_lock<std::mutex> lk(s->busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(FABM_EBUSY, "solver in use by another thread");
     s->hist_kernel = hk;
+    s->direct = hk == FABM_HIST_FP64;
     s->L = L;
     return FABM_OK;
 }
@@ -1458,6 +1461,7 @@ fabm_status fabm_set_history_kernel(fabm_solver *s, int kernel)
     std::unique_lock<std::mutex> lk(s->busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(FABM_EBUSY, "solver in use by another thread");
     s->hist_kernel = kernel;
+    s->direct = false;
     s->L = (kernel == FABM_HIST_TENSOR || kernel == FABM_HIST_TENSOR_WIDE ||
             (kernel == FABM_HIST_AUTO && s->precision == FABM_SPLIT))
                ? kSplitSeg
@@ -1579,8 +1583,9 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
     std::vector<int64_t> ne((size_t)B, n1);
     const int keep_kernel = s->hist_kernel, keep_ctas = s->chunk_ctas, keep_res = s->sm_reserve;
     const int keep_L = s->L;
-    const bool keep_timing = s->timing;
+    const bool keep_timing = s->timing, keep_direct = s->direct;
     s->timing = false;
+    s->direct = false;  // direct sums are the candidates with a CTA target
     s->plan_N = s->N;  // the probes take the full solve's lag and recurrence layout
     double best = 1e300;
     Cand pick{keep_kernel, keep_ctas};
@@ -1648,7 +1653,7 @@ fabm_status fabm_autotune(fabm_solver *s, int64_t B, const double *y0, const dou
     s->plan_N = 0;
     if (st != FABM_OK) {
         s->hist_kernel = keep_kernel, s->chunk_ctas = keep_ctas, s->sm_reserve = keep_res;
-        s->L = keep_L;
+        s->L = keep_L, s->direct = keep_direct;
         return st;
     }
     apply(pick);
