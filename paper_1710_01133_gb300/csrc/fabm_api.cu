@@ -189,9 +189,12 @@ struct fabm_solver {
     DevBuf<float2> auxb;       // tensor path: forcing tables of kAuxRing blocks
     DevBuf<float2> parff, y0ff; // tensor path: float-float parameters and y_0
     bool cols_ready = false;  // tensor path: its recurrence kernels' limits are set
-    DevBuf<unsigned int> err;  // split: timeout flag
-    DevBuf<int64_t> nEach;
-    DevBuf<unsigned long long> status;
+    // the status words of a solve and N_each behind them, written by one copy and
+    // the status words read by one: first non-finite step (all ones: none), waits
+    // that gave up, N_each[B]
+    DevBuf<int64_t> head;
+    unsigned long long *status() const { return reinterpret_cast<unsigned long long *>(head.p); }
+    unsigned int *err() const { return reinterpret_cast<unsigned int *>(head.p + 1); }
     // sR: recurrence; sG, sG2: far history (the CUDA-core history of odd blocks
     // runs on sG2, so that consecutive blocks' history launches overlap)
     // sC: device-to-host copies of finished rows while the solve goes on
@@ -250,9 +253,9 @@ struct fabm_solver {
         wBl.release(), wAl.release(), wDl.release();
         wBf.release(), wAf.release(), wBff.release(), wAff.release(), wDff.release();
         F.release(), Ff.release(), Ystage.release(), G.release(), part.release();
-        Fs.release(), Fe.release(), spart.release(), auxb.release(), err.release();
+        Fs.release(), Fe.release(), spart.release(), auxb.release();
         parff.release(), y0ff.release();
-        y0.release(), par.release(), nEach.release(), status.release();
+        y0.release(), par.release(), head.release();
         for (auto &e : evR)
             if (e) cudaEventDestroy(e);
         for (auto &e : evG)
@@ -535,7 +538,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                 }));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, fs, flops, [&] {
                     return launch_hist_far(s->Fs2.p, s->Fe2.p, s->wH2.p, s->wHe2.p, C,
-                                           (int)(C - 1), n_far, n_ct, (int)cols, fw, s->err.p,
+                                           (int)(C - 1), n_far, n_ct, (int)cols, fw, s->err(),
                                            s->wait_cycles, fs);
                 }));
                 FABM_CUDA_TRY(cudaEventRecord(s->evFK[C & 1], fs));
@@ -551,7 +554,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             const int n_nc = std::min(n_near, s->near_chunks);
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sR, nflops, [&] {
                 return launch_hist_split(s->Fs.p, s->Fe.p, s->wH.p, s->wHe.p, c, (int)lo, n_near,
-                                         0, n_nc, n_ct, (int)cols, s->spart.p, s->err.p,
+                                         0, n_nc, n_ct, (int)cols, s->spart.p, s->err(),
                                          s->wait_cycles, s->sR);
             }));
             if (C >= 2) {
@@ -573,7 +576,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                 FABM_CUDA_TRY(cudaStreamWaitEvent(s->sG, s->evR[(c - 2) % kEvRing], 0));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sG, flops, [&] {
                     return launch_hist_split(s->Fs.p, s->Fe.p, s->wH.p, s->wHe.p, c, 0, (int)(c - 1),
-                                             0, n_far, n_ct, (int)cols, s->spart.p, s->err.p,
+                                             0, n_far, n_ct, (int)cols, s->spart.p, s->err(),
                                              s->wait_cycles, s->sG);
                 }));
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, s->sG, 0.0, [&] {
@@ -586,7 +589,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             const double nflops = 4.0 * L * (double)L * (double)cols;
             FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sR, nflops, [&] {
                 return launch_hist_split(s->Fs.p, s->Fe.p, s->wH.p, s->wHe.p, c, (int)(c - 1), 1,
-                                         split_chunks, 1, n_ct, (int)cols, s->spart.p, s->err.p,
+                                         split_chunks, 1, n_ct, (int)cols, s->spart.p, s->err(),
                                          s->wait_cycles, s->sR);
             }));
             if (n_far > 0) FABM_CUDA_TRY(cudaStreamWaitEvent(s->sR, s->evG[c % 3], 0));
@@ -669,7 +672,7 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
             }
             if (x2)
                 return launch_cluster_fp64(s->rhs, bt, w, s->k, c, L, 1, x2_alone,
-                                           static_cast<const double *>(Gc), X64, s->err.p,
+                                           static_cast<const double *>(Gc), X64, s->err(),
                                            s->wait_cycles, s->sR);
             return launch_recur(s->rhs, bt, w, s->k, c, L, lag, s->precision == FABM_SPLIT, alone,
                                 static_cast<const double *>(Gc), s->sR);
@@ -785,7 +788,7 @@ fabm_status enqueue_clusters(fabm_solver *s, const DevBatch &bt, const DevWeight
         const double near = (double)(T > 0 ? n : 0) + 0.5 * (double)(hi - lo + 1);
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_RECURRENCE, s->sR, 4.0 * (double)(hi - lo) * near * cols, [&] {
             return launch_cluster_fp64(s->rhs, bt, w, s->k, T, n, s->cl_size, s->cl_size > 1, G, X,
-                                       s->err.p,
+                                       s->err(),
                                        s->wait_cycles, s->sR);
         }));
         FABM_CUDA_TRY(cudaEventRecord(s->evR[T % kEvRing], s->sR));
@@ -817,7 +820,9 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     s->launches = 0;
 
     // host-side inputs: per-trajectory steps and parameter rows
-    std::vector<int64_t> ne(B);
+    std::vector<int64_t> head((size_t)B + 2, 0);
+    head[0] = -1;  // no non-finite step yet; no wait has given up
+    int64_t *ne = head.data() + 2;
     int64_t Nmax = 0;
     bool all_full = true;
     for (int64_t b = 0; b < B; ++b) {
@@ -857,8 +862,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     if (!out_on_device) FABM_CUDA_TRY(need(s->Ystage, (size_t)B * (N + 1) * dim));
     FABM_CUDA_TRY(need(s->y0, (size_t)B * dim * 2));  // y0, then y1
     FABM_CUDA_TRY(need(s->par, (size_t)B * kMaxParams));
-    FABM_CUDA_TRY(need(s->nEach, (size_t)B));
-    FABM_CUDA_TRY(need(s->status, 1));
+    FABM_CUDA_TRY(need(s->head, (size_t)B + 2));
     s->cl_size = 0;
     if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0 && !s->direct) {
         plan_cluster(s, B, cols, s->plan_N > 0 ? s->plan_N : N);
@@ -893,10 +897,6 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
             s->release_superblocks();
             s->cl_size = 0;
         }
-        if (s->cl_size) {
-            FABM_CUDA_TRY(need(s->err, 1));
-            FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
-        }
     }
     if (!s->cl_size) FABM_CUDA_TRY(need(s->G, (size_t)3 * 2 * L * cols));
     // two partial buffers: the history launches of blocks c and c+1 may overlap
@@ -907,8 +907,6 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         // cold caches, 28.4 -> 20.5 us a block)
         FABM_CUDA_TRY(s->part.ensure((size_t)2 * max_chunks * part_per_chunk));
         if (rhs_has_forcing(s->rhs, dim)) FABM_CUDA_TRY(s->Xrow.ensure((size_t)2 * L * B));
-        FABM_CUDA_TRY(s->err.ensure(1));
-        FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
     }
     if (hk == FABM_HIST_FP32C) {
         FABM_CUDA_TRY(s->spart.ensure((size_t)2 * max_chunks * part_per_chunk));
@@ -973,8 +971,6 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         }
         if (rhs_has_forcing(s->rhs, dim))
             FABM_CUDA_TRY(s->auxb.ensure((size_t)kAuxRing * kSplitSeg * B));
-        FABM_CUDA_TRY(s->err.ensure(1));
-        FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
     }
     double *Y = out_on_device ? out : s->Ystage.p;
     // a large output into pinned host memory, every trajectory to N: copied
@@ -1008,16 +1004,15 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         FABM_CUDA_TRY(cudaMemsetAsync(s->y0.p + B * dim, 0, sizeof(double) * B * dim, s->sR));
     FABM_CUDA_TRY(cudaMemcpyAsync(s->par.p, par.data(), sizeof(double) * par.size(),
                                   cudaMemcpyHostToDevice, s->sR));
-    FABM_CUDA_TRY(cudaMemcpyAsync(s->nEach.p, ne.data(), sizeof(int64_t) * B,
+    FABM_CUDA_TRY(cudaMemcpyAsync(s->head.p, head.data(), sizeof(int64_t) * head.size(),
                                   cudaMemcpyHostToDevice, s->sR));
-    FABM_CUDA_TRY(cudaMemsetAsync(s->status.p, 0xff, sizeof(unsigned long long), s->sR));
 
     DevBatch bt{};
     bt.dim = dim;
     bt.B = (int)B;
     bt.cols = (int)cols;
     bt.N = N;
-    bt.N_each = s->nEach.p;
+    bt.N_each = s->head.p + 2;
     bt.y0 = s->y0.p;
     bt.y1 = s->alpha > 1.0 ? s->y0.p + B * dim : nullptr;
     bt.params = s->par.p;
@@ -1025,7 +1020,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     bt.Ff = hk == FABM_HIST_FP32C ? s->Ff.p : nullptr;
     bt.ldF = cols;
     bt.Y = Y;
-    bt.status = s->status.p;
+    bt.status = s->status();
     DevWeights w{s->wB.p, s->wA.p, s->wD.p, s->w_ext, s->multi ? s->w_ext + 1 : 0};
 
     // what a captured graph holds: every choice that shapes the launches and every
@@ -1036,7 +1031,7 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         (uintptr_t)(s->sm_reserve + 1), (uintptr_t)s->cols_warps, (uintptr_t)Y,
         (uintptr_t)s->F.p, (uintptr_t)s->Ff.p, (uintptr_t)s->G.p, (uintptr_t)s->part.p, (uintptr_t)s->Fs.p,
         (uintptr_t)s->Fe.p, (uintptr_t)s->spart.p, (uintptr_t)s->y0.p, (uintptr_t)s->par.p,
-        (uintptr_t)s->nEach.p, (uintptr_t)s->status.p, (uintptr_t)s->err.p, (uintptr_t)s->auxb.p,
+        (uintptr_t)s->head.p, (uintptr_t)s->auxb.p,
         (uintptr_t)s->out_stream, (uintptr_t)s->out_group, (uintptr_t)s->wait_cycles,
         (uintptr_t)s->wide, (uintptr_t)split_chunks, (uintptr_t)far_chunks, (uintptr_t)s->Fs2.p, (uintptr_t)s->Fe2.p,
         (uintptr_t)s->fpart.p, (uintptr_t)s->fsum.p, (uintptr_t)s->near_chunks,
@@ -1061,26 +1056,21 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         FABM_CUDA_TRY(need(s->psg, n_sg));
         FABM_CUDA_TRY(need(s->pdone, (size_t)nblk * ncg));
         FABM_CUDA_TRY(need(s->prdone, (size_t)B));
-        FABM_CUDA_TRY(s->err.ensure(1));
         s->recs.clear();
         FABM_CUDA_TRY(cudaMemsetAsync(s->psg.p, 0, sizeof(int) * n_sg, s->sR));
         FABM_CUDA_TRY(cudaMemsetAsync(s->pdone.p, 0, sizeof(int) * nblk * ncg, s->sR));
         FABM_CUDA_TRY(cudaMemsetAsync(s->prdone.p, 0, sizeof(int) * B, s->sR));
-        FABM_CUDA_TRY(cudaMemsetAsync(s->err.p, 0, sizeof(unsigned int), s->sR));
         s->sample_now = true;
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
                                    [&] { return launch_init(s->rhs, bt, s->sR); }));
         const double flops = 2.0 * (double)Nmax * (double)Nmax * (double)cols;
         FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, s->sR, flops, [&] {
             return launch_persist_fp64(s->rhs, bt, w, s->k, nblk, grid, pchunks, s->ppart.p,
-                                       s->pspart.p, s->psg.p, s->pdone.p, s->prdone.p, s->err.p,
+                                       s->pspart.p, s->psg.p, s->pdone.p, s->prdone.p, s->err(),
                                        s->wait_cycles, s->sR);
         }));
         FABM_CUDA_TRY(cudaStreamSynchronize(s->sR));
         FABM_CUDA_TRY(collect_timing(s, s->recs));
-        unsigned int tout = 0;
-        FABM_CUDA_TRY(cudaMemcpy(&tout, s->err.p, sizeof tout, cudaMemcpyDeviceToHost));
-        if (tout) return fail(FABM_ETIMEOUT, "the persistent solve gave up waiting on a flag");
     } else if (!s->use_graphs) {
         s->recs.clear();
         // the side streams start after this solve's inputs are on the device
@@ -1150,13 +1140,12 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     }
 
 
-    unsigned long long st = 0;
-    FABM_CUDA_TRY(cudaMemcpy(&st, s->status.p, sizeof st, cudaMemcpyDeviceToHost));
-    if (split || s->cl_size || hk == FABM_HIST_X2) {  // bounded waits
-        unsigned int tout = 0;
-        FABM_CUDA_TRY(cudaMemcpy(&tout, s->err.p, sizeof tout, cudaMemcpyDeviceToHost));
-        if (tout) return fail(FABM_ETIMEOUT, "a history kernel gave up waiting on a barrier");
-    }
+    unsigned long long end[2] = {};  // status words
+    FABM_CUDA_TRY(cudaMemcpy(end, s->head.p, sizeof end, cudaMemcpyDeviceToHost));
+    const unsigned long long st = end[0];
+    if (end[1])  // bounded waits
+        return fail(FABM_ETIMEOUT, hk == FABM_HIST_FP64_PERSIST ? "the persistent solve gave up waiting on a flag"
+                                                                : "a kernel gave up waiting on a barrier or a value");
 
     if (!out_on_device && !s->out_stream) {
         const size_t row = (size_t)(N + 1) * dim;
