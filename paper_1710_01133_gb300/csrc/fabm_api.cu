@@ -484,13 +484,10 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                         : x2_alone        ? 152 - bt.B
                                           : auto_chunk_ctas(hk, cols);
     const int n_gbuf = lag + 1;  // G of block c is read by R(c) until H(c + lag + 1) starts
+    const FFInputs ff = split ? FFInputs{s->parff.p, s->y0ff.p} : FFInputs{};
     s->sample_now = true;
     FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_INIT, s->sR, 0.0,
-                               [&] { return launch_init(s->rhs, bt, s->sR, split); }));
-    if (split) {
-        s->launches += 2;
-        FABM_CUDA_TRY(launch_ff_inputs(bt, s->parff.p, s->y0ff.p, s->sR));
-    }
+                               [&] { return launch_init(s->rhs, bt, s->sR, split, ff); }));
     // tensor path with forcing: the tables of the time-only part of f, on sG2,
     // up to kAuxRing - 1 blocks ahead of the recurrence
     const bool tables = split && rhs_has_forcing(s->rhs, bt.dim);

@@ -78,9 +78,15 @@ struct StepConsts {
 cudaError_t launch_weights(double alpha, int64_t N, double inv_g1, double inv_g2, double *B,
                            double *A, double *D, cudaStream_t st);
 
+// Float-float copies of the parameters, [B][kMaxParams], and of y_0, [cols], for
+// the recurrence of the tensor-history path, or none.
+struct FFInputs {
+    float2 *par = nullptr, *y0 = nullptr;
+};
 // y_0 into Y, f_0 = f(0, y_0) into F row 0 (as a float-float pair when
-// f_pairs, the tensor-history path).
-cudaError_t launch_init(int rhs, const DevBatch &bt, cudaStream_t st, bool f_pairs = false);
+// f_pairs, the tensor-history path), and the copies asked for.
+cudaError_t launch_init(int rhs, const DevBatch &bt, cudaStream_t st, bool f_pairs = false,
+                        const FFInputs &ff = {});
 
 // a2 (FP64): partial far-history sums of target block c from the points
 // k in [0, (c-lag)L), split into n_chunks chunks of kc points.
@@ -197,7 +203,7 @@ struct HistIn {
     bool near_as_chunk = false;  // one near chunk, added as the chunk after those in G
 };
 struct ColsIn {
-    const float2 *par, *y0;  // float-float copies of the parameters and y_0 (launch_ff_inputs)
+    const float2 *par, *y0;  // float-float copies of the parameters and y_0 (launch_init)
     const float2 *X;         // table of the time-only part of f for block c
                              // (launch_aux_table), required when rhs_has_forcing(rhs)
     __nv_bfloat16 *Fs;       // where the slices and exponents of segment c go (all
@@ -207,8 +213,6 @@ struct ColsIn {
 cudaError_t launch_recur_cols(int rhs, const DevBatch &bt, const float2 *WB, const float2 *WA,
                               const float2 *WD, const StepConsts &k, int64_t c, const HistIn &hin,
                               const ColsIn &in, int warps_per_cta, cudaStream_t st);
-// par[B][kMaxParams], y0[cols] as float-float pairs.
-cudaError_t launch_ff_inputs(const DevBatch &bt, float2 *par, float2 *y0, cudaStream_t st);
 // The right-hand side has a time-dependent part (forcing).
 bool rhs_has_forcing(int rhs, int dim);
 // X[a][b] = aux(t_{64c+1+a}, params of b) as float-float pairs, a < 64, b < B.

@@ -5,10 +5,10 @@ namespace fabm {
 namespace {
 
 template <class Rhs, int D>
-__global__ void init_kernel(DevBatch bt, bool f_pairs)
+__global__ void init_kernel(DevBatch bt, bool f_pairs, FFInputs ff)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < bt.B) init_one<Rhs, D>(bt, b, f_pairs);
+    if (b < bt.B) init_one<Rhs, D>(bt, b, f_pairs, ff);
 }
 
 template <class Rhs, int D, int TPL, bool SPLIT, int LAG>
@@ -44,12 +44,12 @@ bool launch_recur_t(int rhs, const DevBatch &bt, const DevWeights &w, const Step
 
 }  // namespace
 
-cudaError_t launch_init(int rhs, const DevBatch &bt, cudaStream_t st, bool f_pairs)
+cudaError_t launch_init(int rhs, const DevBatch &bt, cudaStream_t st, bool f_pairs, const FFInputs &ff)
 {
     const int threads = 128;
     const unsigned blocks = (unsigned)((bt.B + threads - 1) / threads);
     bool ok = dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
-        init_kernel<R, D><<<blocks, threads, 0, st>>>(bt, f_pairs);
+        init_kernel<R, D><<<blocks, threads, 0, st>>>(bt, f_pairs, ff);
     });
     return ok ? cudaGetLastError() : cudaErrorInvalidValue;
 }

@@ -53,7 +53,7 @@ __device__ inline bool finite_bits(double x)
 
 // y_0 and f_0 = f(0, y_0) of trajectory b; f_pairs: F holds float-float pairs.
 template <class Rhs, int D>
-__device__ inline void init_one(const DevBatch &bt, int b, bool f_pairs = false)
+__device__ inline void init_one(const DevBatch &bt, int b, bool f_pairs = false, const FFInputs &ff = {})
 {
     double y[D], p[kMaxParams];
 #pragma unroll
@@ -62,6 +62,18 @@ __device__ inline void init_one(const DevBatch &bt, int b, bool f_pairs = false)
     for (int i = 0; i < D; ++i) y[i] = bt.y0[(int64_t)b * D + i];
     const double aux = Rhs::aux(0.0, p);
     bool ok = true;
+    if (ff.par) {
+#pragma unroll
+        for (int i = 0; i < kMaxParams; ++i) {
+            const FF v = ff_from_double(p[i]);
+            ff.par[(int64_t)b * kMaxParams + i] = make_float2(v.hi, v.lo);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            const FF v = ff_from_double(y[i]);
+            ff.y0[(int64_t)b * D + i] = make_float2(v.hi, v.lo);
+        }
+    }
 #pragma unroll
     for (int i = 0; i < D; ++i) {
         const double f = Rhs::template one<D>(i, y, p, aux);

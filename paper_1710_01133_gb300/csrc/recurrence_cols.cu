@@ -526,26 +526,6 @@ cudaError_t prepare_recur_cols(int rhs, int dim)
 
 int recur_cols_warps(int dim, int64_t B) { return (int)((B + kWarp / dim - 1) / (kWarp / dim)); }
 
-namespace {
-__global__ void ff_inputs_kernel(const double *__restrict__ x, int64_t n, float2 *__restrict__ y)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const FF v = ff_from_double(x[e]);
-        y[e] = make_float2(v.hi, v.lo);
-    }
-}
-}  // namespace
-
-cudaError_t launch_ff_inputs(const DevBatch &bt, float2 *par, float2 *y0, cudaStream_t st)
-{
-    auto blocks = [](int64_t n) { return (unsigned)std::min<int64_t>((n + 127) / 128, 152 * 8); };
-    const int64_t np = (int64_t)bt.B * kMaxParams;
-    ff_inputs_kernel<<<blocks(np), 128, 0, st>>>(bt.params, np, par);
-    ff_inputs_kernel<<<blocks(bt.cols), 128, 0, st>>>(bt.y0, bt.cols, y0);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_recur_cols(int rhs, const DevBatch &bt, const float2 *WB, const float2 *WA,
                               const float2 *WD, const StepConsts &k, int64_t c, const HistIn &hin,
                               const ColsIn &in, int warps_per_cta, cudaStream_t st)
