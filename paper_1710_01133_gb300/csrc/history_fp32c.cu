@@ -12,29 +12,41 @@
 // order and rounds once to double.  This suits batches with few columns,
 // where a 128-column tensor tile would be mostly padding; wide batches use
 // the tensor-core kernel.
+#include <algorithm>
+
 #include "history_blocks.cuh"
 
 namespace fabm {
 namespace {
 
-// grid = (ceil(n_chunks / pack), ceil(cols / kColsPerCta)); block = pack groups of
-// 32 * kColsPerCta threads, one chunk each.
+// grid = (ceil(n_chunks / PACK), ceil(cols / kColsPerCta)); block = PACK groups of
+// 32 * kColsPerCta threads, one chunk each.  One group per CTA is a kernel of its
+// own: with the groups' barriers and limits it took 79 instead of 56 registers (127
+// instead of 96 with several orders): LCR of two orders, 1000 x 1000, 1.58 ms, now
+// 1.39 (with the recurrence on the same SMs, recurrence.cu).
 constexpr int kGroup = kWarp * hist::kColsPerCta;
 constexpr int kPack = 3;  // groups per CTA where the launch leaves SMs free
-template <bool MULTI>
-__global__ void __launch_bounds__(kPack *kGroup)
+template <bool MULTI, int PACK>
+__global__ void __launch_bounds__(PACK *kGroup)
     hist_fp32c_kernel(const double *__restrict__ F, const float *__restrict__ Ff, int64_t ldF,
                       int cols, const float *__restrict__ WB, const float *__restrict__ WA,
                       int64_t c, int64_t kc, int64_t k_end, int n_chunks, float2 *__restrict__ part,
                       int64_t wstride, int dim)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int g = threadIdx.x / kGroup, chunk = blockIdx.x * (blockDim.x / kGroup) + g;
-    if (chunk >= n_chunks) return;
-    hist::f32c::hist_fp32c_chunk<MULTI>(
-        F, Ff, ldF, cols, WB, WA, c, kc, k_end, part, chunk, blockIdx.y * hist::kColsPerCta, wstride,
-        dim, threadIdx.x % kGroup, reinterpret_cast<hist::f32c::Tiles<MULTI> *>(smem)[g],
-        [g] { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroup) : "memory"); });
+    const int col0 = blockIdx.y * hist::kColsPerCta;
+    if constexpr (PACK == 1) {
+        __shared__ hist::f32c::Tiles<MULTI> tl;
+        hist::f32c::hist_fp32c_chunk<MULTI>(F, Ff, ldF, cols, WB, WA, c, kc, k_end, part, blockIdx.x, col0,
+                                            wstride, dim, threadIdx.x, tl, [] { __syncthreads(); });
+    } else {
+        extern __shared__ __align__(16) unsigned char smem[];
+        const int g = threadIdx.x / kGroup, chunk = blockIdx.x * PACK + g;
+        if (chunk >= n_chunks) return;
+        hist::f32c::hist_fp32c_chunk<MULTI>(
+            F, Ff, ldF, cols, WB, WA, c, kc, k_end, part, chunk, col0, wstride, dim,
+            threadIdx.x % kGroup, reinterpret_cast<hist::f32c::Tiles<MULTI> *>(smem)[g],
+            [g] { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroup) : "memory"); });
+    }
 }
 
 __global__ void to_float_kernel(const double *__restrict__ x, int64_t n, float *__restrict__ y)
@@ -68,23 +80,23 @@ cudaError_t launch_hist_fp32c(const DevBatch &bt, const float *WBf, const float 
     // its own, and so does the recurrence.  The chunks and their sums stay as
     // they are.
     const int groups = (bt.cols + hist::kColsPerCta - 1) / hist::kColsPerCta;
-    const int pack = alone ? kPack : 1;
-    auto run = [&](auto kernel, size_t tiles, int64_t stride, int dim) -> cudaError_t {
-        const size_t packed = tiles * kPack > kAloneSmem ? tiles * kPack : kAloneSmem;
-        const size_t smem = alone ? packed : tiles;
-        if (smem > 48 * 1024) {
-            // the same limit in every call: a solver on another thread may be about
-            // to launch this kernel with the other size
+    auto run = [&]<bool MULTI, int PACK>(int64_t stride, int dim) -> cudaError_t {
+        auto kernel = hist_fp32c_kernel<MULTI, PACK>;
+        size_t smem = 0;
+        if constexpr (PACK > 1) {
+            smem = std::max(sizeof(hist::f32c::Tiles<MULTI>) * PACK, kAloneSmem);
             const cudaError_t e =
-                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)packed);
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kernel<<<dim3((unsigned)((n_chunks + pack - 1) / pack), (unsigned)groups), pack * kGroup, smem, st>>>(
+        kernel<<<dim3((unsigned)((n_chunks + PACK - 1) / PACK), (unsigned)groups), PACK * kGroup, smem, st>>>(
             bt.F, bt.Ff, bt.ldF, bt.cols, WBf, WAf, c, kc, k_end, n_chunks, part, stride, dim);
         return cudaGetLastError();
     };
-    if (wstride) return run(hist_fp32c_kernel<true>, sizeof(hist::f32c::Tiles<true>), wstride, bt.dim);
-    return run(hist_fp32c_kernel<false>, sizeof(hist::f32c::Tiles<false>), 0, 1);
+    if (wstride)
+        return alone ? run.template operator()<true, kPack>(wstride, bt.dim)
+                     : run.template operator()<true, 1>(wstride, bt.dim);
+    return alone ? run.template operator()<false, kPack>(0, 1) : run.template operator()<false, 1>(0, 1);
 }
 
 bool fp32c_alone(int n_chunks, int cols, int B)
