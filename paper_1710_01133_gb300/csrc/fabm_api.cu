@@ -956,8 +956,17 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
         // does not wait for far CTAs to retire (one CTA sums its segments in turn)
         const int far_free = 152 - 2 * n_ct * far_chunks;
         s->near_chunks = std::clamp(far_free / n_ct, 1, 3);
-        // one team of warps per CTA unless set; the lane-per-target layout on request
-        s->cols_warps = s->rec_layout == FABM_REC_TARGETS ? 0 : std::max(1, s->rec_warps);
+        // one team of warps per CTA unless set; a lane per target on request, and for
+        // narrow batches of one component, whose step is short beside what a team hands
+        // over (us, targets / columns; linear: 300 x 1000 473 / 581, 1000 x 1000 551 /
+        // 596, 1300 x 1000 654 / 613, 1300 x 4000 2714 / 2836, 2000 x 4000 3397 / 3177;
+        // forced: 300 x 4000 2202 / 2617, 500 x 1000 709 / 716, 1000 x 1000 805 / 728;
+        // Lorenz type 300 x 1000 740 / 659)
+        const bool forcing = rhs_has_forcing(s->rhs, dim);
+        const bool targets = s->rec_layout == FABM_REC_TARGETS ||
+                             (s->rec_layout == FABM_REC_AUTO && dim == 1 && !columns &&
+                              cwarps <= (forcing ? 12 : nplan >= 3072.0 ? 50 : 32));
+        s->cols_warps = targets ? 0 : std::max(1, s->rec_warps);
         if (!s->cols_ready) {  // here, as a narrow batch never needs it (0.1 ms)
             FABM_CUDA_TRY(prepare_recur_cols(s->rhs, dim));
             s->cols_ready = true;
