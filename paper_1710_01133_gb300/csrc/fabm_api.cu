@@ -445,6 +445,28 @@ int history_lag(int hk, int64_t N, int64_t cols)
     return 1;
 }
 
+// One or two blocks of 32 steps for many trajectories of few components: every
+// point is within the lag block, so there is no history to launch, and a warp per
+// component (recur_block) fills the SMs better than the cluster kernel's nine warps
+// per trajectory.  Measured, us, cluster kernel / recur_block: scalar, 64 steps, 400
+// trajectories 49 / 57, 700 73 / 63, 4096 191 / 162, 10,000 409 / 387; forced
+// oscillator, 32 steps, 400 57 / 58, 1000 97 / 82, 10,000 520 / 493, 45 steps and
+// 4096 301 / 338; Lorenz type, 32 steps, 1000 100 / 111.
+bool short_solve(int dim, int64_t B, int64_t N)
+{
+    return B > 512 && N <= (dim == 1 ? 64 : dim == 2 ? 32 : 0);
+}
+
+// A forced scalar system of very many trajectories: the table of its forcing, a
+// launch of its own per superblock, is what the steps of so few superblocks wait for
+// (manufactured problem, us, superblocks / blocks of 32: 80 steps, 2048 trajectories
+// 237 / 229, 4096 395 / 374, 10,000 929 / 852; 160 steps, 4096 743 / 692; 200 steps
+// 972 / 1024).
+bool short_forced_scalar(const fabm_solver *s, int64_t B, int64_t N)
+{
+    return s->dim == 1 && B >= 4096 && N <= 160 && rhs_has_forcing(s->rhs, 1);
+}
+
 // FP64X2: a CTA's four warps share a chunk of its four columns, so that chunks may
 // be short; at_most: no more than want_ctas CTAs (one wave of an SM each).
 void plan_chunks_x2(int64_t k_end, int cols, int64_t max_chunks, int want_ctas, bool at_most,
@@ -871,7 +893,9 @@ fabm_status run_batch(fabm_solver *s, int64_t B, const double *y0, const double 
     FABM_CUDA_TRY(need(s->par, (size_t)B * kMaxParams));
     FABM_CUDA_TRY(need(s->head, (size_t)B + 2));
     s->cl_size = 0;
-    if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0 && !s->direct) {
+    if (hk == FABM_HIST_FP64 && s->chunk_ctas == 0 && !s->direct &&
+        !short_solve(dim, B, s->plan_N > 0 ? s->plan_N : Nmax) &&
+        !short_forced_scalar(s, B, s->plan_N > 0 ? s->plan_N : Nmax)) {
         plan_cluster(s, B, cols, s->plan_N > 0 ? s->plan_N : N);
         const int n = s->cl_n;
         const int64_t nsb = (Nmax + n - 1) / n;

@@ -1,0 +1,40 @@
+"""Which kernels take the steps of short solves (needs a GPU): both sides of each
+rule on lengths and batch sizes, against the oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+TOL_FP64 = 1e-12
+PARAMS = {"linear": (1.0,), "manufactured": (0.5, 1.0, 2.0), "duffing": (0.1, 1.2, 0.7),
+          "lorenz": (10.0, 28.0, 8 / 3)}
+
+
+def rel_err(got, ref):
+    scale = np.max(np.abs(ref), axis=-2, keepdims=True)
+    return float(np.max(np.abs(got - ref) / np.where(scale == 0, 1.0, scale)))
+
+
+def solve(gpu_lib, parity, rhs, dim, precision, B, N, tol, **kw):
+    y0 = 0.5 + np.linspace(-0.2, 0.2, B * dim).reshape(B, dim)
+    ne = np.full(B, N, dtype=np.int64)
+    ne[B // 2] = N // 2 + 1
+    with gpu_lib.Solver(rhs, dim, 0.9, 1e-3, N, PARAMS[rhs], precision=precision, **kw) as s:
+        got = s.solve_batch(y0, N_each=ne)
+        launches = s.last_launch_count
+    idx = np.array([0, B // 2, B - 1])
+    ref = oracle.solve_batch(rhs, 0.9, 1e-3, N, y0[idx], params=PARAMS[rhs], N_each=ne[idx])
+    for j, b in enumerate(idx):
+        parity(rel_err(got[b, : ne[b] + 1], ref[j, : ne[b] + 1]), tol, f"traj{b}")
+    return got, launches
+
+
+# launches: initial values, then one per block or superblock, and one per forcing table
+@pytest.mark.parametrize("rhs,dim,B,N,launches", [
+    ("linear", 1, 512, 64, 2), ("linear", 1, 513, 64, 3), ("linear", 1, 513, 65, 2), ("linear", 1, 600, 1, 2),
+    ("duffing", 2, 513, 32, 2), ("duffing", 2, 513, 33, 3), ("lorenz", 3, 600, 40, 2),
+    ("manufactured", 1, 4095, 128, 3), ("manufactured", 1, 4096, 128, 7)])
+def test_fp64(gpu_lib, parity, rhs, dim, B, N, launches):
+    assert solve(gpu_lib, parity, rhs, dim, "fp64", B, N, TOL_FP64)[1] == launches
