@@ -646,11 +646,12 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
                 double2 *xp = reinterpret_cast<double2 *>(s->part.p) + poff;
                 const DevWeightsLo wl{s->wBl.p, s->wAl.p, s->wDl.p};
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, gs, flops, [&] {
-                    return launch_hist_x2(bt, w, wl, c, lag, n_chunks, kc, x2_alone, xp, gs);
+                    return launch_hist_x2(bt, w, wl, c, lag, n_chunks, kc, x2_alone, xp, Gbuf, gs);
                 }));
-                FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, gs, 0.0, [&] {
-                    return launch_reduce_x2(xp, n_chunks, (int)cols, Gbuf, gs);
-                }));
+                if (n_chunks > 1)
+                    FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_COMBINE, gs, 0.0, [&] {
+                        return launch_reduce_x2(xp, n_chunks, (int)cols, Gbuf, gs);
+                    }));
             } else if (hk == FABM_HIST_FP32C) {
                 FABM_CUDA_TRY(timed_launch(s, FABM_KERNEL_HISTORY, gs, flops, [&] {
                     return launch_hist_fp32c(bt, s->wBf.p, s->wAf.p, w.stride, c, lag, n_chunks,

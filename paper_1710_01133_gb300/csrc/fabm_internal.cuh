@@ -309,11 +309,11 @@ cudaError_t launch_weights_x2(double alpha, int64_t n, double ig1_hi, double ig1
                               double *Al, double *Dh, double *Dl, cudaStream_t st);
 
 // a2 in double-double: partial far-history sums of target block c (32 targets)
-// over k < (c-lag)*32 as (hi, lo) pairs, n_chunks x 2 x 32 x cols; alone: one CTA
-// per SM.
+// over k < (c-lag)*32 as (hi, lo) pairs, n_chunks x 2 x 32 x cols; of a single chunk,
+// their sum G instead.  alone: one CTA per SM.
 cudaError_t launch_hist_x2(const DevBatch &bt, const DevWeights &w, const DevWeightsLo &wl,
                            int64_t c, int lag, int n_chunks, int64_t kc, bool alone, double2 *part,
-                           cudaStream_t st);
+                           double *G, cudaStream_t st);
 // a3: G = sum over chunks in double-double, rounded once to double.
 cudaError_t launch_reduce_x2(const double2 *part, int n_chunks, int cols, double *G, cudaStream_t st);
 

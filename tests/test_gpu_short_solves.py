@@ -38,3 +38,15 @@ def solve(gpu_lib, parity, rhs, dim, precision, B, N, tol, **kw):
     ("manufactured", 1, 4095, 128, 3), ("manufactured", 1, 4096, 128, 7)])
 def test_fp64(gpu_lib, parity, rhs, dim, B, N, launches):
     assert solve(gpu_lib, parity, rhs, dim, "fp64", B, N, TOL_FP64)[1] == launches
+
+
+@pytest.mark.parametrize("rhs,dim,B,N", [("linear", 1, 4861, 200), ("manufactured", 1, 4900, 97), ("lorenz", 3, 1621, 170)])
+def test_fp64x2_single_chunk(gpu_lib, parity, rhs, dim, B, N):
+    """From 4861 columns on a block's history is one chunk, which writes the rounded
+    sums itself; they are those of a narrow batch's chunks, bit for bit (sums of about
+    100 bits before the one rounding)."""
+    got, _ = solve(gpu_lib, parity, rhs, dim, "fp64x2", B, N, TOL_FP64)
+    y0 = 0.5 + np.linspace(-0.2, 0.2, B * dim).reshape(B, dim)
+    with gpu_lib.Solver(rhs, dim, 0.9, 1e-3, N, PARAMS[rhs], precision="fp64x2") as s:
+        for b in (0, B - 1):
+            assert np.array_equal(got[b], s.solve_batch(y0[b : b + 1])[0])
