@@ -46,8 +46,12 @@ constexpr int kWin = kTile + kL;
 __device__ __forceinline__ int exp_field(unsigned hi) { return (int)(hi >> 20); }
 __device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
-// The power of two with exponent field e, kept finite and away from subnormals: a
-// sum beyond the range ends as an infinity or a NaN as it would anyway.
+// The power of two with exponent field e, kept finite and away from subnormals.
+// Where the rule asks for a field beyond kTopField, terms scaled down by kScaleBits
+// are added instead, so that sums up to the end of the range stay finite and exact.
+constexpr int kTopField = 2046;
+constexpr int kScaleBits = 64;
+constexpr double kScaleDown = 0x1p-64, kScaleUp = 0x1p64;
 __device__ __forceinline__ double pow2_field(int e)
 {
     e = e < 64 ? 64 : (e > 2046 ? 2046 : e);
@@ -102,6 +106,42 @@ union Smem {
     Tiles t;
     Sums s;
 };
+
+// The sums of hist_x2_kernel's chunk k0 .. k1-1 where values are so large (|f| from
+// about 2^1005 on) that M would pass the end of the range: one thread per sum, terms
+// scaled down, products with their errors and TwoSum.  Out of line, as the test costs
+// a solve of ordinary values under 1 % this way and 2 to 5 % with the scaling inside the
+// kernel's loop.
+template <bool MULTI>
+__device__ __noinline__ void top_chunk(const double *F, int64_t ldF, int cols, const double *WBh,
+                                       const double *WBl, const double *WAh, const double *WAl,
+                                       int64_t c, int64_t k0, int64_t k1, double2 *part,
+                                       int64_t wstride, int dim, double *G)
+{
+    const int col0 = blockIdx.y * kCols, ncol = min(kCols, cols - col0);
+    for (int o = threadIdx.x; o < ncol * 2 * kWarp; o += kWarp * kWarps) {
+        const int q = o / (2 * kWarp), kind = o / kWarp % 2, t = o % kWarp;
+        const int64_t col = col0 + q, wo = (MULTI ? col % dim * wstride : 0) + c * kL + 1 + t;
+        const double *wh = (kind ? WAh : WBh) + wo, *wl = (kind ? WAl : WBl) + wo;
+        unsigned mx = 0;
+        for (int64_t k = k0; k < k1; ++k) mx = max(mx, abs_hi(F[k * ldF + col]));
+        const bool down = exp_field(mx) > 1023;
+        double hi = 0.0, lo = 0.0;
+        for (int64_t k = k0; k < k1; ++k) {
+            const double f = F[k * ldF + col] * (down ? kScaleDown : 1.0), p = wh[-k] * f;
+            const double e = fma(wh[-k], f, -p);
+            two_sum(hi, lo, p);
+            lo += e;
+            lo = fma(wl[-k], f, lo);
+        }
+        if (down) hi *= kScaleUp, lo *= kScaleUp;
+        const int64_t out = (kind * kL + t) * (int64_t)cols + col;
+        if (G)
+            G[out] = hi + lo;
+        else
+            part[(int64_t)blockIdx.x * 2 * kL * cols + out] = make_double2(hi, lo);
+    }
+}
 
 // grid = (n_chunks, ceil(cols / 4)); block = 128.  Chunk `chunk` covers the
 // points [chunk*kc, min((chunk+1)*kc, k_end)) of target block c (targets
@@ -172,10 +212,17 @@ __global__ void __launch_bounds__(kWarp *kWarps)
         // |w f| < 2^(ef + ew - 2044) for exponent fields ef, ew; nk terms; times four
         const int lg = 32 - __clz(nk);
         double M[kCols], sum[kCols][2];
+        bool top = false;
 #pragma unroll
         for (int q = 0; q < kCols; ++q) {
-            M[q] = pow2_field(exp_field(max_f[par][q]) + exp_field(max_w[par][MULTI ? q : 0]) - 1019 + lg);
+            const int e = exp_field(max_f[par][q]) + exp_field(max_w[par][MULTI ? q : 0]) - 1019 + lg;
+            top = top || e > kTopField;
+            M[q] = pow2_field(e);
             sum[q][0] = sum[q][1] = M[q];
+        }
+        if (top) {  // in every thread, or in none
+            top_chunk<MULTI>(F, ldF, cols, WBh, WBl, WAh, WAl, c, k0, k1, part, wstride, dim, G);
+            return;
         }
         const int j0 = w * nk / kWarps, j1 = (w + 1) * nk / kWarps;
         const int base = a + nk - 1;  // d - d_min for point t0+j: a + nk-1-j
@@ -258,7 +305,14 @@ __global__ void reduce_x2_kernel(const double2 *__restrict__ part, int n_chunks,
 #pragma unroll
             for (int off = R / 2; off > 0; off >>= 1)
                 mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            const double M = pow2_field(exp_field(mx) + 3 + lg);
+            int e = exp_field(mx) + 3 + lg;
+            const bool big = e > kTopField;  // the same in the output's lanes
+            if (big) {
+                e -= kScaleBits, lo *= kScaleDown;
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) v[u].x *= kScaleDown, v[u].y *= kScaleDown;
+            }
+            const double M = pow2_field(e);
             double s = M;
 #pragma unroll
             for (int u = 0; u < kBatch; ++u) {
@@ -267,10 +321,12 @@ __global__ void reduce_x2_kernel(const double2 *__restrict__ part, int n_chunks,
                 lo += v[u].y;
                 s = n;
             }
+            double x = s - M;
+            if (big) x *= kScaleUp, lo *= kScaleUp;
             if (one)
-                hi = s - M;
+                hi = x;
             else
-                two_sum(hi, lo, s - M);
+                two_sum(hi, lo, x);
         }
 #pragma unroll
         for (int off = R / 2; off > 0; off >>= 1) {
