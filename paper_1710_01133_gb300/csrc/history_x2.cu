@@ -215,8 +215,9 @@ __global__ void __launch_bounds__(kWarp *kWarps)
         bool top = false;
 #pragma unroll
         for (int q = 0; q < kCols; ++q) {
-            const int e = exp_field(max_f[par][q]) + exp_field(max_w[par][MULTI ? q : 0]) - 1019 + lg;
-            top = top || e > kTopField;
+            const int ef = exp_field(max_f[par][q]);
+            const int e = ef + exp_field(max_w[par][MULTI ? q : 0]) - 1019 + lg;
+            top = top || (e > kTopField && ef < 2047);  // infinities and NaNs stay what they are
             M[q] = pow2_field(e);
             sum[q][0] = sum[q][1] = M[q];
         }
