@@ -277,7 +277,9 @@ fabm_status fabm_set_graphs(fabm_solver *s, int enable);
  * (solver work space, server admissions; process-wide) fail as if the device
  * were out of memory, without calling the allocator: the call that needed the
  * memory returns FABM_ENOMEM (a server marks that request failed with
- * FABM_ENOMEM), and later calls allocate normally.  n = 0 cancels what is left.
+ * FABM_ENOMEM) or does without it, and later calls allocate normally.  The host
+ * buffer of a served result counts as well: the step that finishes the request
+ * returns FABM_ENOMEM and the next one tries again.  n = 0 cancels what is left.
  * FABM_EINVAL for n < 0. */
 fabm_status fabm_set_wait_limit(fabm_solver *s, int64_t cycles);
 fabm_status fabm_inject_alloc_failures(int n);

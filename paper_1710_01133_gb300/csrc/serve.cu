@@ -66,9 +66,6 @@ struct SlotDev {
     int resumed, pad2;  // history, solution and status come from a checkpoint
 };
 
-// Block that the slot runs at server step e, or -1.
-__device__ inline int64_t slot_block(const SlotDev &s, int64_t e) { return e < s.start ? -1 : s.c0 + e; }
-
 // Chunking of block c's far history for one slot: depends on c only, so a
 // request's partial sums do not depend on the other requests in flight.
 __host__ __device__ inline void slot_chunks(int64_t c, int64_t *kc, int *n)
@@ -82,6 +79,14 @@ __host__ __device__ inline void slot_chunks(int64_t c, int64_t *kc, int *n)
 }
 
 __host__ __device__ inline int64_t slot_blocks(int64_t N) { return (N + kSL - 1) / kSL; }
+
+// Block that the slot runs at server step e, or -1: not begun, or finished and waiting
+// for host memory for its result.
+__device__ inline int64_t slot_block(const SlotDev &s, int64_t e)
+{
+    const int64_t c = s.c0 + e;
+    return e < s.start || c >= slot_blocks(s.N) ? -1 : c;
+}
 
 __device__ inline DevBatch slot_batch(const SlotDev &s)
 {
@@ -849,8 +854,19 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
             s.pending = false;
             continue;
         }
-        s.c += 1;
+        s.c = std::min(s.c + 1, s.nblk);  // at nblk already if a result had no room before
         if (s.c >= s.nblk) S->h_idx[n_done++] = i;
+    }
+    // room for every result before anything is copied; without it the finished slots
+    // wait for the next step
+    for (int j = 0; j < n_done; ++j) {
+        const Slot &s = S->slots[S->h_idx[j]];
+        Result &res = S->results[s.req.ticket];
+        res.n = (size_t)(s.req.N + 1) * s.req.dim;
+        if (!take_injected_alloc_failure())
+            res.y.reset(new (std::nothrow) double[res.n]());  // touched here: the copy engine
+                                                              // is slow on new pages
+        if (!res.y) return srv_fail(FABM_ENOMEM, "host memory for a result");
     }
     if (n_done > 0) {
         SRV_TRY(cudaMemcpyAsync(S->d_idx, S->h_idx, sizeof(int) * n_done, cudaMemcpyHostToDevice, S->sR));
@@ -861,10 +877,6 @@ fabm_status server_step(fabm_server *S, int *n_active, int *n_waiting)
         for (int j = 0; j < n_done; ++j) {
             Slot &s = S->slots[S->h_idx[j]];
             Result &res = S->results[s.req.ticket];
-            res.n = (size_t)(s.req.N + 1) * s.req.dim;
-            res.y.reset(new (std::nothrow) double[res.n]());  // touched here: the copy engine
-                                                                // is slow on new pages
-            if (!res.y) return srv_fail(FABM_ENOMEM, "host memory for a result");
             SRV_TRY(cudaMemcpyAsync(res.y.get(), s.dev.Y, sizeof(double) * res.n, cudaMemcpyDeviceToHost, S->sR));
         }
         SRV_TRY(cudaStreamSynchronize(S->sR));
