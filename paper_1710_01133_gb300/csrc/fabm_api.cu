@@ -454,7 +454,7 @@ int history_lag(int hk, int64_t N, int64_t cols)
 // 4096 301 / 338; Lorenz type, 32 steps, 1000 100 / 111.
 bool short_solve(int dim, int64_t B, int64_t N)
 {
-    return B > 512 && N <= (dim == 1 ? 64 : dim == 2 ? 32 : 0);
+    return B >= 512 && N <= (dim == 1 ? 64 : dim == 2 ? 32 : 0);
 }
 
 // A forced scalar system of very many trajectories: the table of its forcing, a

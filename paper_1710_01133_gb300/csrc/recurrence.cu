@@ -12,7 +12,7 @@ __global__ void init_kernel(DevBatch bt, bool f_pairs, FFInputs ff)
 }
 
 template <class Rhs, int D, int TPL, bool SPLIT, int LAG>
-__global__ void __launch_bounds__((D + 1) * kWarp)
+__global__ void __launch_bounds__((SPLIT ? D + 1 : D) * kWarp)
     recur_kernel(DevBatch bt, DevWeights w, StepConsts kc, int64_t c, const double *G)
 {
     if constexpr (SPLIT) {

@@ -33,8 +33,8 @@ def solve(gpu_lib, parity, rhs, dim, precision, B, N, tol, **kw):
 
 # launches: initial values, then one per block or superblock, and one per forcing table
 @pytest.mark.parametrize("rhs,dim,B,N,launches", [
-    ("linear", 1, 512, 64, 2), ("linear", 1, 513, 64, 3), ("linear", 1, 513, 65, 2), ("linear", 1, 600, 1, 2),
-    ("duffing", 2, 513, 32, 2), ("duffing", 2, 513, 33, 3), ("lorenz", 3, 600, 40, 2),
+    ("linear", 1, 511, 64, 2), ("linear", 1, 512, 64, 3), ("linear", 1, 513, 65, 2), ("linear", 1, 600, 1, 2),
+    ("duffing", 2, 512, 32, 2), ("duffing", 2, 513, 33, 3), ("lorenz", 3, 600, 40, 2),
     ("manufactured", 1, 4095, 128, 3), ("manufactured", 1, 4096, 128, 7)])
 def test_fp64(gpu_lib, parity, rhs, dim, B, N, launches):
     assert solve(gpu_lib, parity, rhs, dim, "fp64", B, N, TOL_FP64)[1] == launches
