@@ -199,11 +199,14 @@ int fabm_last_history_kernel(const fabm_solver *s);
 /* Step layouts of the split-precision recurrence on the tensor-history path
  * (fabm_set_recurrence_layout); both compute the same steps in float-float. */
 enum {
-    FABM_REC_AUTO = 0,     /* COLUMNS                                               */
+    FABM_REC_AUTO = 0,     /* COLUMNS; TARGETS for systems of one component of up to
+                              1024 trajectories (1600 from 3072 steps on; 384 of a
+                              forced system)                                        */
     FABM_REC_COLUMNS = 1,  /* one lane per column (trajectory, component), 32/dim
                               trajectories per team of five warps                   */
     FABM_REC_TARGETS = 2   /* one lane per target, one CTA of dim warps per
-                              trajectory: most parallelism for narrow batches        */
+                              trajectory; the segments' slices by a launch of their
+                              own                                                    */
 };
 
 /* Choose the recurrence layout (one of FABM_REC_*) for later solves on the
@@ -213,9 +216,10 @@ fabm_status fabm_set_recurrence_layout(fabm_solver *s, int layout);
 /* The layout set on the solver (FABM_REC_*), or -1 for NULL. */
 int fabm_get_recurrence_layout(const fabm_solver *s);
 /* Teams of warps per CTA of the lane-per-column recurrence (FABM_REC_COLUMNS)
- * for later solves: 0 chooses automatically (one), 1..12 fixes it (more than
- * three run as three); the arithmetic and the results do not depend on it.  FABM_EINVAL outside 0..12, FABM_EBUSY while
- * another thread uses the solver. */
+ * for later solves: 0 chooses automatically (one), 1..12 fixes it, of which a CTA
+ * holds three at most (more run as three); the arithmetic and the results do not
+ * depend on it.  FABM_EINVAL outside 0..12, FABM_EBUSY while another thread uses
+ * the solver. */
 fabm_status fabm_set_recurrence_warps(fabm_solver *s, int warps);
 /* The width set on the solver (0: automatic), or -1 for NULL. */
 int fabm_get_recurrence_warps(const fabm_solver *s);
@@ -265,13 +269,14 @@ fabm_status fabm_set_graphs(fabm_solver *s, int enable);
 /* Failure handling (Sec. 5 of the design has no counterpart in the paper; these
  * make the library's error paths testable without faulting a GPU).
  *
- * fabm_set_wait_limit: the tensor-core history kernel waits on barriers that
- * other warps of its CTA complete; each such wait gives up after `cycles` SM
- * clock cycles (0: the default, about 2 s at 2 GHz).  A CTA that gives up sets
- * the solver's status word, waits for its own copies and MMAs in flight, frees
- * its tensor memory and returns, and the solve returns FABM_ETIMEOUT; the
- * solver stays usable.  A tiny limit forces that path.  FABM_EINVAL for
- * cycles < 0.
+ * fabm_set_wait_limit: the tensor-core history kernels wait on barriers that
+ * other warps of their CTA complete, the FP64 and FP64X2 steps on values that
+ * other warps of their CTA or cluster produce, the persistent FP64 solve on other
+ * CTAs' flags; each such wait gives up after `cycles` SM clock cycles (0: the
+ * default, about 2 s at 2 GHz).  A kernel that gives up sets the solver's status
+ * word, waits for its own copies and MMAs in flight, frees its tensor memory and
+ * ends, and the solve returns FABM_ETIMEOUT; the solver stays usable.  A tiny
+ * limit forces that path.  FABM_EINVAL for cycles < 0.
  *
  * fabm_inject_alloc_failures: the next n device allocations the library makes
  * (solver work space, server admissions; process-wide) fail as if the device

@@ -412,7 +412,7 @@ class Solver:
         fabm_set_graphs(self.handle, enable)
 
     def set_wait_limit(self, cycles: int = 0):
-        """Clock cycles after which the tensor kernel's waits give up (0: default)."""
+        """Clock cycles after which the kernels' waits give up (0: default)."""
         fabm_set_wait_limit(self.handle, cycles)
 
     def set_timing(self, period: int = 1):

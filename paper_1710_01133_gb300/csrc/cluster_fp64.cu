@@ -35,7 +35,7 @@
 // code) about 50 cycles later than the FP64 unit itself, and a store to 16 CTAs
 // holds up the stores behind it, so only the exchange stands between the
 // instructions of a step, and the copies of f follow it.  Cycles per step: 355
-// for the scalar system (five FP64 instructions), 720 for the Lorenz type (six
+// for the scalar system (four FP64 instructions and one hand-over), 720 for the Lorenz type (six
 // and two exchanges).  Blocks of 32 with a warp instruction per kind took 457
 // and 765; a chain of newest points only, the rest of the block summed by
 // another warp a target ahead, 560 and 920 (the way there and back is longer

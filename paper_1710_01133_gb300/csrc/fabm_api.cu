@@ -423,10 +423,6 @@ int resolve_hist_kernel(const fabm_solver *s, int64_t cols)
     return cols >= 64 ? FABM_HIST_TENSOR : FABM_HIST_FP32C;
 }
 
-// Enqueues one solve on the solver's two streams (or records it into the
-// graph being captured): init, then per block the far history on stream G and
-// the recurrence (and, split path, the slicing of the finished segment) on
-// stream R.
 // Lag of the history launches: the history of block c covers the points
 // k < (c - lag) L and the recurrence sums the lag blocks before c.  With lag 2
 // (CUDA-core history kernels, long histories) the history of block c waits
@@ -749,7 +745,9 @@ fabm_status enqueue_solve(fabm_solver *s, const DevBatch &bt, const DevWeights &
 // 1 x 2^15 11.3 (1024: 11.9), 12 x 2^14 5.9 / 6.1, 16 x 2^14 7.7 / 6.2 / 6.7,
 // 30 x 2^13 - / 3.5 / 3.9, 120 x 2^13 - / 9.4 / 6.5 (64: 7.1); oscillator 16 x 2^14
 // 6.5 / 6.6 / 6.9, 60 x 2^13 - / 5.9 / 3.9 (64: 4.6); LCR 256 x 2^13 - / 10.4 / 7.9
-// (64: 10.6).
+// (64: 10.6).  One CTA per trajectory also where they come in many waves, against the
+// block schedule (us): 4096 x 1000 Lorenz type 28,400 -> 14,300, LCR 22,200 -> 10,500,
+// scalar 8950 -> 4670; 16,384 x 250 13,000 -> 9860, 11,400 -> 7560, 3130 -> 3140.
 struct ClusterShape {
     int CS, n2, n3;
 };
@@ -769,7 +767,8 @@ void plan_cluster(fabm_solver *s, int64_t B, int64_t cols, int64_t Nmax)
         s->cl_size = c.CS, s->cl_n = n;
         break;
     }
-    // spectra of f: 32 bytes per point and column
+    // spectra of f: 32 bytes per point and column, up to 16 GB; beyond that neither
+    // schedule has been timed against the other (nor 65,535 columns, a grid's limit)
     if (s->cl_size && Nmax > 2 * s->cl_n && (cols > 65535 || Nmax * cols > (1LL << 29))) s->cl_size = 0;
 }
 

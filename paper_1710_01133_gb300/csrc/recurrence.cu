@@ -11,17 +11,16 @@ __global__ void init_kernel(DevBatch bt, bool f_pairs, FFInputs ff)
     if (b < bt.B) init_one<Rhs, D>(bt, b, f_pairs, ff);
 }
 
-template <class Rhs, int D, int TPL, bool SPLIT, int LAG>
+template <class Rhs, int D, bool SPLIT, int LAG>
 __global__ void __launch_bounds__((SPLIT ? D + 1 : D) * kWarp)
     recur_kernel(DevBatch bt, DevWeights w, StepConsts kc, int64_t c, const double *G)
 {
     if constexpr (SPLIT) {
-        static_assert(TPL == 1);
         __shared__ __align__(16) float smem_f[recur_split_smem_floats<D, LAG>()];
         recur_block_split<Rhs, D, LAG>(bt, blockIdx.x, w, kc, c, G, smem_f);
     } else {
-        __shared__ double smem[recur_smem_doubles<D, TPL, LAG>()];
-        recur_block<Rhs, D, TPL, LAG>(bt, blockIdx.x, w, kc, c, G, smem);
+        __shared__ double smem[recur_smem_doubles<D, 1, LAG>()];
+        recur_block<Rhs, D, 1, LAG>(bt, blockIdx.x, w, kc, c, G, smem);
     }
 }
 
@@ -31,14 +30,14 @@ __global__ void __launch_bounds__((SPLIT ? D + 1 : D) * kWarp)
 // one SM together (LCR of two orders, 200 x 4000: 4.5 ms without, 3.5 with).
 constexpr int kHistCarveout = 57;
 
-template <int TPL, bool SPLIT, int LAG>
+template <bool SPLIT, int LAG>
 bool launch_recur_t(int rhs, const DevBatch &bt, const DevWeights &w, const StepConsts &k,
                     int64_t c, bool alone, const double *G, cudaStream_t st)
 {
     bool set = true;
     const bool ok = dispatch_rhs(rhs, bt.dim, [&]<class R, int D>() {
         constexpr int warps = SPLIT ? recur_split_warps<R, D>() : D;
-        auto kernel = recur_kernel<R, D, TPL, SPLIT, LAG>;
+        auto kernel = recur_kernel<R, D, SPLIT, LAG>;
         const size_t smem = alone ? kAloneSmem : 0;
         if (SPLIT && !alone)
             set = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -69,11 +68,11 @@ cudaError_t launch_recur(int rhs, const DevBatch &bt, const DevWeights &w, const
 {
     bool ok = false;
     if (L == kWarp && lag == 1)
-        ok = split ? launch_recur_t<1, true, 1>(rhs, bt, w, k, c, alone, G, st)
-                   : launch_recur_t<1, false, 1>(rhs, bt, w, k, c, false, G, st);
+        ok = split ? launch_recur_t<true, 1>(rhs, bt, w, k, c, alone, G, st)
+                   : launch_recur_t<false, 1>(rhs, bt, w, k, c, false, G, st);
     else if (L == kWarp && lag == 2)
-        ok = split ? launch_recur_t<1, true, 2>(rhs, bt, w, k, c, alone, G, st)
-                   : launch_recur_t<1, false, 2>(rhs, bt, w, k, c, false, G, st);
+        ok = split ? launch_recur_t<true, 2>(rhs, bt, w, k, c, alone, G, st)
+                   : launch_recur_t<false, 2>(rhs, bt, w, k, c, false, G, st);
     return ok ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 
