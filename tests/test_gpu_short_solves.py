@@ -50,3 +50,17 @@ def test_fp64x2_single_chunk(gpu_lib, parity, rhs, dim, B, N):
     with gpu_lib.Solver(rhs, dim, 0.9, 1e-3, N, PARAMS[rhs], precision="fp64x2") as s:
         for b in (0, B - 1):
             assert np.array_equal(got[b], s.solve_batch(y0[b : b + 1])[0])
+
+
+@pytest.mark.parametrize("alpha", [0.4, 0.8, 0.95, 1.5])
+def test_error_of_blocks_against_binary128(gpu_lib, parity, alpha):
+    """A value takes the points of its own block of 32 one by one, 16 on average, each
+    rounded to a unit of its last place: sqrt(16 / 3) 2^-53 = 2.6e-16 for mantissas of
+    one, less for larger ones.  With the 32 points of the block before taken the same way
+    it would be sqrt(48 / 3) 2^-53 = 4.4e-16.  2-norms over 15 trajectories; the bar is
+    the first of the two and a tenth for f, the corrector and the rest of the sums."""
+    N, y0 = 60, np.linspace(0.3, 1.5, 600)[:, None]
+    with gpu_lib.Solver("linear", 1, alpha, 2e-3, N, [1.0]) as s:
+        got = s.solve_batch(y0)[::40]
+    ref = np.stack([oracle.solve_q("linear", alpha, 2e-3, N, y, params=[1.0]) for y in y0[::40]])
+    parity(float(np.linalg.norm(got - ref) / np.linalg.norm(ref)), 2.8e-16)
